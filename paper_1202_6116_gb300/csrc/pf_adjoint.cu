@@ -119,15 +119,15 @@ __global__ void __launch_bounds__(MTX* MTY) k_tdgl_adj(Geo g, Bc<T> bc, const T*
 #pragma unroll
     for (int q = 0; q < ADJ_NV; ++q) acc[q] = Acc<T>();
     march_direct<T, L3<T>, MTX, MTY, VX, 4, 3, ADJ_D>(g, s, smem, hsrc, osrc, emit, post);
-    double v[ADJ_NV];
+    typename SumOf<T>::type v[ADJ_NV];
 #pragma unroll
-    for (int q = 0; q < ADJ_NV; ++q) v[q] = acc[q].value();
-    tile_partials<ADJ_NV, MTX * MTY>(v, part, t);
+    for (int q = 0; q < ADJ_NV; ++q) v[q] = acc[q].sum();
+    tile_partials<ADJ_NV, MTX * MTY>(v, part, t, smem);
   }
   sched_finish(ts);
   if (!last_block<MTX * MTY>(&S->ticket)) return;
   double sum[ADJ_NV];
-  gather_partials<ADJ_NV, MTX * MTY>(part, mc.ntiles, sum);
+  gather_partials<ADJ_NV, MTX * MTY>(part, mc.ntiles, sum, smem);
   if (threadIdx.x != 0 || threadIdx.y != 0) return;
   const double dtL = (double)k.dtL;
   grad[0] += -dtL * sum[0];

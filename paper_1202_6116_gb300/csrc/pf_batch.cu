@@ -38,6 +38,12 @@ __global__ void __launch_bounds__(256) k_batch_ramp(const BatchFilm* films, cons
 
 constexpr int REC_THREADS = 256;
 
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+  return v;
+}
+
 __global__ void __launch_bounds__(REC_THREADS) k_batch_record(const BatchFilm* films, int nfilms, int buf,
                                                               BatchState* bs, double* part, double* hist) {
   __shared__ double red[3][REC_THREADS / 32];

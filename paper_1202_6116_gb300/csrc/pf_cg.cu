@@ -151,13 +151,13 @@ __global__ void __launch_bounds__(MTX* MTY, (sizeof(T) == 4 && !EPS) ? 3 : 2) k_
     } else {
       march<T, F, Out, MTX, MTY, VX, NH, 1, CG_D>(g, s, smem, hsrc, osrc, val, emit, post);
     }
-    double v[1] = {apq.value()};
-    tile_partials<1, MTX * MTY>(v, part, t);
+    typename SumOf<T>::type v[1] = {apq.sum()};
+    tile_partials<1, MTX * MTY>(v, part, t, smem);
   }
   sched_finish(ts);
   if (last_block<MTX * MTY>(&S->ticket)) {
     double out[1];
-    gather_partials<1, MTX * MTY>(part, mc.ntiles, out);
+    gather_partials<1, MTX * MTY>(part, mc.ntiles, out, smem);
     if (threadIdx.x == 0 && threadIdx.y == 0) {
       const double pq = out[0];
       S->pq = pq;
@@ -226,13 +226,13 @@ __global__ void __launch_bounds__(FLAT_THREADS) k_cg_r(Geo g, Bc<T> bc, const T*
   }
   arr.flush();
   arz.flush();
-  double v[2] = {arr.value(), arz.value()};
+  typename SumOf<T>::type v[2] = {arr.sum(), arz.sum()};
   if (publish_partials<2, FLAT_THREADS>(v, part, &S->ticket)) {
     double out[2];
     gather_partials<2, FLAT_THREADS>(part, gridDim.x, out);
     if (threadIdx.x == 0) {
       const double rr = out[0], rz = out[1];
-      const double rel = sqrt(rr) / sqrt(S->bb);
+      const double rel = sqrt(rr) / S->bnorm;
       S->rr = rr;
       S->last_rel = rel;
       if (!isfinite(rr)) {

@@ -88,6 +88,7 @@ __device__ __forceinline__ T inv_flat(const Geo& g, const Bc<T>& bc, long long e
 // Solver state in device memory (inside the caller's workspace).
 struct Scalars {
   double bb;        // ||b||^2
+  double bnorm;     // ||b||
   double rz;        // r.z of the current residual
   double rr;        // ||r||^2
   double alpha;
@@ -121,11 +122,39 @@ struct Scalars {
 };
 
 // ---------------------------------------------------------------- reductions
+//
+// What a thread sums in FP32 it keeps as an unevaluated pair (hi, lo), and the
+// block adds its threads' pairs as pairs; only the block's (or tile's) total
+// becomes a double.  The FP64 unit issues one warp instruction in 19 cycles
+// per SM (measured: 1.67 thread operations per clock), so converting and
+// shuffling doubles in every thread -- 93 FP64 warp instructions per value and
+// tile -- cost more than the stencil of a shallow tile: 1.77 kcycles per value
+// against about 0.12 for the pairs.  The right-hand side of a 256 x 256 x 64
+// film (2048 tiles, three sums) took 78 us that way, the diagnostics (seven
+// sums) of 512 x 512 x 64 210 us.
 
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  return v;
+// Sum of a block's threads: a pair of floats (FP32 fields) or a double.
+template <typename T>
+struct SumOf;
+template <>
+struct SumOf<double> {
+  using type = double;
+};
+template <>
+struct SumOf<float> {
+  using type = float2;
+};
+
+// (a.x + a.y) + (b.x + b.y) as a normalised pair: TwoSum (Knuth) of the
+// leading parts, the rest in the second part; relative error about 2^-46 of
+// |a| + |b|.
+__device__ __forceinline__ float2 pair_add(float2 a, float2 b) {
+  const float s = __fadd_rn(a.x, b.x);
+  const float z = __fsub_rn(s, a.x);
+  float e = __fadd_rn(__fsub_rn(a.x, __fsub_rn(s, z)), __fsub_rn(b.x, z));
+  e = __fadd_rn(e, __fadd_rn(a.y, b.y));
+  const float h = __fadd_rn(s, e);
+  return make_float2(h, __fsub_rn(e, __fsub_rn(h, s)));
 }
 
 // Dot-product accumulators.  FP64 fields: plain FMA accumulation.  FP32
@@ -133,11 +162,11 @@ __device__ __forceinline__ double warp_sum(double v) {
 // is summed by plain FMAs; the run totals are summed with TwoSum (Knuth), the
 // error terms collected in a second float ("cascaded" summation: the
 // compensated sum of Ogita, Rump & Oishi, SIAM J. Sci. Comput. 26, 2005,
-// applied to runs instead of single products); flush() moves the pair into an
-// FP64 total, so the FP64 unit sees a handful of adds per tile.  A run of k
-// products carries a relative error of about k u (u = 2^-24) of its absolute
-// sum, so with k = 4 the dot keeps close to FP32 working accuracy of the
-// absolute sum instead of the growth with the length of a plain FP32 sum.
+// applied to runs instead of single products); flush() normalises the pair in
+// long loops.  A run of k products carries a relative error of about k u (u =
+// 2^-24) of its absolute sum, so with k = 4 the dot keeps close to FP32
+// working accuracy of the absolute sum instead of the growth with the length
+// of a plain FP32 sum.
 template <typename T>
 struct Acc;
 
@@ -147,14 +176,13 @@ struct Acc<double> {
   __device__ __forceinline__ void add(double a, double b) { s = fma(a, b, s); }
   __device__ __forceinline__ void run() {}
   __device__ __forceinline__ void flush() {}
-  __device__ __forceinline__ double value() const { return s; }
+  __device__ __forceinline__ double sum() const { return s; }
 };
 
 template <>
 struct Acc<float> {
   float part = 0.f;               // the current run
   float hi = 0.f, lo = 0.f;       // compensated sum of the closed runs
-  double tot = 0.0;
   __device__ __forceinline__ void add(float a, float b) { part = fmaf(a, b, part); }
   __device__ __forceinline__ void run() {
     const float s = __fadd_rn(hi, part);
@@ -166,73 +194,66 @@ struct Acc<float> {
   }
   __device__ __forceinline__ void flush() {
     run();
-    tot += (double)hi + (double)lo;
-    hi = 0.f;
-    lo = 0.f;
+    const float s = __fadd_rn(hi, lo);
+    lo = __fsub_rn(lo, __fsub_rn(s, hi));
+    hi = s;
   }
-  __device__ __forceinline__ double value() const { return tot + (double)hi + (double)lo + (double)part; }
+  __device__ __forceinline__ float2 sum() {
+    run();
+    return make_float2(hi, lo);
+  }
 };
 
-// Block-reduce NV values, publish the block's partials, and tell whether this
-// block is the last one of the grid to finish (the classic threadfence
-// reduction: no block ever waits for another).  Must be called by every
-// thread of the block.
-template <int NV, int NT = NTHREADS>
-__device__ __forceinline__ bool publish_partials(double (&v)[NV], double* part, unsigned* ticket) {
-  __shared__ double sm[NV][NT / 32];
-  __shared__ bool last;
+__device__ __forceinline__ double sum_add(double a, double b) { return a + b; }
+__device__ __forceinline__ float2 sum_add(float2 a, float2 b) { return pair_add(a, b); }
+__device__ __forceinline__ double sum_xor(double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
+__device__ __forceinline__ float2 sum_xor(float2 v, int o) {
+  return make_float2(__shfl_xor_sync(0xffffffffu, v.x, o), __shfl_xor_sync(0xffffffffu, v.y, o));
+}
+__device__ __forceinline__ double sum_double(double v) { return v; }
+__device__ __forceinline__ double sum_double(float2 v) { return (double)v.x + (double)v.y; }
+
+// Sums of NV values over the NT = 256 threads of a block; the sum of value k
+// is returned (as a double) in lane 0 of warp k.  Every thread must call it;
+// it ends without a barrier.  Warp k adds value k of all threads from shared
+// memory: 12 additions a value, where a shuffle tree in each of the eight
+// warps takes 45.  sm: sum_scratch<V>(NV) bytes, 8-byte aligned, that nobody
+// else uses until the block's next barrier -- the plane marches lend their
+// staging buffers, which are idle between tiles (12 KB of static shared
+// memory beside them shrank the L1 and cost k_rhs_w 7 %).  Not inlined: it
+// runs once per tile, and its temporaries would count in the march.
+template <int NV, int NT, typename V>
+__device__ __noinline__ double shared_sums(const V* sm) {
   const int tid = threadIdx.x + threadIdx.y * blockDim.x;
   const int lane = tid & 31, wid = tid >> 5;
+  V d = sm[wid * NT + lane];
 #pragma unroll
-  for (int k = 0; k < NV; ++k) v[k] = warp_sum(v[k]);
-  if (lane == 0) {
+  for (int j = 1; j < NT / 32; ++j) d = sum_add(d, sm[wid * NT + lane + 32 * j]);
 #pragma unroll
-    for (int k = 0; k < NV; ++k) sm[k][wid] = v[k];
-  }
+  for (int o = 16; o > 0; o >>= 1) d = sum_add(d, sum_xor(d, o));
+  return sum_double(d);
+}
+template <int NV, int NT, typename V>
+__device__ __forceinline__ double block_sums(const V (&v)[NV], void* scratch) {
+  static_assert(NT == 256 && NV <= 8, "eight warps, a value per warp");
+  V* sm = static_cast<V*>(scratch);
+  const int tid = threadIdx.x + threadIdx.y * blockDim.x;
+  __syncthreads();                 // the scratch may still be read
+#pragma unroll
+  for (int k = 0; k < NV; ++k) sm[k * NT + tid] = v[k];
   __syncthreads();
-  if (wid == 0) {
-#pragma unroll
-    for (int k = 0; k < NV; ++k) {
-      double x = (lane < NT / 32) ? sm[k][lane] : 0.0;
-      v[k] = warp_sum(x);
-    }
-    if (lane == 0) {
-#pragma unroll
-      for (int k = 0; k < NV; ++k) part[(long long)blockIdx.x * NV + k] = v[k];
-      __threadfence();
-      unsigned t = atomicAdd(ticket, 1u);
-      last = (t == gridDim.x - 1);
-    }
-  }
-  __syncthreads();
-  return last;
+  return (tid >> 5) < NV ? shared_sums<NV, NT>(sm) : 0.0;
 }
 
-// Block-reduce NV values of one work tile and store them at part[t*NV + k]
-// (thread 0).  Kernels that hand out tiles dynamically reduce per tile, so the
-// final sum (over tiles, in tile order) does not depend on which block ran
-// which tile.  Must be called by every thread of the block.
-template <int NV, int NT>
-__device__ __forceinline__ void tile_partials(double (&v)[NV], double* part, long long t) {
-  __shared__ double sm[NV][NT / 32];
+// Block-reduce NV values of one work tile and store them at part[t*NV + k].
+// Kernels that hand out tiles dynamically reduce per tile, so the final sum
+// (over tiles, in tile order) does not depend on which block ran which tile.
+// Must be called by every thread of the block (scratch: see block_sums).
+template <int NV, int NT, typename V>
+__device__ __forceinline__ void tile_partials(const V (&v)[NV], double* part, long long t, void* scratch) {
+  const double d = block_sums<NV, NT>(v, scratch);
   const int tid = threadIdx.x + threadIdx.y * blockDim.x;
-  const int lane = tid & 31, wid = tid >> 5;
-#pragma unroll
-  for (int k = 0; k < NV; ++k) v[k] = warp_sum(v[k]);
-  __syncthreads();                 // sm[] may still be read from the previous tile
-  if (lane == 0) {
-#pragma unroll
-    for (int k = 0; k < NV; ++k) sm[k][wid] = v[k];
-  }
-  __syncthreads();
-  if (wid == 0) {
-#pragma unroll
-    for (int k = 0; k < NV; ++k) {
-      double x = (lane < NT / 32) ? sm[k][lane] : 0.0;
-      x = warp_sum(x);
-      if (lane == 0) part[t * NV + k] = x;
-    }
-  }
+  if ((tid & 31) == 0 && (tid >> 5) < NV) part[t * NV + (tid >> 5)] = d;
 }
 
 // After every block stored its tile partials: is this the last block to finish?
@@ -249,34 +270,42 @@ __device__ __forceinline__ bool last_block(unsigned* ticket) {
   return last;
 }
 
+// Block-reduce NV values, publish the block's partials, and tell whether this
+// block is the last one of the grid to finish (the classic threadfence
+// reduction: no block ever waits for another).  Must be called by every
+// thread of the block.
+template <int NV, int NT = NTHREADS, typename V>
+__device__ __forceinline__ bool publish_partials(const V (&v)[NV], double* part, unsigned* ticket) {
+  __shared__ V sm[NV * NT];
+  tile_partials<NV, NT>(v, part, blockIdx.x, sm);
+  return last_block<NT>(ticket);
+}
+
 // In the last block: sum the published partials in a fixed order (so results
-// are reproducible run to run).  Result valid in thread 0.
+// are reproducible run to run).
 template <int NV, int NT = NTHREADS>
-__device__ __forceinline__ void gather_partials(const double* part, long long nblocks, double (&out)[NV]) {
-  __shared__ double sm[NV][NT / 32];
+__device__ __forceinline__ void gather_partials(const double* part, long long nblocks, double (&out)[NV],
+                                                void* scratch) {
+  __shared__ double res[NV];
   const int tid = threadIdx.x + threadIdx.y * blockDim.x;
-  const int lane = tid & 31, wid = tid >> 5;
   double acc[NV];
 #pragma unroll
   for (int k = 0; k < NV; ++k) acc[k] = 0.0;
+#pragma unroll 1
   for (long long i = tid; i < nblocks; i += NT) {
 #pragma unroll
-    for (int k = 0; k < NV; ++k) acc[k] += __ldcg(part + (long long)i * NV + k);
+    for (int k = 0; k < NV; ++k) acc[k] += __ldcg(part + i * NV + k);
   }
-#pragma unroll
-  for (int k = 0; k < NV; ++k) acc[k] = warp_sum(acc[k]);
-  if (lane == 0) {
-#pragma unroll
-    for (int k = 0; k < NV; ++k) sm[k][wid] = acc[k];
-  }
+  const double d = block_sums<NV, NT>(acc, scratch);
+  if ((tid & 31) == 0 && (tid >> 5) < NV) res[tid >> 5] = d;
   __syncthreads();
-  if (wid == 0) {
 #pragma unroll
-    for (int k = 0; k < NV; ++k) {
-      double x = (lane < NT / 32) ? sm[k][lane] : 0.0;
-      out[k] = warp_sum(x);
-    }
-  }
+  for (int k = 0; k < NV; ++k) out[k] = res[k];
+}
+template <int NV, int NT = NTHREADS>
+__device__ __forceinline__ void gather_partials(const double* part, long long nblocks, double (&out)[NV]) {
+  __shared__ double sm[NV * NT];
+  gather_partials<NV, NT>(part, nblocks, out, sm);
 }
 
 // ------------------------------------------------------------- tile decoding

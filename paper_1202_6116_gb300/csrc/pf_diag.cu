@@ -79,15 +79,15 @@ __global__ void __launch_bounds__(MTX* MTY) k_diag(Geo g, Bc<T> bc, const T* __r
 #pragma unroll
     for (int q = 0; q < DIAG_NV; ++q) acc[q] = Acc<T>();
     march_direct<T, T, MTX, MTY, VX, 4, 0, DIAG_D>(g, s, smem, hsrc, osrc, emit, post);
-    double v[DIAG_NV];
+    typename SumOf<T>::type v[DIAG_NV];
 #pragma unroll
-    for (int q = 0; q < DIAG_NV; ++q) v[q] = acc[q].value();
-    tile_partials<DIAG_NV, MTX * MTY>(v, part, t);
+    for (int q = 0; q < DIAG_NV; ++q) v[q] = acc[q].sum();
+    tile_partials<DIAG_NV, MTX * MTY>(v, part, t, smem);
   }
   sched_finish(ts);
   if (!last_block<MTX * MTY>(&S->ticket)) return;
   double sum[DIAG_NV];
-  gather_partials<DIAG_NV, MTX * MTY>(part, mc.ntiles, sum);
+  gather_partials<DIAG_NV, MTX * MTY>(part, mc.ntiles, sum, smem);
   if (threadIdx.x != 0 || threadIdx.y != 0) return;
 #pragma unroll
   for (int q = 0; q < DIAG_NV; ++q) out[q] = sum[q];

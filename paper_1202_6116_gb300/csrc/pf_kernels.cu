@@ -112,7 +112,7 @@ __global__ void __launch_bounds__(NTHREADS) k_cg_finish(Geo g, T* __restrict__ x
     }
     ax.flush();
   }
-  double v[1] = {ax.value()};
+  typename SumOf<T>::type v[1] = {ax.sum()};
   if (publish_partials<1>(v, part, &S->ticket)) {
     double out[1];
     gather_partials<1>(part, gridDim.x, out);

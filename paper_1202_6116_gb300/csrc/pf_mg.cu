@@ -710,8 +710,8 @@ __global__ void __launch_bounds__(MTX* MTY, 3) k_mg_pp(MgView<float> L, MgView<f
       }
     }
     cp_wait<0>();
-    double v[1] = {arz.value()};
-    tile_partials<1, MTX * MTY>(v, part, t);
+    float2 v[1] = {arz.sum()};
+    tile_partials<1, MTX * MTY>(v, part, t, smem);
   }
   sched_finish(ts);
 }
@@ -822,15 +822,15 @@ __global__ void __launch_bounds__(MTX* MTY, (sizeof(T) == 4 && !EPS) ? (INT ? 5 
     arz = Acc<T>();
     march_direct<T, T, MTX, MTY, VX, NH, NO, MG_D, 0, INT>(L.g, s, smem, hsrc, osrc, emit, post);
     if (LAST) {
-      double v[1] = {arz.value()};
-      tile_partials<1, MTX * MTY>(v, part + pofs, t);
+      typename SumOf<T>::type v[1] = {arz.sum()};
+      tile_partials<1, MTX * MTY>(v, part + pofs, t, smem);
     }
   }
   sched_finish(ts);
   if (!LAST) return;
   if (last_block<MTX * MTY>(&S->ticket)) {
     double out[1];
-    gather_partials<1, MTX * MTY>(part, ptot, out);
+    gather_partials<1, MTX * MTY>(part, ptot, out, smem);
     if (threadIdx.x == 0 && threadIdx.y == 0) {
       const double rz = out[0];
       if (!isfinite(rz)) {

@@ -69,10 +69,10 @@ __device__ __forceinline__ T divergence(const Stencil7<Raw<T, NH>>& s, int dlo, 
 // test of the start (or, MEAN, the mean of b).  Called by every thread.
 template <int NV, bool MEAN, bool COMP>
 __device__ __forceinline__ void rhs_close(const Geo& g, double* part, Scalars* S, long long ntiles,
-                                          cudaGraphConditionalHandle cond, int use_cond) {
+                                          cudaGraphConditionalHandle cond, int use_cond, void* smem) {
   if (!last_block<MTX * MTY>(&S->ticket)) return;
   double out[NV];
-  gather_partials<NV, MTX * MTY>(part, ntiles, out);
+  gather_partials<NV, MTX * MTY>(part, ntiles, out, smem);
   if (threadIdx.x != 0 || threadIdx.y != 0) return;
   if (MEAN) {
     S->mean_b = out[0] / (double)g.n;
@@ -81,6 +81,7 @@ __device__ __forceinline__ void rhs_close(const Geo& g, double* part, Scalars* S
   }
   const double bb = out[0], rr = out[NV > 1 ? 1 : 0], rz = out[NV > 2 ? 2 : 0];
   S->bb = bb;
+  S->bnorm = sqrt(bb);
   S->rr = rr;
   S->rz = rz;
   S->iter = 0;
@@ -192,12 +193,12 @@ __global__ void __launch_bounds__(MTX* MTY) k_rhs(Geo g, Bc<T> bc, const T* __re
     arr = Acc<T>();
     arz = Acc<T>();
     march_direct<T, T, MTX, MTY, VX, NH, NO, STEP_D>(g, s, smem, hsrc, osrc, emit, post);
-    double v[3] = {abb.value(), arr.value(), arz.value()};
-    double (&vv)[NV] = *reinterpret_cast<double(*)[NV]>(v);
-    tile_partials<NV, MTX * MTY>(vv, part, t);
+    typename SumOf<T>::type v[3] = {abb.sum(), arr.sum(), arz.sum()};
+    auto& vv = *reinterpret_cast<typename SumOf<T>::type(*)[NV]>(v);
+    tile_partials<NV, MTX * MTY>(vv, part, t, smem);
   }
   sched_finish(ts);
-  rhs_close<NV, MEAN, COMP>(g, part, S, mc.ntiles, cond, use_cond);
+  rhs_close<NV, MEAN, COMP>(g, part, S, mc.ntiles, cond, use_cond, smem);
 }
 
 // k_rhs for a compensated FP32 start with eps = 1 on whole tiles of 64 x 16
@@ -419,11 +420,11 @@ __global__ void __launch_bounds__(MTX* MTY, RW_D == 1 ? 3 : 2) k_rhs_w(Geo g, Bc
       else plane(false);
     }
     cp_wait<0>();
-    double vals[3] = {abb.value(), arr.value(), arz.value()};
-    tile_partials<3, MTX * MTY>(vals, part, t);
+    float2 vals[3] = {abb.sum(), arr.sum(), arz.sum()};
+    tile_partials<3, MTX * MTY>(vals, part, t, smem);
   }
   sched_finish(ts);
-  rhs_close<3, false, true>(g, part, S, mc.ntiles, cond, use_cond);
+  rhs_close<3, false, true>(g, part, S, mc.ntiles, cond, use_cond, smem);
 }
 
 template <typename T>
