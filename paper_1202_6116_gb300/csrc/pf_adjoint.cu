@@ -146,8 +146,10 @@ static void adj_t(const LaunchCfg& L, const Geo& g, const Dev<T>& d, const T* la
     allow_smem(k_tdgl_adj<T, VX>, bytes);
     once = true;
   }
-  k_tdgl_adj<T, VX><<<L.march.grid, dim3(MTX, MTY), bytes, L.stream>>>(
-      g, d.bc, lam, lam_out, psi, P, d.eps, k, grad, gv_lo, gv_hi, d.part, d.S, L.march);
+  static int occ = 0;
+  const MarchCfg mc = kernel_tiling(k_tdgl_adj<T, VX>, bytes, L, occ, false);
+  k_tdgl_adj<T, VX><<<mc.grid, dim3(MTX, MTY), bytes, L.stream>>>(
+      g, d.bc, lam, lam_out, psi, P, d.eps, k, grad, gv_lo, gv_hi, d.part, d.S, mc);
 }
 
 template <typename T>

@@ -1209,10 +1209,9 @@ pf_status pf_create(const pf_params* params, void* cuda_stream, pf_ctx** out) {
   pf::setup_launch(params, ctx->nsm, ctx->stream, g, ctx->L);
   ctx->lay = layout_of(params);
   if (!ctx->lay.mg.empty()) {
-    const int rmg = ctx->nsm * (params->precision == PF_FP32 ? pf::mg_blocks_per_sm<float>()
-                                                             : pf::mg_blocks_per_sm<double>());
+    const bool fp32 = params->precision == PF_FP32;
     for (MgLevelHost& l : ctx->lay.mg)
-      l.mc = pf::march_cfg(l.nx, l.ny, l.nz, rmg, l.fz == 2, params->precision == PF_FP32 ? 4 : 8);
+      l.mc = pf::march_cfg(l.nx, l.ny, l.nz, ctx->nsm, fp32 && !params->has_eps ? 4 : 2, 32, l.fz == 2, fp32 ? 4 : 8);
   }
   ctx->tlo_h.assign((size_t)g.nxy, 0);
   ctx->thi_h.assign((size_t)g.nxy, 0);
@@ -1558,6 +1557,7 @@ pf_status pf_set_tiling(pf_ctx* ctx, const pf_tiling* t) {
   m.bps = t->blocks_per_sm;
   drop_graphs(ctx);
   ctx->L.march = m;
+  ctx->L.tiled = 1;
   ctx->tile_bps = t->blocks_per_sm;
   ctx->mg_whole = t->mg_whole;
   ctx->gen += 1;

@@ -267,8 +267,10 @@ static void launch_cg_p_t(const LaunchCfg& L, const Geo& g, const Dev<T>& d) {
     allow_smem(k_cg_p<T, EPS, MG, VX, DIRECT, FIRST, SECOND>, bytes);
     once = true;
   }
-  k_cg_p<T, EPS, MG, VX, DIRECT, FIRST, SECOND><<<L.march.grid, dim3(MTX, MTY), bytes, L.stream>>>(
-      g, d.bc, d.eps, d.invd, MG ? d.z : d.r, d.p0, d.p1, d.q, d.phi, d.part, d.S, L.march);
+  static int occ = 0;
+  const MarchCfg mc = kernel_tiling(k_cg_p<T, EPS, MG, VX, DIRECT, FIRST, SECOND>, bytes, L, occ, true);
+  k_cg_p<T, EPS, MG, VX, DIRECT, FIRST, SECOND><<<mc.grid, dim3(MTX, MTY), bytes, L.stream>>>(
+      g, d.bc, d.eps, d.invd, MG ? d.z : d.r, d.p0, d.p1, d.q, d.phi, d.part, d.S, mc);
 }
 
 template <typename T, bool EPS, bool MG, bool FIRST = false, bool SECOND = false>

@@ -103,8 +103,9 @@ static void diag_t(const LaunchCfg& L, const Geo& g, const Dev<T>& d, const T* P
     allow_smem(k_diag<T, VX>, bytes);
     once = true;
   }
-  k_diag<T, VX><<<L.march.grid, dim3(MTX, MTY), bytes, L.stream>>>(g, d.bc, P, d.phi, k, out, d.part, d.S,
-                                                                   L.march);
+  static int occ = 0;
+  const MarchCfg mc = kernel_tiling(k_diag<T, VX>, bytes, L, occ, true);
+  k_diag<T, VX><<<mc.grid, dim3(MTX, MTY), bytes, L.stream>>>(g, d.bc, P, d.phi, k, out, d.part, d.S, mc);
 }
 
 template <typename T>

@@ -7,6 +7,7 @@
 #include <stdint.h>
 
 #include <algorithm>
+#include <cmath>
 
 #include "pf.h"
 #include "pf_common.cuh"
@@ -36,10 +37,16 @@ inline bool mg_split_level(long long n, int nz, int periodic_z, int eps) {
   return !periodic_z && nz >= 2 * MG_SPLIT_B + 2 && n >= (eps ? MG_SPLIT_CELLS_EPS : MG_SPLIT_CELLS);
 }
 
+constexpr int PLAN_OCC = 6;      // tilings are planned for up to this many blocks per SM
+
 struct LaunchCfg {
   int grid;            // simple per-cell kernels (TX x TY blocks over tiles)
   dim3 block;
-  MarchCfg march;      // plane-march kernels (MTX x MTY blocks)
+  MarchCfg march;      // plane-march kernels (MTX x MTY blocks): the tiling asked for
+                       // (tiled = 1), or the default of the CG operator
+  int tiled;           // 1: a tiling was set (pf_set_tiling); 0: every kernel plans its own
+  int nsm, word, nx, ny, nz;
+  mutable MarchCfg plan[2][PLAN_OCC];   // planned tilings (ntiles = 0: not yet), see kernel_tiling
   int flat_grid;       // flat vector kernels (FLAT_THREADS blocks, grid-stride)
   cudaStream_t stream;
 };
@@ -194,12 +201,71 @@ void launch_batch_ramp(const BatchFilm* films, int nfilms, long long max_nxy, co
 void launch_batch_record(const BatchFilm* films, int nfilms, int buf, BatchState* bs, double* part, double* hist,
                          cudaStream_t st);
 
-// Tiling of a plane-march launch on an nx x ny x nz grid: the deepest z
-// chunk that still gives about three tiles per resident block.
 // Resident plane-march blocks (MTX x MTY threads) per SM for this precision.
 int march_blocks_per_sm(int fp32, int eps);
 
-inline MarchCfg march_cfg(int nx, int ny, int nz, int resident, bool even_tz, int word) {
+// Relative time of a plane-march launch whose tiles are cols columns of tz
+// planes (the last one shorter) on nsm SMs with occ resident blocks each.
+// A tile costs its planes plus the pipeline's fill and the two halo planes
+// (about 3 planes in FP32; FP64 marches are bound by the FP64 unit, which the
+// halo planes do not use: half a plane).  The tiles go to the SMs in order,
+// each to the first one free (groups of SMs free at the same time are kept
+// together); b blocks sharing an SM take 1 + k (b - 1) times as long as one
+// alone, k = 0.6 in FP32 and 0.8 in FP64 (fitted to sweeps of the depth).
+inline double march_cost(long long cols, int nz, int tz, int nsm, int occ, int word) {
+  const double c = word == 4 ? 3.0 : 0.5, k = word == 4 ? 0.6 : 0.8;
+  struct Group {
+    double t;
+    long long m;
+  };
+  Group q[160];
+  int nq = 1;
+  q[0] = Group{0.0, nsm};
+  auto insert = [&](double t, long long m) {      // groups in ascending order of t
+    int i = nq;
+    while (i > 0 && q[i - 1].t > t) --i;
+    if (i > 0 && q[i - 1].t == t) {
+      q[i - 1].m += m;
+      return;
+    }
+    for (int j = nq; j > i; --j) q[j] = q[j - 1];
+    q[i] = Group{t, m};
+    ++nq;
+  };
+  double span = 0.0;
+  for (int z = 0; z < nz; z += tz) {
+    const double d = std::min(tz, nz - z) + c;
+    for (long long left = cols; left > 0;) {
+      const double t = q[0].t;
+      long long m = q[0].m, rounds = 1;
+      if (nq == 1 && left > m) rounds = left / m;   // every SM free at once: whole rounds
+      m = std::min(m, left);
+      if (m == q[0].m) {
+        for (int j = 1; j < nq; ++j) q[j - 1] = q[j];
+        --nq;
+      } else {
+        q[0].m -= m;
+      }
+      insert(t + rounds * d, m);
+      span = std::max(span, t + rounds * d);
+      left -= m * rounds;
+    }
+  }
+  const double tiles = span / (std::min(tz, nz) + c);      // whole tiles on the busiest SM
+  const double full = std::floor(tiles / occ), rest = tiles - full * occ;
+  const double f = full * (1.0 + k * (occ - 1)) + (rest <= 1.0 ? rest : 1.0 + k * (rest - 1));
+  return span * f / tiles;
+}
+
+// Tiling of a plane march over an nx x ny x nz grid: 16 bytes of cells per
+// thread when nx allows it, and the tile depth (at most tzmax planes, even for
+// even_tz) of least march_cost.  One rule for every size: a film of 1024 x 1024
+// columns takes the deepest tiles, one of 64 x 64 a couple of planes per tile.
+// (The rule before it, the deepest of 32 .. 2 planes with three tiles per
+// resident block, gave a 256 x 256 x 64 film tiles of 2 planes: 55 us for the
+// right-hand side, 33 for the search direction; planned, 39 with 16 planes and
+// 22 with 10.)
+inline MarchCfg march_cfg(int nx, int ny, int nz, int nsm, int occ, int tzmax, bool even_tz, int word) {
   MarchCfg m{};
   const int v = 16 / word;
   m.vx = nx % v == 0 ? v : 1;
@@ -207,15 +273,48 @@ inline MarchCfg march_cfg(int nx, int ny, int nz, int resident, bool even_tz, in
   m.tiles_x = (nx + bx - 1) / bx;
   m.tiles_y = (ny + MTY - 1) / MTY;
   const long long cols = (long long)m.tiles_x * m.tiles_y;
+  double best = 0.0;
   m.tz = even_tz ? 2 : 1;
-  for (int tz : {32, 16, 8, 4, 2}) {
-    if (cols * ((nz + tz - 1) / tz) >= 3LL * resident) {
+  int last = 0;
+  for (int tz = std::min(tzmax, nz); tz >= 1; --tz) {
+    if (even_tz && (tz & 1)) continue;
+    const int chunks = (nz + tz - 1) / tz;
+    if (chunks > 128) break;
+    // of the depths with this many chunks: the deepest, the even split, multiples of 8
+    if (chunks == last && (nz + chunks - 1) / chunks != tz && tz % 8 != 0) continue;
+    last = chunks;
+    const double cost = march_cost(cols, nz, tz, nsm, occ, word);
+    if (best == 0.0 || cost < 0.999 * best) {
+      best = cost;
       m.tz = tz;
-      break;
     }
   }
   m.ntiles = cols * ((nz + m.tz - 1) / m.tz);
-  m.grid = (int)std::min<long long>(m.ntiles, std::min(MAX_GRID, resident));
+  m.grid = (int)std::min<long long>(m.ntiles, std::min(MAX_GRID, nsm * occ));
+  return m;
+}
+
+// Tiling of one plane-march kernel on the fine grid (its shared-memory limit
+// already raised; occ caches its occupancy): the one asked for, on its own
+// occupancy, or the planned one.  deep: tiles of up to 64 planes (the kernels
+// that sum over their tiles), else 32 (the TDGL update on 1024 x 1024 x 128:
+// 1.00 ms with 32 planes, 1.02 with 64).
+template <class K>
+inline MarchCfg kernel_tiling(K kernel, size_t bytes, const LaunchCfg& L, int& occ, bool deep) {
+  if (occ == 0) {
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, MTX * MTY, bytes) != cudaSuccess) occ = 1;
+    cudaGetLastError();
+    occ = std::max(occ, 1);
+  }
+  if (L.tiled) {
+    MarchCfg m = L.march;
+    const int bps = m.bps > 0 ? std::min(m.bps, occ) : occ;
+    m.grid = (int)std::min<long long>(m.ntiles, std::min<long long>(MAX_GRID, (long long)bps * L.nsm));
+    return m;
+  }
+  const int o = std::min(occ, PLAN_OCC);
+  MarchCfg& m = L.plan[deep ? 1 : 0][o - 1];
+  if (m.ntiles == 0) m = march_cfg(L.nx, L.ny, L.nz, L.nsm, o, deep ? 64 : 32, false, L.word);
   return m;
 }
 
@@ -246,8 +345,12 @@ inline void setup_launch(const pf_params* p, int nsm, cudaStream_t stream, Geo& 
   g.ntiles = cols * g.tiles_z;
   L = LaunchCfg{};
   const int fp32 = p->precision == PF_FP32;
-  const int resident = nsm * march_blocks_per_sm(fp32, p->has_eps);
-  L.march = march_cfg(g.nx, g.ny, g.nz, resident, false, fp32 ? 4 : 8);
+  L.nsm = nsm;
+  L.word = fp32 ? 4 : 8;
+  L.nx = g.nx;
+  L.ny = g.ny;
+  L.nz = g.nz;
+  L.march = march_cfg(g.nx, g.ny, g.nz, nsm, std::min(PLAN_OCC, march_blocks_per_sm(fp32, p->has_eps)), 64, false, L.word);
   const long long nvec = (g.n + 3) / 4;
   L.flat_grid = (int)std::max<long long>(
       1, std::min<long long>((nvec + FLAT_THREADS - 1) / FLAT_THREADS, std::min(MAX_GRID, 4 * nsm)));
@@ -292,8 +395,6 @@ template <typename T>
 int launch_mg_post1(const LaunchCfg& L, const MgView<T>& lv, const MgView<T>& cv, Scalars* S);
 template <typename T>
 int launch_mg_post2(const LaunchCfg& L, const MgView<T>& lv, int last, double* part, Scalars* S);
-template <typename T>
-int mg_blocks_per_sm();
 // Permittivity of a coarse level (the mean of the fine children, into ceps)
 // and 1/diag of its operator (into cinvd).
 template <typename T>

@@ -1547,19 +1547,6 @@ void launch_mg_tail(const LaunchCfg& L, const MgTail<T>& t, int singular, Scalar
   k_mg_tail<T><<<1, MG_MAX_COARSE, (size_t)t.smem_elems * sizeof(T), L.stream>>>(t, singular, S);
 }
 
-template <typename T>
-int mg_blocks_per_sm() {
-  constexpr int V = vec_of(sizeof(T));
-  allow_smem(k_mg_post1<T, V, false>, MgPipeP<T, V>::bytes());
-  int nb = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_mg_post1<T, V, false>, MTX * MTY,
-                                                    MgPipeP<T, V>::bytes()) != cudaSuccess) {
-    cudaGetLastError();
-    return 1;
-  }
-  return nb > 0 ? nb : 1;
-}
-
 #define PF_MG_INSTANTIATE(T)                                                           \
   template int launch_mg_pre<T>(const LaunchCfg&, const MgView<T>&, Scalars*);                   \
   template int launch_mg_rr<T>(const LaunchCfg&, const MgView<T>&, const MgView<T>&, Scalars*);  \
@@ -1572,8 +1559,7 @@ int mg_blocks_per_sm() {
   template void launch_mg_tail<T>(const LaunchCfg&, const MgTail<T>&, int, Scalars*);            \
   template int launch_mg_post1<T>(const LaunchCfg&, const MgView<T>&, const MgView<T>&, Scalars*); \
   template int launch_mg_post2<T>(const LaunchCfg&, const MgView<T>&, int, double*, Scalars*);         \
-  template void launch_mg_eps_level<T>(const LaunchCfg&, const MgView<T>&, const MgView<T>&, T*, T*);  \
-  template int mg_blocks_per_sm<T>();
+  template void launch_mg_eps_level<T>(const LaunchCfg&, const MgView<T>&, const MgView<T>&, T*, T*);
 
 PF_MG_INSTANTIATE(float)
 PF_MG_INSTANTIATE(double)

@@ -855,31 +855,15 @@ static void smem_attr(K kernel, size_t bytes, bool& done) {
 // the march's tiles are whole 64 x 16 tiles.
 static bool rhs_whole(const Geo& g, const MarchCfg& mc) { return mc.vx == 4 && g.nx % 64 == 0 && g.ny % MTY == 0; }
 
-// Grid of a whole-tile kernel: its own occupancy (or the blocks per SM a
-// tiling asked for, if fewer) on every SM, at most a block per tile.
-template <class K>
-static int own_grid(K kernel, size_t bytes, const MarchCfg& mc, int& occ, int& nsm) {
-  if (occ == 0) {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-      nsm = 1;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, MTX * MTY, bytes) != cudaSuccess) occ = 1;
-    cudaGetLastError();
-    occ = std::max(occ, 1);
-  }
-  const int bps = mc.bps > 0 ? std::min(mc.bps, occ) : occ;
-  return (int)std::min<long long>(mc.ntiles, std::min<long long>(MAX_GRID, (long long)bps * nsm));
-}
-
 static void rhs_w(const LaunchCfg& L, const Geo& g, const Dev<float>& d, const float* P, cudaGraphConditionalHandle cond,
                   int use_cond) {
   static bool f = false;
-  static int occ = 0, nsm = 0;
+  static int occ = 0;
   const size_t bytes = rhs_w_smem_bytes();
   smem_attr(k_rhs_w, bytes, f);
-  const int grid = own_grid(k_rhs_w, bytes, L.march, occ, nsm);
-  k_rhs_w<<<grid, dim3(MTX, MTY), bytes, L.stream>>>(g, d.bc, P, d.cp.hi, d.cp.lo, d.r, d.part, d.S, L.march, cond,
-                                                     use_cond);
+  const MarchCfg mc = kernel_tiling(k_rhs_w, bytes, L, occ, true);
+  k_rhs_w<<<mc.grid, dim3(MTX, MTY), bytes, L.stream>>>(g, d.bc, P, d.cp.hi, d.cp.lo, d.r, d.part, d.S, mc, cond,
+                                                        use_cond);
 }
 
 template <typename T, bool EPS, bool MEAN, int VX, bool COMP>
@@ -894,8 +878,10 @@ static void rhs_t(const LaunchCfg& L, const Geo& g, const Dev<T>& d, const T* P,
   static bool f = false;
   const size_t bytes = StepPipe<T, EPS, VX, COMP ? 1 : 0>::bytes();
   smem_attr(k_rhs<T, EPS, MEAN, VX, COMP>, bytes, f);
-  k_rhs<T, EPS, MEAN, VX, COMP><<<L.march.grid, dim3(MTX, MTY), bytes, L.stream>>>(
-      g, d.bc, P, COMP ? d.cp.hi : d.phi, d.cp.lo, d.eps, d.invd, d.r, d.part, d.S, L.march, cond, use_cond);
+  static int occ = 0;
+  const MarchCfg mc = kernel_tiling(k_rhs<T, EPS, MEAN, VX, COMP>, bytes, L, occ, true);
+  k_rhs<T, EPS, MEAN, VX, COMP><<<mc.grid, dim3(MTX, MTY), bytes, L.stream>>>(
+      g, d.bc, P, COMP ? d.cp.hi : d.phi, d.cp.lo, d.eps, d.invd, d.r, d.part, d.S, mc, cond, use_cond);
 }
 
 template <typename T, bool MEAN, bool COMP>
@@ -941,8 +927,10 @@ static void tdgl_t(const LaunchCfg& L, const Geo& g, const Dev<T>& d, const T* P
   static bool f = false;
   const size_t bytes = StepPipe<T, false, VX>::bytes();
   smem_attr(k_tdgl<T, CORR, NOISE, VX, COMP>, bytes, f);
-  k_tdgl<T, CORR, NOISE, VX, COMP><<<L.march.grid, dim3(MTX, MTY), bytes, L.stream>>>(g, d.bc, P, Pn, d.phi, k, d.S,
-                                                                                     L.march, d.plo);
+  static int occ = 0;
+  const MarchCfg mc = kernel_tiling(k_tdgl<T, CORR, NOISE, VX, COMP>, bytes, L, occ, false);
+  k_tdgl<T, CORR, NOISE, VX, COMP><<<mc.grid, dim3(MTX, MTY), bytes, L.stream>>>(g, d.bc, P, Pn, d.phi, k, d.S, mc,
+                                                                                d.plo);
 }
 
 template <typename T, bool CORR, bool NOISE>
@@ -953,11 +941,11 @@ static void tdgl_v(const LaunchCfg& L, const Geo& g, const Dev<T>& d, const T* P
     if constexpr (!NOISE) {
       if (d.plo && rhs_whole(g, L.march)) {       // whole 64 x 16 tiles
         static bool f = false;
-        static int occ = 0, nsm = 0;
+        static int occ = 0;
         const size_t bytes = tdgl_w_smem_bytes();
         smem_attr(k_tdgl_w, bytes, f);
-        const int grid = own_grid(k_tdgl_w, bytes, L.march, occ, nsm);
-        k_tdgl_w<<<grid, dim3(MTX, MTY), bytes, L.stream>>>(g, d.bc, P, Pn, d.phi, k, d.S, L.march, d.plo);
+        const MarchCfg mc = kernel_tiling(k_tdgl_w, bytes, L, occ, false);
+        k_tdgl_w<<<mc.grid, dim3(MTX, MTY), bytes, L.stream>>>(g, d.bc, P, Pn, d.phi, k, d.S, mc, d.plo);
         return;
       }
     }
