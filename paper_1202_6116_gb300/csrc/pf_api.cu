@@ -80,6 +80,10 @@ struct Layout {
       total;
   bool adj = false;               // psi and vzero exist (PF_FLAG_ADJOINT)
   size_t psi = 0, vzero = 0;      // adjoint potential; zero face voltages
+  size_t cinv = 0;                // inverse of the coarsest multigrid operator (and scratch of two columns)
+  size_t blob = 0;                // descriptors and masks of the small levels' launch
+  size_t tail0 = 0;               // the first of those levels
+  pf::MgTail tail{};
   std::vector<MgLevelHost> mg;
 };
 
@@ -136,6 +140,33 @@ bool comp_buffers(const pf_params* p) { return extrapolates(p) && p->precision =
 bool comp_state(const pf_params* p) {
   return p->precision == PF_FP32 && p->integrator == PF_EULER &&
          !(p->flags & (PF_FLAG_PLAIN_FP32 | PF_FLAG_ADJOINT));
+}
+
+// Which levels the small levels' launch takes (from the first of at most
+// mg_sub_cells cells on), where one block takes over (the first level small
+// enough for it from which on all levels' arrays and masks fit in its shared
+// memory), and the sizes of its blob and its shared memory.
+void mg_tail_layout(Layout& L, size_t word) {
+  const size_t nl = L.mg.size();
+  size_t k0 = nl - 1;
+  while (k0 > 0 && L.mg[k0 - 1].n() <= pf::mg_sub_cells(word)) --k0;
+  const size_t desc = word == 4 ? sizeof(pf::SubDesc<float>) : sizeof(pf::SubDesc<double>);
+  auto up16 = [](size_t v) { return (v + 15) / 16 * 16; };
+  auto fields = [&](size_t k) { return 3 * (size_t)L.mg[k].n() * word; };
+  auto masks = [&](size_t k) { return 2 * (size_t)L.mg[k].nxy(); };
+  size_t b0 = nl - 1, fb = fields(b0), mb = masks(b0);
+  while (b0 > k0 && L.mg[b0 - 1].n() <= pf::mg_solo_cells(word) &&
+         (nl - k0) * desc + fb + mb + fields(b0 - 1) + masks(b0 - 1) + 32 <= (size_t)pf::MG_TAIL_SMEM) {
+    --b0;
+    fb += fields(b0);
+    mb += masks(b0);
+  }
+  L.tail0 = k0;
+  L.tail.nl = (int)(nl - k0);
+  L.tail.solo = (int)(b0 - k0);
+  L.tail.coarse = (int)L.mg[nl - 1].n();
+  L.tail.blob_bytes = (int)up16((nl - k0) * desc + mb);
+  L.tail.smem_bytes = L.tail.blob_bytes + (int)fb;
 }
 
 Layout layout_of(const pf_params* p) {
@@ -202,6 +233,10 @@ Layout layout_of(const pf_params* p) {
         }
       }
     }
+    const size_t nc = (size_t)L.mg.back().n();
+    L.cinv = take((nc * nc + 2 * nc) * sizeof(double));
+    mg_tail_layout(L, w);
+    L.blob = take((size_t)L.tail.blob_bytes);
   }
   L.total = off;
   return L;
@@ -232,6 +267,7 @@ struct pf_ctx {
   int cur = 0;                    // 0: state in P_user, 1: in the workspace copy
   int singular = 1;               // no Dirichlet face anywhere (or periodic z)
   bool invd_dirty = true;
+  bool cinv_dirty = true;         // the coarsest multigrid inverse is stale (bind, electrode layout)
   int est_iters = 8;              // iterations issued before the first poll
   int est_iters_adj = 8;          // the same for the adjoint solves
   std::vector<int8_t> tlo_h, thi_h;
@@ -463,32 +499,21 @@ void refresh_invd(pf_ctx* ctx, const pf::LaunchCfg& L, bool count) {
   ctx->invd_dirty = false;
 }
 
-// First level of the one-block V-cycle tail: the first level after the
-// finest with at most MG_TAIL_CELLS cells, or the coarsest level (no tail)
-// when that leaves fewer than two levels for the tail.
-size_t mg_tail_start(const Layout& lay, size_t word) {
-  const size_t nl = lay.mg.size();
-  size_t k0 = nl - 1;
-  for (size_t k = 1; k < nl; ++k)
-    if (lay.mg[k].n() <= pf::MG_TAIL_CELLS) {
-      k0 = k;
-      break;
-    }
-  // the tail's level arrays must fit in shared memory
-  for (; k0 + 1 < nl; ++k0) {
-    size_t cells = 0;
-    for (size_t k = k0; k < nl; ++k) cells += (size_t)lay.mg[k].n();
-    if (3 * cells * word <= (size_t)pf::MG_TAIL_SMEM && nl - k0 <= (size_t)pf::MG_TAIL_LEVELS) break;
-  }
-  return k0;
+// Refresh whatever depends on the permittivity and the electrode layout.
+template <typename T>
+void refresh_operators(pf_ctx* ctx, const pf::LaunchCfg& L, bool count) {
+  refresh_invd<T>(ctx, L, count);
+  if (ctx->prm.solver != PF_PCG_MG || !ctx->cinv_dirty) return;
+  ctx->launches += pf::launch_coarse_inverse<T>(L, mg_view<T>(ctx, ctx->lay.mg.size() - 1), ctx->singular,
+                                                (double*)(ctx->ws + ctx->lay.cinv));
+  ctx->cinv_dirty = false;
 }
 
 // One V-cycle z = M^-1 r (number j of its solve, for the profiler): one
-// kernel per phase down to level k0, the rest of the cycle in one block.
+// kernel per phase down to level k0, the rest of the cycle in one launch.
 template <typename T>
 void vcycle(pf_ctx* ctx, int j) {
-  const size_t nl = ctx->lay.mg.size();
-  const size_t k0 = mg_tail_start(ctx->lay, sizeof(T));
+  const size_t k0 = ctx->lay.tail0;
   const double w = sizeof(T);
   pf::Scalars* S = (pf::Scalars*)(ctx->ws + ctx->lay.S);
   double* part = (double*)(ctx->ws + ctx->lay.part);
@@ -522,26 +547,10 @@ void vcycle(pf_ctx* ctx, int j) {
     after_launch(ctx, mg_fam(F_MG_RR, k), (2 + e + rest) * N * w, 2, j);
     ctx->launches += nk - 1;
   }
-  if (k0 + 1 < nl) {
-    pf::MgTail<T> t{};
-    t.nl = (int)(nl - k0);
-    int off = 0;
-    for (size_t k = k0; k < nl; ++k) {
-      t.lv[k - k0] = mg_view<T>(ctx, k);
-      t.off[k - k0] = off;
-      off += 3 * (int)t.lv[k - k0].g.n;
-    }
-    t.smem_elems = off;
-    const double cells = (double)t.lv[0].g.n;
-    before_launch(ctx);
-    pf::launch_mg_tail<T>(ctx->L, t, ctx->singular, S);
-    after_launch(ctx, mg_fam(F_MG_COARSE, k0), 2.0 * cells * w, 2, j);
-  } else {
-    const pf::MgView<T> cv = mg_view<T>(ctx, nl - 1);
-    before_launch(ctx);
-    pf::launch_mg_coarse<T>(ctx->L, cv, ctx->singular, S);
-    after_launch(ctx, mg_fam(F_MG_COARSE, nl - 1), 2.0 * (double)cv.g.n * w, 2, j);
-  }
+  before_launch(ctx);
+  pf::launch_mg_sub<T>(ctx->L, ctx->lay.tail, ctx->prm.has_eps, ctx->ws + ctx->lay.blob,
+                       (const double*)(ctx->ws + ctx->lay.cinv), k0 == 0, part, S);
+  after_launch(ctx, mg_fam(F_MG_COARSE, k0), 2.0 * (double)ctx->lay.mg[k0].n() * w, 2, j);
   for (size_t k = k0; k-- > 0;) {
     const pf::MgView<T> lv = view(k), cv = view(k + 1);
     const double N = (double)lv.g.n;
@@ -682,7 +691,7 @@ pf_status solve(pf_ctx* ctx, const T* P, bool adj = false, bool step_solve = fal
   int& est_iters = adj ? ctx->est_iters_adj : ctx->est_iters;
   const Geo& g = ctx->geo;
   const double N = (double)g.n, w = sizeof(T), e = ctx->prm.has_eps ? 1.0 : 0.0;
-  refresh_invd<T>(ctx, ctx->L, true);
+  refresh_operators<T>(ctx, ctx->L, true);
   if (step_solve && plain_extrap(ctx)) {
     before_launch(ctx);
     launch_extrap_of<T>(ctx, ctx->L);
@@ -762,11 +771,10 @@ bool refresh_step(const pf_ctx* ctx) {
 }
 
 // Kernels of one step outside the Krylov loops, and per Krylov iteration.
-// Kernels of one V-cycle: four per level above the tail (two for a split
-// level's pre and post1, and for its post2 below the finest), plus the tail or
-// the coarse solve.
+// Kernels of one V-cycle: four per level above the small ones (two for a split
+// level's pre and post1, and for its post2 below the finest), plus their launch.
 int64_t vcycle_kernels(const pf_ctx* ctx) {
-  const size_t k0 = mg_tail_start(ctx->lay, ctx->prm.precision == PF_FP32 ? 4 : 8);
+  const size_t k0 = ctx->lay.tail0;
   int64_t n = 1;
   for (size_t k = 0; k < k0; ++k) {
     const MgLevelHost& l = ctx->lay.mg[k];
@@ -971,7 +979,7 @@ bool run_steps_graph(pf_ctx* ctx, int nsteps, pf_status* st) {
     }
     ctx->graph_key = ctx->singular;
   }
-  refresh_invd<T>(ctx, ctx->L, false);
+  refresh_operators<T>(ctx, ctx->L, false);
   const bool heun = ctx->prm.integrator == PF_HEUN;
   // many forward-Euler steps that all solve: pairs of them in one persistent launch
   if (!heun && ctx->prm.poisson_every <= 1 && ctx->cur == 0 && nsteps >= 4 && !ctx->loop_broken) {
@@ -1082,6 +1090,56 @@ pf_status run_steps(pf_ctx* ctx, int nsteps, bool keep_parity = false) {
   return consolidate<T>(ctx);
 }
 
+// The blob of the small levels' launch: masks[2k], masks[2k+1] are the face
+// masks of level k.
+template <typename T>
+std::vector<char> tail_blob(pf_ctx* ctx, const std::vector<std::vector<int8_t>>& masks) {
+  const Layout& L = ctx->lay;
+  std::vector<char> out((size_t)L.tail.blob_bytes, 0);
+  size_t off = 0, moff = (size_t)L.tail.nl * sizeof(pf::SubDesc<T>);
+  for (int k = 0; k < L.tail.nl; ++k) {
+    const MgLevelHost& l = L.mg[L.tail0 + k];
+    const pf::MgView<T> v = mg_view<T>(ctx, L.tail0 + k);
+    pf::SubDesc<T> d{};
+    d.nx = l.nx;
+    d.ny = l.ny;
+    d.nz = l.nz;
+    d.nxy = (int)l.nxy();
+    d.n = (int)l.n();
+    d.per = ctx->prm.periodic_z;
+    d.fx = l.fx;
+    d.fy = l.fy;
+    d.fz = l.fz;
+    d.rnx = 1.0f / (float)l.nx;
+    d.rny = 1.0f / (float)l.ny;
+    d.ax = v.ax;
+    d.ay = v.ay;
+    d.az = v.az;
+    for (int i = 0; i < 9; ++i) {
+      auto faces = [](int kind) { return kind == 0 ? 1 : 2 * (kind - 1); };
+      d.tab[i] = T(1) / (T(2) * v.ax + T(2) * v.ay + T(faces(i / 3) + faces(i % 3)) * v.az);
+    }
+    d.f = v.f;
+    d.e = v.e;
+    d.et = v.et;
+    d.tlo = v.tlo;
+    d.thi = v.thi;
+    d.eps = v.eps;
+    d.invd = v.invd;
+    if (k >= L.tail.solo) {
+      d.off = (int)((size_t)L.tail.blob_bytes / sizeof(T) + off);
+      off += 3 * (size_t)l.n();
+      d.moff = (int)moff;
+      const size_t nxy = (size_t)l.nxy(), m = 2 * (L.tail0 + k);
+      std::memcpy(out.data() + moff, masks[m].data(), nxy);
+      std::memcpy(out.data() + moff + nxy, masks[m + 1].data(), nxy);
+      moff += 2 * nxy;
+    }
+    std::memcpy(out.data() + (size_t)k * sizeof(d), &d, sizeof(d));
+  }
+  return out;
+}
+
 // Copy the host face masks to the device: the fine level and, for the
 // multigrid hierarchy, every coarse level (a coarse face cell is an electrode
 // where any of its fine children is).  Waits for the copies.
@@ -1112,6 +1170,11 @@ pf_status upload_masks(pf_ctx* ctx) {
                             ctx->stream));
     PF_CUDA(cudaMemcpyAsync(ctx->ws + c.thi, masks[2 * k + 3].data(), (size_t)c.nxy(), cudaMemcpyHostToDevice,
                             ctx->stream));
+  }
+  std::vector<char> blob;
+  if (!L.mg.empty()) {
+    blob = ctx->prm.precision == PF_FP32 ? tail_blob<float>(ctx, masks) : tail_blob<double>(ctx, masks);
+    PF_CUDA(cudaMemcpyAsync(ctx->ws + L.blob, blob.data(), blob.size(), cudaMemcpyHostToDevice, ctx->stream));
   }
   PF_CUDA(cudaStreamSynchronize(ctx->stream));
   return PF_OK;
@@ -1244,6 +1307,7 @@ pf_status pf_bind(pf_ctx* ctx, void* P, void* phi, const void* eps, void* worksp
   ctx->cur = 0;
   ctx->nstep = 0;
   ctx->invd_dirty = true;
+  ctx->cinv_dirty = true;
   const Layout& L = ctx->lay;
   PF_CUDA(cudaMemsetAsync(ctx->ws + L.tlo, 0, L.part - L.tlo, ctx->stream));
   std::fill(ctx->tlo_h.begin(), ctx->tlo_h.end(), 0);
@@ -1296,6 +1360,7 @@ pf_status pf_set_bc(pf_ctx* ctx, int32_t face, const int8_t* type_xy, const doub
   ctx->invd_dirty = true;
   ctx->gen += 1;
   if (types_changed) {           // a new electrode layout: the old potentials are no guide
+    ctx->cinv_dirty = true;
     st = reset_history(ctx);
     if (st != PF_OK) return st;
   }
@@ -1876,8 +1941,8 @@ pf_status pf_batch_step(pf_batch* b, int32_t nsteps, pf_step_info* info) {
   for (pf_ctx* c : b->films) {
     pf_status st = reset_scalars(c);
     if (st != PF_OK) return b->fail(st, "film: %s", c->err.c_str());
-    if (c->prm.precision == PF_FP32) refresh_invd<float>(c, c->L, false);
-    else refresh_invd<double>(c, c->L, false);
+    if (c->prm.precision == PF_FP32) refresh_operators<float>(c, c->L, false);
+    else refresh_operators<double>(c, c->L, false);
   }
   const bool heun = f0->prm.integrator == PF_HEUN;
   auto book = [&](int refresh, long long steps) {    // host bookkeeping of graph-run steps

@@ -213,18 +213,18 @@ __device__ __forceinline__ float2 sum_xor(float2 v, int o) {
 __device__ __forceinline__ double sum_double(double v) { return v; }
 __device__ __forceinline__ double sum_double(float2 v) { return (double)v.x + (double)v.y; }
 
-// Sums of NV values over the NT = 256 threads of a block; the sum of value k
-// is returned (as a double) in lane 0 of warp k.  Every thread must call it;
+// Sums of NV values over the NT threads of a block; the sum of value k
+// is returned (as a double) in lane 0 of warp k.  Every thread must call it
+// with its linear index;
 // it ends without a barrier.  Warp k adds value k of all threads from shared
-// memory: 12 additions a value, where a shuffle tree in each of the eight
-// warps takes 45.  sm: sum_scratch<V>(NV) bytes, 8-byte aligned, that nobody
+// memory: 12 additions a value with 256 threads, where a shuffle tree in each
+// of the eight warps takes 45.  sm: sum_scratch<V>(NV) bytes, 8-byte aligned, that nobody
 // else uses until the block's next barrier -- the plane marches lend their
 // staging buffers, which are idle between tiles (12 KB of static shared
 // memory beside them shrank the L1 and cost k_rhs_w 7 %).  Not inlined: it
 // runs once per tile, and its temporaries would count in the march.
 template <int NV, int NT, typename V>
-__device__ __noinline__ double shared_sums(const V* sm) {
-  const int tid = threadIdx.x + threadIdx.y * blockDim.x;
+__device__ __noinline__ double shared_sums(const V* sm, int tid) {
   const int lane = tid & 31, wid = tid >> 5;
   V d = sm[wid * NT + lane];
 #pragma unroll
@@ -234,15 +234,14 @@ __device__ __noinline__ double shared_sums(const V* sm) {
   return sum_double(d);
 }
 template <int NV, int NT, typename V>
-__device__ __forceinline__ double block_sums(const V (&v)[NV], void* scratch) {
-  static_assert(NT == 256 && NV <= 8, "eight warps, a value per warp");
+__device__ __forceinline__ double block_sums(const V (&v)[NV], void* scratch, int tid) {
+  static_assert(NT % 32 == 0 && NV * 32 <= NT, "a value per warp");
   V* sm = static_cast<V*>(scratch);
-  const int tid = threadIdx.x + threadIdx.y * blockDim.x;
   __syncthreads();                 // the scratch may still be read
 #pragma unroll
   for (int k = 0; k < NV; ++k) sm[k * NT + tid] = v[k];
   __syncthreads();
-  return (tid >> 5) < NV ? shared_sums<NV, NT>(sm) : 0.0;
+  return (tid >> 5) < NV ? shared_sums<NV, NT>(sm, tid) : 0.0;
 }
 
 // Block-reduce NV values of one work tile and store them at part[t*NV + k].
@@ -251,8 +250,8 @@ __device__ __forceinline__ double block_sums(const V (&v)[NV], void* scratch) {
 // Must be called by every thread of the block (scratch: see block_sums).
 template <int NV, int NT, typename V>
 __device__ __forceinline__ void tile_partials(const V (&v)[NV], double* part, long long t, void* scratch) {
-  const double d = block_sums<NV, NT>(v, scratch);
   const int tid = threadIdx.x + threadIdx.y * blockDim.x;
+  const double d = block_sums<NV, NT>(v, scratch, tid);
   if ((tid & 31) == 0 && (tid >> 5) < NV) part[t * NV + (tid >> 5)] = d;
 }
 
@@ -296,7 +295,7 @@ __device__ __forceinline__ void gather_partials(const double* part, long long nb
 #pragma unroll
     for (int k = 0; k < NV; ++k) acc[k] += __ldcg(part + i * NV + k);
   }
-  const double d = block_sums<NV, NT>(acc, scratch);
+  const double d = block_sums<NV, NT>(acc, scratch, tid);
   if ((tid & 31) == 0 && (tid >> 5) < NV) res[tid >> 5] = d;
   __syncthreads();
 #pragma unroll

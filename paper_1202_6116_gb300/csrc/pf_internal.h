@@ -17,10 +17,14 @@ namespace pf {
 constexpr int MAX_GRID = 4096;   // reduction partials are sized for this many blocks
 constexpr int MAX_NV = 8;        // values reduced per block or tile
 constexpr int MG_MAX_LEVELS = 24;
-constexpr int MG_MAX_COARSE = 1024;   // cells of the coarsest multigrid level (one block)
-constexpr int MG_TAIL_CELLS = 4096;   // levels at most this large run in the one-block V-cycle tail
-constexpr int MG_TAIL_LEVELS = 16;
-constexpr int MG_TAIL_SMEM = 192 * 1024;   // shared-memory limit of the tail's level arrays (bytes)
+constexpr int MG_MAX_COARSE = 1024;   // cells of the coarsest multigrid level (solved by its inverse)
+// The V-cycle's small levels run as one cluster launch (pf_coarse.cu): from
+// the first level of at most mg_sub_cells on; its levels of at most
+// mg_solo_cells in one block of the cluster.
+inline long long mg_sub_cells(size_t word) { return word == 4 ? 65536 : 16384; }
+inline long long mg_solo_cells(size_t word) { return word == 4 ? 4096 : 256; }
+constexpr int MG_TAIL_LEVELS = 24;
+constexpr int MG_TAIL_SMEM = 192 * 1024;   // shared-memory limit of the solo levels' arrays (bytes)
 // A multigrid sweep over a large level whose z faces are not periodic runs as
 // two launches: the interior planes [b, nz - b), compiled without the face
 // code (fewer registers, more resident blocks), and the two face slabs of b
@@ -99,14 +103,28 @@ struct MgView {
   int split;          // 1: its split sweeps run as interior + face-slab launches (mg_split_level)
 };
 
-// The small levels of the V-cycle (lv[0] .. lv[nl - 1], the last one the
-// coarsest) handled by one block.
-template <typename T>
+// The small levels of the V-cycle, handled by one cluster (pf_coarse.cu): nl
+// levels, those from solo on by the cluster's first block, the coarsest of
+// coarse cells.
 struct MgTail {
-  MgView<T> lv[MG_TAIL_LEVELS];
-  int off[MG_TAIL_LEVELS];   // shared-memory offset (elements) of level k's f, e, e_tmp
-  int nl;
-  int smem_elems;            // 3 x the cells of all tail levels
+  int nl, solo, coarse;
+  int blob_bytes;             // descriptors and solo masks, a multiple of 16
+  int smem_bytes;             // the blob, then the solo levels' f, e, e_tmp
+};
+
+// One of those levels, as the kernel reads it (host-filled, see MgTail).
+template <typename T>
+struct SubDesc {
+  int nx, ny, nz, nxy, n, per;
+  int fx, fy, fz;             // coarsening factors to the next level
+  int off, moff;              // shared memory: element offset of the fields, byte offset of the masks (solo levels)
+  float rnx, rny;             // 1 / nx, 1 / ny
+  T ax, ay, az;
+  T tab[9];                   // 1/diag with eps = 1, by 3 (kind of the lower z face) + kind of the upper one
+                              // (0 interior, 1 open, 2 electrode)
+  T *f, *e, *et;
+  const int8_t *tlo, *thi;
+  const T *eps, *invd;
 };
 
 template <typename T>
@@ -387,10 +405,16 @@ bool mg_fused_post(const MgView<T>& lv);
 template <typename T>
 int launch_mg_pp(const LaunchCfg& L, const MgView<T>& lv, const MgView<T>& cv, T* ep, T* z, double* part,
                  Scalars* S, const std::function<void(int)>& mark);
+// The small levels (see MgTail; blob: their descriptors and masks in device
+// memory); cinv: the coarsest level's inverse; last: the first of them is the
+// finest level (r.z and beta are formed too).
 template <typename T>
-void launch_mg_coarse(const LaunchCfg& L, const MgView<T>& cv, int singular, Scalars* S);
+cudaError_t launch_mg_sub(const LaunchCfg& L, const MgTail& t, int eps, const void* blob, const double* cinv, int last,
+                          double* part, Scalars* S);
+// Inverse of the coarsest operator into cinv (n^2 doubles, and 2 n of
+// scratch after them); returns the launches.
 template <typename T>
-void launch_mg_tail(const LaunchCfg& L, const MgTail<T>& t, int singular, Scalars* S);
+int launch_coarse_inverse(const LaunchCfg& L, const MgView<T>& C, int singular, double* cinv);
 template <typename T>
 int launch_mg_post1(const LaunchCfg& L, const MgView<T>& lv, const MgView<T>& cv, Scalars* S);
 template <typename T>

@@ -9,8 +9,8 @@
 // scaled transpose), smoothing is two Jacobi sweeps with the Chebyshev weights
 // of mg_omega1/mg_omega2 before the coarse correction and the same two in
 // reverse order after it (the adjoint smoother), so the V-cycle is a symmetric
-// positive definite preconditioner.  The coarsest level (<= MG_MAX_COARSE cells) is
-// solved by FP64 conjugate gradients inside one thread block.
+// positive definite preconditioner.  The small levels, down to the product with
+// the coarsest level's inverse, run as one launch (pf_coarse.cu).
 //
 // With a permittivity field every level carries its own cell permittivity
 // (level 0: the bound eps; a coarse cell: the mean of its children) and 1/diag
@@ -28,40 +28,11 @@
 //                                                        reads et, f, writes e
 #include "pf_internal.h"
 #include "pf_march.cuh"
+#include "pf_mg.cuh"
 
 namespace pf {
 
 constexpr int MG_D = 2;   // planes of cp.async look-ahead
-
-// Jacobi weights of the two smoothing sweeps: the reciprocals of the roots of
-// the degree-2 Chebyshev polynomial on [b/4, b], b = 1.9, which bound the
-// spectrum of diag(A)^-1 A (in [0, 2] for this M-matrix) from below b/4 up,
-// i.e. 1/lambda_k with lambda_k = (b + a)/2 + (b - a)/2 cos((2k - 1) pi / 4),
-// a = b/4.  The pair damps the upper three quarters of the spectrum (the part
-// the coarse grid cannot represent) by |(1 - w1 l)(1 - w2 l)| <= 0.35 on
-// [b/4, 2]; weighted Jacobi with 6/7 twice leaves up to 0.51 there.  The
-// pre-smoother applies w1 then w2, the post-smoother w2 then w1.
-template <typename T>
-__device__ __forceinline__ T mg_omega1() {
-  return T(0.5912564121058501);
-}
-template <typename T>
-__device__ __forceinline__ T mg_omega2() {
-  return T(1.462658863889015);
-}
-
-// 1/diag of a level's operator at column xy of plane z.
-template <typename T>
-__device__ __forceinline__ T mg_inv(const MgView<T>& L, int xy, int z, T inv_int) {
-  if (L.g.periodic_z || (z > 0 && z < L.g.nz - 1)) return inv_int;
-  const int cz = (z > 0 ? 1 : 2 * (int)L.tlo[xy]) + (z < L.g.nz - 1 ? 1 : 2 * (int)L.thi[xy]);
-  return T(1) / (T(2) * L.ax + T(2) * L.ay + T(cz) * L.az);
-}
-
-template <typename T>
-__device__ __forceinline__ T mg_inv_int(const MgView<T>& L) {
-  return T(1) / (T(2) * L.ax + T(2) * L.ay + T(2) * L.az);
-}
 
 // A v at a level with per-direction coefficients ax, ay, az = 1/h^2; the z
 // face logic only on the planes next to a z face (bt).
@@ -847,384 +818,6 @@ __global__ void __launch_bounds__(MTX* MTY, (sizeof(T) == 4 && !EPS) ? (INT ? 5 
   }
 }
 
-// ------------------------------------------------------ coarsest-level solve
-
-// Sum over a warp with every lane receiving the total.  The butterfly adds
-// the same two partial sums in every lane of a pair, so all lanes end with
-// bitwise the same value (addition is commutative).
-__device__ __forceinline__ double warp_sum_all(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
-// Barrier of the first nw warps of the block (named barrier 1; one warp:
-// a warp barrier).
-__device__ __forceinline__ void warps_sync(int nw) {
-  if (nw == 1) __syncwarp();
-  else asm volatile("bar.sync 1, %0;\n" ::"r"(nw * 32) : "memory");
-}
-
-// Sum over the first nw warps, the same value in every thread (fixed order).
-__device__ __forceinline__ double warps_sum(double v, int nw, double* red) {
-  v = warp_sum_all(v);
-  if (nw == 1) return v;
-  warps_sync(nw);                  // red[] may still be read from the previous sum
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-  warps_sync(nw);
-  double s = 0.0;
-  for (int i = 0; i < nw; ++i) s += red[i];
-  return s;
-}
-
-// Jacobi-preconditioned conjugate gradients on the coarsest level, FP64, one
-// cell per thread in the first ceil(n / 32) warps of the block (the other
-// warps return at once; the caller's next __syncthreads joins them), to a
-// relative residual of 1e-12.  The diagonal scaling matters where a
-// permittivity field makes the coarse operator's diagonal vary by orders of
-// magnitude.  With no electrode the level is singular: the right-hand side and
-// the solution are projected to zero mean.
-// A coarsest level that is one z column (1 x 1 x nz: the in-plane faces join a
-// cell to itself and drop out) with non-periodic z is tridiagonal: solved
-// directly by the Thomas algorithm (forward elimination, back substitution)
-// in FP64 by one thread, with scratch for 2 nz values.  Jacobi-PCG on such a
-// column (a film whose z axis stops coarsening, as under air layers) needed up
-// to nz iterations of three block reductions each.
-template <typename T>
-__device__ __forceinline__ void coarse_column_solve(const MgView<T>& C, const T* cf, T* ce, double* scratch) {
-  const int n = C.g.nz;
-  const double az = C.az;
-  double* cpr = scratch;                        // c'_z
-  double* dpr = scratch + n;                    // d'_z
-  auto w = [&](int z, int nb) -> double {       // face weight between cells z and nb
-    if (!C.eps) return 1.0;
-    const double ec = (double)C.eps[z], en = (double)C.eps[nb];
-    return 2.0 * ec * en / (ec + en);
-  };
-  double prev_c = 0.0, prev_d = 0.0;
-  for (int z = 0; z < n; ++z) {
-    const double wm = z > 0 ? w(z, z - 1) : 0.0, wp = z < n - 1 ? w(z, z + 1) : 0.0;
-    const double wd = C.eps ? (double)C.eps[z] : 1.0;
-    double diag = az * (wm + wp);
-    if (z == 0 && C.tlo[0]) diag += az * 2.0 * wd;
-    if (z == n - 1 && C.thi[0]) diag += az * 2.0 * wd;
-    const double lower = -az * wm, upper = -az * wp;
-    const double m = diag - lower * prev_c;
-    prev_c = upper / m;
-    prev_d = ((double)cf[z] - lower * prev_d) / m;
-    cpr[z] = prev_c;
-    dpr[z] = prev_d;
-  }
-  double x = 0.0;
-  for (int z = n - 1; z >= 0; --z) {
-    x = dpr[z] - cpr[z] * x;
-    ce[z] = (T)x;
-  }
-}
-
-template <typename T>
-__device__ __forceinline__ void mg_coarse_solve(const MgView<T>& C, const T* cf, T* ce, int singular, double* ps,
-                                                double* red) {
-  if (C.g.nx == 1 && C.g.ny == 1 && !C.g.periodic_z && !singular && 2 * C.g.nz <= MG_MAX_COARSE &&
-      (C.tlo[0] || C.thi[0])) {
-    if (threadIdx.x == 0) coarse_column_solve(C, cf, ce, ps);
-    return;
-  }
-  const int n = (int)C.g.n, tid = threadIdx.x;
-  const int nw = (n + 31) >> 5;
-  if (tid >= nw * 32) return;
-  const bool on = tid < n;
-  int x = 0, y = 0, z = 0;
-  if (on) {
-    x = tid % C.g.nx;
-    y = (tid / C.g.nx) % C.g.ny;
-    z = tid / (int)C.g.nxy;
-  }
-  const int xm = (x == 0 ? C.g.nx - 1 : x - 1) + (tid - x), xp = (x == C.g.nx - 1 ? 0 : x + 1) + (tid - x);
-  const int rowo = z * (int)C.g.nxy;
-  const int ym = rowo + (y == 0 ? C.g.ny - 1 : y - 1) * C.g.nx + x;
-  const int yp = rowo + (y == C.g.ny - 1 ? 0 : y + 1) * C.g.nx + x;
-  const int zb = z > 0 ? z - 1 : (C.g.periodic_z ? C.g.nz - 1 : -1);
-  const int za = z < C.g.nz - 1 ? z + 1 : (C.g.periodic_z ? 0 : -1);
-  const int zm = zb >= 0 ? zb * (int)C.g.nxy + y * C.g.nx + x : -1;
-  const int zp = za >= 0 ? za * (int)C.g.nxy + y * C.g.nx + x : -1;
-  const int xy = y * C.g.nx + x;
-  const double ax = C.ax, ay = C.ay, az = C.az;
-  const int dlo = (on && zb < 0) ? (int)C.tlo[xy] : 0;
-  const int dhi = (on && za < 0) ? (int)C.thi[xy] : 0;
-  // face weights: 1, or the harmonic mean of the cells' eps (electrode: 2 eps_c)
-  double wxm = 1.0, wxp = 1.0, wym = 1.0, wyp = 1.0, wzm = 1.0, wzp = 1.0, wd = 1.0;
-  if (C.eps && on) {
-    const double ec = (double)C.eps[tid];
-    auto hm = [&](int nb) { const double en = (double)C.eps[nb]; return 2.0 * ec * en / (ec + en); };
-    wxm = hm(xm);
-    wxp = hm(xp);
-    wym = hm(ym);
-    wyp = hm(yp);
-    wzm = zm >= 0 ? hm(zm) : 0.0;
-    wzp = zp >= 0 ? hm(zp) : 0.0;
-    wd = ec;
-  }
-  auto apply = [&](const double* v) -> double {
-    const double c = v[tid];
-    double sz = 0.0;
-    if (zm >= 0) sz += wzm * (c - v[zm]);
-    else if (dlo) sz += 2.0 * wd * c;
-    if (zp >= 0) sz += wzp * (c - v[zp]);
-    else if (dhi) sz += 2.0 * wd * c;
-    return ax * (wxm * (c - v[xm]) + wxp * (c - v[xp])) + ay * (wym * (c - v[ym]) + wyp * (c - v[yp])) + az * sz;
-  };
-  double dg = ax * (wxm + wxp) + ay * (wym + wyp);
-  dg += az * ((zm >= 0 ? wzm : (dlo ? 2.0 * wd : 0.0)) + (zp >= 0 ? wzp : (dhi ? 2.0 * wd : 0.0)));
-  const double dinv = (on && dg > 0.0) ? 1.0 / dg : 0.0;
-  double b = on ? (double)cf[tid] : 0.0;
-  if (singular) b -= warps_sum(b, nw, red) / n;
-  double xv = 0.0, r = b;
-  const double bb = warps_sum(r * r, nw, red);
-  if (bb > 0.0) {
-    double zv = r * dinv;
-    double p = zv;
-    double rz = warps_sum(r * zv, nw, red);
-    for (int it = 0; it < 4 * n + 20; ++it) {
-      warps_sync(nw);              // ps[] may still be read from the previous iteration
-      if (on) ps[tid] = p;
-      warps_sync(nw);
-      const double q = on ? apply(ps) : 0.0;
-      const double pq = warps_sum(p * q, nw, red);
-      if (!(pq > 0.0)) break;
-      const double a = rz / pq;
-      xv += a * p;
-      r -= a * q;
-      const double rrn = warps_sum(r * r, nw, red);
-      if (rrn <= 1e-24 * bb) break;
-      zv = r * dinv;
-      const double rzn = warps_sum(r * zv, nw, red);
-      p = zv + (rzn / rz) * p;
-      rz = rzn;
-    }
-  }
-  if (singular) xv -= warps_sum(on ? xv : 0.0, nw, red) / n;
-  if (on) ce[tid] = (T)xv;
-}
-
-template <typename T>
-__global__ void __launch_bounds__(MG_MAX_COARSE) k_mg_coarse(MgView<T> C, int singular, Scalars* S) {
-  __shared__ double ps[MG_MAX_COARSE];
-  __shared__ double red[32];
-  if (S->done) return;
-  mg_coarse_solve(C, C.f, C.e, singular, ps, red);
-}
-
-// ------------------------------------------------------------ the V-cycle tail
-
-// Column walk of a small level: thread t of the block takes the columns t,
-// t + blockDim.x, ... of the nx x ny plane and walks them along z, so the
-// in-plane neighbour offsets, the face masks and the boundary diagonals are
-// formed once per column instead of from the linear index at every cell.
-// When the level has fewer columns than the block has threads (a deep, narrow
-// level such as 8 x 8 x 37), each column is cut into z chunks walked by
-// different threads.  body(o, x, y, z0, z1) walks planes [z0, z1).
-struct TailCol {
-  int xy;                   // the column (y nx + x)
-  int dxm, dxp, dym, dyp;   // offsets of the in-plane neighbours (periodic wrap)
-  int dlo, dhi;             // electrode masks of the column's z faces
-};
-
-// Quotient of small non-negative ints (a < 2^22) by d >= 1 through a float
-// reciprocal formed once per level: the rounded product is at most one off,
-// and one compare on each side corrects it.  The column walks divide by the
-// level's sizes at every item of every phase; an integer division there cost
-// more than the arithmetic of the cell it located.
-struct SmallDiv {
-  int d;
-  float r;
-  __device__ __forceinline__ explicit SmallDiv(int d_) : d(d_), r(1.0f / (float)d_) {}
-  __device__ __forceinline__ int operator()(int a) const {
-    int q = (int)((float)a * r);
-    if (q * d > a) --q;
-    else if ((q + 1) * d <= a) ++q;
-    return q;
-  }
-};
-
-template <typename T, class Body>
-__device__ __forceinline__ void tail_cols(const MgView<T>& L, Body body) {
-  const int nx = L.g.nx, ny = L.g.ny, nxy = (int)L.g.nxy, nz = L.g.nz;
-  const int nch = nxy >= (int)blockDim.x ? 1 : min(nz, (int)blockDim.x / nxy);   // z chunks per column
-  const SmallDiv by_nxy(nxy), by_nch(nch), by_nx(nx);
-  for (int item = threadIdx.x; item < nxy * nch; item += blockDim.x) {
-    const int ch = nch > 1 ? by_nxy(item) : 0, col = item - ch * nxy;
-    const int z0 = nch > 1 ? by_nch(ch * nz) : 0, z1 = nch > 1 ? by_nch((ch + 1) * nz) : nz;
-    const int y = by_nx(col), x = col - y * nx;
-    TailCol o;
-    o.xy = col;
-    o.dxm = x == 0 ? nx - 1 : -1;
-    o.dxp = x == nx - 1 ? -(nx - 1) : 1;
-    o.dym = y == 0 ? (ny - 1) * nx : -nx;
-    o.dyp = y == ny - 1 ? -(ny - 1) * nx : nx;
-    o.dlo = L.g.periodic_z ? 0 : (int)L.tlo[col];
-    o.dhi = L.g.periodic_z ? 0 : (int)L.thi[col];
-    body(o, x, y, z0, z1);
-  }
-}
-
-// 1/diag at plane z of a column (eps = 1); iint: the interior value.
-template <typename T>
-__device__ __forceinline__ T col_inv(const MgView<T>& L, const TailCol& o, int z, T iint) {
-  const int nz = L.g.nz;
-  if (L.g.periodic_z || (z > 0 && z < nz - 1)) return iint;
-  int cz = 2;
-  if (z == 0) cz += 2 * o.dlo - 1;
-  if (z == nz - 1) cz += 2 * o.dhi - 1;
-  return T(1) / (T(2) * L.ax + T(2) * L.ay + T(cz) * L.az);
-}
-
-// (A v) at plane z of a column and 1/diag there: the same operator, face
-// order and diagonal as the sweep kernels (per-direction 1/h^2; with eps the
-// harmonic-mean face weights and the precomputed 1/diag; iint: the interior
-// 1/diag with eps = 1, so only the face planes divide).
-template <typename T>
-__device__ __forceinline__ T col_apply(const MgView<T>& L, const T* v, const TailCol& o, int z, T& inv, T iint) {
-  const int nz = L.g.nz, nxy = (int)L.g.nxy;
-  const int c = z * nxy + o.xy;
-  const T vc = v[c];
-  const int zm = z > 0 ? c - nxy : (L.g.periodic_z ? c + (nz - 1) * nxy : -1);
-  const int zp = z < nz - 1 ? c + nxy : (L.g.periodic_z ? c - (nz - 1) * nxy : -1);
-  if (L.eps) {
-    const T ec = L.eps[c];
-    auto face = [&](int nb) { return hmean2(ec, L.eps[nb]) * (vc - v[nb]); };
-    const T sx = face(c + o.dxm) + face(c + o.dxp);
-    const T sy = face(c + o.dym) + face(c + o.dyp);
-    T sz = T(0);
-    if (zm >= 0) sz += face(zm);
-    else if (o.dlo) sz += T(2) * ec * vc;
-    if (zp >= 0) sz += face(zp);
-    else if (o.dhi) sz += T(2) * ec * vc;
-    inv = L.invd[c];
-    return L.ax * sx + L.ay * sy + L.az * sz;
-  }
-  const T sx = (vc - v[c + o.dxm]) + (vc - v[c + o.dxp]);
-  const T sy = (vc - v[c + o.dym]) + (vc - v[c + o.dyp]);
-  T sz = T(0);
-  if (zm >= 0) sz += vc - v[zm];
-  else if (o.dlo) sz += T(2) * vc;
-  if (zp >= 0) sz += vc - v[zp];
-  else if (o.dhi) sz += T(2) * vc;
-  inv = col_inv(L, o, z, iint);
-  return L.ax * sx + L.ay * sy + L.az * sz;
-}
-
-// The V-cycle below level k0 (all levels small) in one block: per level two
-// pre-smoothing sweeps from zero, the residual, its restriction, the coarsest
-// solve, then prolongation and two post-smoothing sweeps, each phase a walk
-// over the level's columns followed by a block barrier.  Same operators,
-// weights and transfers as the one-kernel-per-phase path above it.  Every
-// level's f, e, e_tmp live in shared memory (t.off[k]: offset of level k's
-// three arrays, in elements); the first level's f comes from and its e goes
-// back to global memory.
-template <typename T>
-__global__ void __launch_bounds__(MG_MAX_COARSE) k_mg_tail(MgTail<T> t, int singular, Scalars* S) {
-  extern __shared__ __align__(16) unsigned char tail_smem[];
-  __shared__ double ps[MG_MAX_COARSE];
-  __shared__ double red[32];
-  if (S->done) return;
-  T* sm = reinterpret_cast<T*>(tail_smem);
-  auto F = [&](int k) { return sm + t.off[k]; };
-  auto E = [&](int k) { return sm + t.off[k] + t.lv[k].g.n; };
-  auto ET = [&](int k) { return sm + t.off[k] + 2 * t.lv[k].g.n; };
-  const T om1 = mg_omega1<T>(), om2 = mg_omega2<T>();
-  const int nt = blockDim.x;
-  {
-    const int n0 = (int)t.lv[0].g.n;
-    T* f0 = F(0);
-    for (int c = threadIdx.x; c < n0; c += nt) f0[c] = t.lv[0].f[c];
-    __syncthreads();
-  }
-  for (int k = 0; k + 1 < t.nl; ++k) {
-    const MgView<T>& L = t.lv[k];
-    const MgView<T>& C = t.lv[k + 1];
-    T *f = F(k), *e = E(k), *et = ET(k);
-    const int nxy = (int)L.g.nxy, nz = L.g.nz;
-    const T iint = mg_inv_int(L);
-    tail_cols(L, [&](const TailCol& o, int, int, int z0, int z1) {
-      for (int z = z0; z < z1; ++z) {
-        const int c = z * nxy + o.xy;
-        const T inv = L.eps ? L.invd[c] : col_inv(L, o, z, iint);
-        et[c] = om1 * inv * f[c];
-      }
-    });
-    __syncthreads();
-    tail_cols(L, [&](const TailCol& o, int, int, int z0, int z1) {
-      for (int z = z0; z < z1; ++z) {
-        T inv;
-        const T Ae = col_apply(L, et, o, z, inv, iint);
-        const int c = z * nxy + o.xy;
-        e[c] = et[c] + om2 * inv * (f[c] - Ae);
-      }
-    });
-    __syncthreads();
-    // the residual (into e_tmp, free again), then the sum of each coarse
-    // cell's children in the order dz, dy, dx
-    tail_cols(L, [&](const TailCol& o, int, int, int z0, int z1) {
-      for (int z = z0; z < z1; ++z) {
-        T inv;
-        const T Ae = col_apply(L, e, o, z, inv, iint);
-        const int c = z * nxy + o.xy;
-        et[c] = f[c] - Ae;
-      }
-    });
-    __syncthreads();
-    const T scale = T(1) / T(L.fx * L.fy * L.fz);
-    T* fc = F(k + 1);
-    const int ncxy = (int)C.g.nxy;
-    tail_cols(C, [&](const TailCol& o, int X, int Y, int z0, int z1) {
-      for (int Z = z0; Z < z1; ++Z) {
-        T acc = T(0);
-        for (int dz = 0; dz < L.fz; ++dz)
-          for (int dy = 0; dy < L.fy; ++dy)
-            for (int dx = 0; dx < L.fx; ++dx)
-              acc += et[((Z * L.fz + dz) * L.g.ny + Y * L.fy + dy) * L.g.nx + X * L.fx + dx];
-        fc[Z * ncxy + o.xy] = acc * scale;
-      }
-    });
-    __syncthreads();
-  }
-  mg_coarse_solve(t.lv[t.nl - 1], F(t.nl - 1), E(t.nl - 1), singular, ps, red);
-  __syncthreads();
-  for (int k = t.nl - 2; k >= 0; --k) {
-    const MgView<T>& L = t.lv[k];
-    const MgView<T>& C = t.lv[k + 1];
-    T *f = F(k), *e = E(k), *et = ET(k);
-    const T* ec = E(k + 1);
-    const int nxy = (int)L.g.nxy, nz = L.g.nz;
-    const T iint = mg_inv_int(L);
-    tail_cols(L, [&](const TailCol& o, int x, int y, int z0, int z1) {
-      const int pxy = (y >> (L.fy - 1)) * C.g.nx + (x >> (L.fx - 1));
-      for (int z = z0; z < z1; ++z) e[z * nxy + o.xy] += ec[(z >> (L.fz - 1)) * (int)C.g.nxy + pxy];
-    });
-    __syncthreads();
-    tail_cols(L, [&](const TailCol& o, int, int, int z0, int z1) {
-      for (int z = z0; z < z1; ++z) {
-        T inv;
-        const T Ae = col_apply(L, e, o, z, inv, iint);
-        const int c = z * nxy + o.xy;
-        et[c] = e[c] + om2 * inv * (f[c] - Ae);
-      }
-    });
-    __syncthreads();
-    T* eo = k == 0 ? t.lv[0].e : e;                    // the first level's result goes to global memory
-    tail_cols(L, [&](const TailCol& o, int, int, int z0, int z1) {
-      for (int z = z0; z < z1; ++z) {
-        T inv;
-        const T Ae = col_apply(L, et, o, z, inv, iint);
-        const int c = z * nxy + o.xy;
-        eo[c] = et[c] + om1 * inv * (f[c] - Ae);
-      }
-    });
-    __syncthreads();
-  }
-}
-
 // ---------------------------------------------------------------- launchers
 
 template <typename K>
@@ -1418,12 +1011,6 @@ int launch_mg_rr(const LaunchCfg& L, const MgView<T>& lv, const MgView<T>& cv, S
 }
 
 template <typename T>
-void launch_mg_coarse(const LaunchCfg& L, const MgView<T>& cv, int singular, Scalars* S) {
-  const int threads = ((int)cv.g.n + 31) / 32 * 32;
-  k_mg_coarse<T><<<1, threads, 0, L.stream>>>(cv, singular, S);
-}
-
-template <typename T>
 int launch_mg_post1(const LaunchCfg& L, const MgView<T>& lv, const MgView<T>& cv, Scalars* S) {
   constexpr int V = vec_of(sizeof(T));
   if (lv.eps) {
@@ -1540,13 +1127,6 @@ void launch_mg_eps_level(const LaunchCfg& L, const MgView<T>& fine, const MgView
   k_mg_invdiag<T><<<g1, 256, 0, L.stream>>>(c, cinvd);
 }
 
-template <typename T>
-void launch_mg_tail(const LaunchCfg& L, const MgTail<T>& t, int singular, Scalars* S) {
-  static bool f = false;
-  smem_once(k_mg_tail<T>, MG_TAIL_SMEM, f);
-  k_mg_tail<T><<<1, MG_MAX_COARSE, (size_t)t.smem_elems * sizeof(T), L.stream>>>(t, singular, S);
-}
-
 #define PF_MG_INSTANTIATE(T)                                                           \
   template int launch_mg_pre<T>(const LaunchCfg&, const MgView<T>&, Scalars*);                   \
   template int launch_mg_rr<T>(const LaunchCfg&, const MgView<T>&, const MgView<T>&, Scalars*);  \
@@ -1555,8 +1135,6 @@ void launch_mg_tail(const LaunchCfg& L, const MgTail<T>& t, int singular, Scalar
   template bool mg_fused_post<T>(const MgView<T>&);                                              \
   template int launch_mg_pp<T>(const LaunchCfg&, const MgView<T>&, const MgView<T>&, T*, T*, double*, Scalars*, \
                                 const std::function<void(int)>&);                                             \
-  template void launch_mg_coarse<T>(const LaunchCfg&, const MgView<T>&, int, Scalars*);          \
-  template void launch_mg_tail<T>(const LaunchCfg&, const MgTail<T>&, int, Scalars*);            \
   template int launch_mg_post1<T>(const LaunchCfg&, const MgView<T>&, const MgView<T>&, Scalars*); \
   template int launch_mg_post2<T>(const LaunchCfg&, const MgView<T>&, int, double*, Scalars*);         \
   template void launch_mg_eps_level<T>(const LaunchCfg&, const MgView<T>&, const MgView<T>&, T*, T*);
