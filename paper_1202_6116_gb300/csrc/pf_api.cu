@@ -302,7 +302,8 @@ struct pf_ctx {
     int fam;
     double bytes;
     int kind;                     // 0 always runs; 1 CG launch of iteration iter_no (1-based);
-                                  // 2 V-cycle number iter_no (0-based) of its solve
+                                  // 2 V-cycle number iter_no (0-based) of its solve;
+                                  // 3 a whole CG loop (bytes per iteration)
     int iter_no;
     int first_bytes_alt;          // 1: cg_p, first iteration moves bytes_first
     double bytes_first;
@@ -337,10 +338,10 @@ namespace {
 
 enum Fam {
   F_RHS_MEAN, F_RHS, F_CG_P, F_CG_R, F_FINISH, F_SUB_MEAN, F_TDGL, F_INVDIAG, F_TDGL_ADJ, F_DIAG, F_EXTRAP,
-  F_MG_PRE, F_MG_RR, F_MG_COARSE, F_MG_POST1, F_MG_POST2, F_MG_PRR, F_MG_PP, F_COUNT
+  F_CG_LOOP, F_MG_PRE, F_MG_RR, F_MG_COARSE, F_MG_POST1, F_MG_POST2, F_MG_PRR, F_MG_PP, F_COUNT
 };
 const char* const FAM_NAMES[F_COUNT] = {"rhs_mean", "rhs",      "cg_p",     "cg_r",     "cg_finish",
-                                        "sub_mean", "tdgl",     "invdiag",  "tdgl_adj", "diag",     "extrap",
+                                        "sub_mean", "tdgl",     "invdiag",  "tdgl_adj", "diag",     "extrap", "cg_loop",
                                         "mg_pre",   "mg_rr",    "mg_bottom", "mg_post1", "mg_post2", "mg_prr",
                                         "mg_pp"};
 constexpr int MG_KINDS = F_COUNT - F_MG_PRE;
@@ -407,7 +408,7 @@ void prof_harvest(pf_ctx* ctx, int executed_iters, int done) {
     }
     st.launches += 1;
     st.total_ms += ms;
-    st.bytes += (r.first_bytes_alt && r.iter_no == 1) ? r.bytes_first : r.bytes;
+    st.bytes += (r.first_bytes_alt && r.iter_no == 1) ? r.bytes_first : r.bytes * (r.kind == 3 ? executed_iters : 1);
   }
   ctx->recs.clear();
   ctx->have_base = false;
@@ -679,6 +680,8 @@ void adjoint_view(pf_ctx* ctx, pf::Dev<T>& d) {
   d.bc.vhi = d.bc.vlo;
 }
 
+bool cg_loop_of(pf_ctx* ctx);
+
 // One Poisson solve for the polarization P (device pointer of the current
 // state): r0, PCG iterations until the device flag says done, final update.
 // adj: solve for the adjoint potential instead (P is then the cotangent).
@@ -708,12 +711,24 @@ pf_status solve(pf_ctx* ctx, const T* P, bool adj = false, bool step_solve = fal
   const int mg = ctx->prm.solver == PF_PCG_MG;
   if (mg) vcycle<T>(ctx, 0);
   PF_CUDA(cudaGetLastError());
+  bool looped = false;
+  if (cg_loop_of(ctx)) {                   // every iteration in one launch
+    before_launch(ctx);
+    looped = pf::launch_cg_loop<T>(ctx->L, g, d, false);
+    PF_CUDA(cudaGetLastError());
+    after_launch(ctx, F_CG_LOOP, 9 * N * w, 3);
+    pf_status st = read_scalars(ctx);
+    if (st != PF_OK) return st;
+    prof_harvest(ctx, ctx->S_host->iter, ctx->S_host->done);
+    if (ctx->S_host->timeout) return ctx->fail(PF_ERR_TIMEOUT, "a wait of the persistent CG loop ran out");
+    if (!ctx->S_host->done) return ctx->fail(PF_ERR_STATE, "internal: the CG loop did not finish");
+  }
   // Every issued iteration either runs or returns at entry once the device
   // flag is set, and the device sets it by iteration maxit at the latest.
   const int maxit = ctx->prm.poisson_maxit;
   int issued = 0;
   int batch = std::max(1, std::min(est_iters, maxit));
-  for (;;) {
+  while (!looped) {
     for (int i = 0; i < batch; ++i) {
       const int it = issued + i + 1;
       before_launch(ctx);
@@ -763,6 +778,13 @@ void drop_graphs(pf_ctx* ctx) {
   ctx->graph_key = -1;
 }
 
+// Does a solve run its Krylov loop as one persistent launch?
+bool cg_loop_of(pf_ctx* ctx) {
+  if (ctx->prm.solver != PF_PCG_JACOBI || ctx->prm.has_eps) return false;
+  return ctx->prm.precision == PF_FP32 ? pf::launch_cg_loop<float>(ctx->L, ctx->geo, pf::Dev<float>{}, true)
+                                       : pf::launch_cg_loop<double>(ctx->L, ctx->geo, pf::Dev<double>{}, true);
+}
+
 // Does step ctx->nstep solve the potential (poisson_every, Section Numerical
 // Performance)?
 bool refresh_step(const pf_ctx* ctx) {
@@ -784,15 +806,16 @@ int64_t vcycle_kernels(const pf_ctx* ctx) {
   return n;
 }
 
-void step_kernel_counts(const pf_ctx* ctx, int refresh, int64_t* fixed, int64_t* per_iter) {
+void step_kernel_counts(pf_ctx* ctx, int refresh, int64_t* fixed, int64_t* per_iter) {
   const int64_t vc = ctx->prm.solver == PF_PCG_MG ? vcycle_kernels(ctx) : 0;
   const bool heun = ctx->prm.integrator == PF_HEUN;
   const int64_t per_solve = (ctx->singular ? 2 : 0) + 2 + vc + (plain_extrap(ctx) ? 1 : 0);
-  *per_iter = 2 + vc;
+  const bool loop = cg_loop_of(ctx);
+  *per_iter = loop ? 0 : 2 + vc;
   // graph-captured multigrid solves run their first iteration (compensated
   // ones their first two) outside the loop
   const int64_t peeled = vc ? *per_iter * (peel_second(ctx) ? 2 : 1) : 0;
-  *fixed = (refresh ? (heun ? 2 : 1) * (per_solve + peeled) : 0) + (heun ? 2 : 1);
+  *fixed = (refresh ? (heun ? 2 : 1) * (per_solve + peeled + (loop ? 1 : 0)) : 0) + (heun ? 2 : 1);
 }
 
 // Append one whole time step of film ctx, reading P from buffer cur, to
@@ -839,12 +862,19 @@ cudaError_t append_step(pf_ctx* ctx, cudaGraph_t graph, std::vector<cudaGraphNod
   if (compensated(ctx)) comp_view<T>(ctx, ds);
   auto solve_nodes = [&](const T* P) {
     const pf::Dev<T>& d = ds;
+    const bool loop = cg_loop_of(ctx);     // then no conditional node either
     cudaGraphConditionalHandle h = 0;
-    if (e == cudaSuccess) e = cudaGraphConditionalHandleCreate(&h, graph, 1, cudaGraphCondAssignDefault);
+    if (e == cudaSuccess && !loop) e = cudaGraphConditionalHandleCreate(&h, graph, 1, cudaGraphCondAssignDefault);
+    bool looped = false;
     segment([&] {
       if (plain_extrap(ctx)) launch_extrap_of<T>(ctx, ctx->L);
       if (ctx->singular) pf::launch_rhs_mean<T>(ctx->L, g, d, P);
-      pf::launch_rhs<T>(ctx->L, g, d, P, h, 1);
+      pf::launch_rhs<T>(ctx->L, g, d, P, h, loop ? 0 : 1);
+      if (loop) {
+        looped = pf::launch_cg_loop<T>(ctx->L, g, d, false);
+        pf::launch_cg_finish<T>(ctx->L, g, d, ctx->singular);
+        if (ctx->singular) pf::launch_sub_mean<T>(ctx->L, g, d);
+      }
       if (mg) {                  // the first iteration (p = z) runs outside the loop
         vcycle<T>(ctx, 0);
         pf::launch_cg_p<T>(ctx->L, g, d, mg, 1);
@@ -857,7 +887,8 @@ cudaError_t append_step(pf_ctx* ctx, cudaGraph_t graph, std::vector<cudaGraphNod
         }
       }
     });
-    if (e != cudaSuccess) return;
+    if (e == cudaSuccess && loop && !looped) e = cudaErrorNotSupported;
+    if (e != cudaSuccess || loop) return;
     cudaGraphNode_t cnode = nullptr;
     cudaGraphNodeParams cp{};
     cp.type = cudaGraphNodeTypeConditional;
@@ -1186,7 +1217,8 @@ pf_status finish_info(pf_ctx* ctx, int nsteps, pf_step_info* info) {
   prof_harvest(ctx, 0, 1);
   const Scalars& s = *ctx->S_host;
   pf_status result = PF_OK;
-  if (s.nonfinite) result = ctx->fail(PF_ERR_NONFINITE, "non-finite value in the Poisson solver scalars");
+  if (s.timeout) result = ctx->fail(PF_ERR_TIMEOUT, "a wait of the persistent CG loop ran out");
+  else if (s.nonfinite) result = ctx->fail(PF_ERR_NONFINITE, "non-finite value in the Poisson solver scalars");
   else if (s.nonconv) result = ctx->fail(PF_ERR_NOCONV, "%d Poisson solve(s) hit poisson_maxit", s.nonconv);
   if (info) {
     info->steps_done = nsteps;
@@ -2003,7 +2035,8 @@ pf_status pf_batch_step(pf_batch* b, int32_t nsteps, pf_step_info* info) {
     pf_step_info& fi = b->infos[i];
     fi = pf_step_info{};
     const pf_status st = finish_info(c, nsteps, &fi);
-    if (st == PF_ERR_CUDA || st == PF_ERR_STATE) return b->fail(st, "film %d: %s", i, c->err.c_str());
+    if (st == PF_ERR_CUDA || st == PF_ERR_STATE || st == PF_ERR_TIMEOUT)
+      return b->fail(st, "film %d: %s", i, c->err.c_str());
     if (st == PF_ERR_NONFINITE || (st == PF_ERR_NOCONV && worst == PF_OK)) worst = st;
     sum.last_iters = std::max(sum.last_iters, fi.last_iters);
     sum.total_iters += fi.total_iters;

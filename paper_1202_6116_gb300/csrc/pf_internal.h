@@ -141,6 +141,11 @@ void launch_cg_p(const LaunchCfg& L, const Geo& g, const Dev<T>& d, int mg, int 
 template <typename T>
 void launch_cg_r(const LaunchCfg& L, const Geo& g, const Dev<T>& d, int mg, cudaGraphConditionalHandle cond,
                  int use_cond);
+// The whole Jacobi-PCG loop as one launch (pf_cgloop.cu).  Returns false, with
+// nothing launched, when the grid does not qualify or the launch is not
+// possible here; dry: only whether it is.
+template <typename T>
+bool launch_cg_loop(const LaunchCfg& L, const Geo& g, const Dev<T>& d, bool dry);
 template <typename T>
 void launch_cg_finish(const LaunchCfg& L, const Geo& g, const Dev<T>& d, int singular);
 template <typename T>

@@ -157,8 +157,17 @@ pf_status solve(const pf_params* prm, cudaStream_t st, char* base, const Layout&
   pf::launch_rhs<T>(L, g, d, P, 0, 0);
   if (launched("rhs") != PF_OK) return PF_ERR_CUDA;
   pf::Scalars host;
+  const bool loop = pf::launch_cg_loop<T>(L, g, d, true);
+  if (loop) {                              // every iteration in one launch
+    pf::launch_cg_loop<T>(L, g, d, false);
+    if (launched("cg_loop") != PF_OK) return PF_ERR_CUDA;
+    launches += 1;
+    NA_CUDA(cudaMemcpyAsync(&host, d.S, sizeof(host), cudaMemcpyDeviceToHost, st));
+    NA_CUDA(cudaStreamSynchronize(st));
+    if (host.timeout) return fail(PF_ERR_TIMEOUT, "a wait of the persistent CG loop ran out");
+  }
   int issued = 0, batch = std::min(16, prm->poisson_maxit);
-  for (;;) {
+  while (!loop) {
     for (int i = 0; i < batch; ++i) {
       pf::launch_cg_p<T>(L, g, d, 0);
       if (launched("cg_p") != PF_OK) return PF_ERR_CUDA;

@@ -84,6 +84,7 @@ __device__ __forceinline__ void rhs_close(const Geo& g, double* part, Scalars* S
   S->bnorm = sqrt(bb);
   S->rr = rr;
   S->rz = rz;
+  S->bar = 0u;
   S->iter = 0;
   S->first = 1;
   S->pending = 0;

@@ -1,0 +1,97 @@
+"""The V-cycle's small levels as one launch (levels spread over a cluster,
+levels in one block, the product with the coarsest level's inverse) and the
+persistent Jacobi-PCG loop, at the sizes where each of their branches begins:
+potentials against the FP64 oracle, FP64 bar 1e-10 as in the parity tests."""
+import numpy as np
+import pytest
+import torch
+
+import oracle as O
+from paper_1202_6116_gb300 import build as B
+from paper_1202_6116_gb300 import pf
+from paper_1202_6116_gb300.film import Film
+
+from helpers import mixed_workload, oracle_grid, relerr
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    B.build()
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    pf.lib()
+
+
+def solve(w, **over):
+    f = Film(w, **over)
+    st, info = f.solve_potential()
+    phi = f.numpy()[1]
+    f.close()
+    assert st == pf.PF_OK
+    return phi, info
+
+
+@pytest.mark.parametrize("shape,eps,faces", [
+    ((16, 16, 1), False, "mixed"),      # one block runs every level; coarsest 1 cell
+    ((16, 8, 8), True, "mixed"),        # the finest level spread over the cluster (FP64), with eps
+    ((24, 20, 12), False, "mixed"),     # coarsest 3 x 5 x 3: a row per thread
+    ((16, 16, 16), False, "periodic"),  # singular: constant vector taken out of the inverse
+    ((36, 20, 9), True, "mixed"),       # coarsest 9 x 5 x 9 = 405: a row per warp over the cluster
+    ((42, 36, 8), False, "open"),       # coarsest 21 x 9 x 1, singular, rows of no whole vectors
+    ((64, 34, 8), False, "mixed"),      # 17 x 1 coarse rows, levels above the launch
+    ((8, 8, 37), True, "mixed"),        # a z column is left: 1 x 1 x 37
+])
+def test_small_levels_match_oracle_fp64(shape, eps, faces):
+    w = mixed_workload(*shape, 61, eps=eps).with_(solver="mg", maxit=300, rtol=1e-13)
+    if faces != "mixed":
+        z8 = np.zeros_like(w.type_lo)
+        w = w.with_(type_lo=z8, type_hi=z8, periodic_z=faces == "periodic")
+    phio, st, _, _ = O.solve_potential(oracle_grid(w), w.P0, rtol=1e-14)
+    assert st == O.OK
+    phi, info = solve(w)
+    assert relerr(phi, phio) <= 1e-10
+    assert info["last_iters"] <= 60
+
+
+def test_new_electrode_layout_renews_the_inverse():
+    """A second layout on the same context: the solve must use its own coarsest operator."""
+    w = mixed_workload(36, 20, 9, 62).with_(solver="mg", maxit=300, rtol=1e-13)
+    w2 = mixed_workload(36, 20, 9, 63, tol_dirichlet=0.1).with_(solver="mg", maxit=300, rtol=1e-13)
+    f = Film(w)
+    f.solve_potential()
+    f.set_bc(pf.PF_ZLO, w2.type_lo, w2.volt_lo)
+    f.set_bc(pf.PF_ZHI, w2.type_hi, w2.volt_hi)
+    f.phi.zero_()
+    _, info = f.solve_potential()
+    phi = f.numpy()[1]
+    f.close()
+    phio, st, _, _ = O.solve_potential(oracle_grid(w2.with_(P0=w.P0)), w.P0, rtol=1e-14)
+    assert st == O.OK and relerr(phi, phio) <= 1e-10
+    fresh, info2 = solve(w2.with_(P0=w.P0))
+    assert info["last_iters"] == info2["last_iters"]
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("shape,faces", [
+    ((1, 1, 1), "mixed"), ((5, 3, 2), "mixed"), ((17, 33, 3), "mixed"),   # a thread per cell, ragged tiles
+    ((32, 32, 32), "mixed"), ((24, 16, 12), "periodic"), ((24, 16, 12), "open"),
+    ((160, 64, 32), "mixed"),                                             # 16-byte vectors (FP32: 4 cells)
+    ((164, 100, 41), "mixed"),                                            # vectors on ragged tiles, several per thread
+])
+def test_cg_loop_matches_the_two_kernel_iteration(precision, shape, faces):
+    """The persistent loop against the same solve with a permittivity field of
+    ones, which iterates with one launch per half step: same operator, same
+    iteration, sums in another order.  FP64 within 1e-10 of the largest
+    potential, FP32 within the solve tolerance times the grid's conditioning
+    (1e-4, as in the parity tests)."""
+    w = mixed_workload(*shape, 64, precision=precision, rtol=1e-13 if precision == "fp64" else 1e-7)
+    if faces != "mixed":
+        z8 = np.zeros_like(w.type_lo)
+        w = w.with_(type_lo=z8, type_hi=z8, periodic_z=faces == "periodic")
+    phi, info = solve(w)
+    ref, info_ref = solve(w.with_(eps=np.ones(w.shape)))
+    assert relerr(phi, ref) <= (1e-10 if precision == "fp64" else 1e-4)
+    assert abs(info["last_iters"] - info_ref["last_iters"]) <= max(2, info_ref["last_iters"] // 50)
+    # the whole loop is one launch
+    assert info["kernel_launches"] <= 5 < info_ref["kernel_launches"] or shape == (1, 1, 1)
