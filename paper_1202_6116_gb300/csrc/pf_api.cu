@@ -709,7 +709,6 @@ pf_status solve(pf_ctx* ctx, const T* P, bool adj = false, bool step_solve = fal
   pf::launch_rhs<T>(ctx->L, g, d, P, 0, 0);
   after_launch(ctx, F_RHS, (5 + 2 * e + (comp ? 1 : 0)) * N * w);
   const int mg = ctx->prm.solver == PF_PCG_MG;
-  if (mg) vcycle<T>(ctx, 0);
   PF_CUDA(cudaGetLastError());
   bool looped = false;
   if (cg_loop_of(ctx)) {                   // every iteration in one launch
@@ -731,6 +730,7 @@ pf_status solve(pf_ctx* ctx, const T* P, bool adj = false, bool step_solve = fal
   while (!looped) {
     for (int i = 0; i < batch; ++i) {
       const int it = issued + i + 1;
+      if (mg) vcycle<T>(ctx, it - 1);
       before_launch(ctx);
       pf::launch_cg_p<T>(ctx->L, g, d, mg, it == 1, comp && mg && e == 0.0 && it == 2);
       // the multigrid first iteration stages z alone (p = z), except with eps
@@ -739,7 +739,6 @@ pf_status solve(pf_ctx* ctx, const T* P, bool adj = false, bool step_solve = fal
       after_launch(ctx, F_CG_P, cgp, 1, it, (mg && e == 0.0) ? 3 * N * w : (6 + 2 * e) * N * w);
       pf::launch_cg_r<T>(ctx->L, g, d, mg, 0, 0);
       after_launch(ctx, F_CG_R, (3 + e) * N * w, 1, it);
-      if (mg) vcycle<T>(ctx, it);
     }
     issued += batch;
     PF_CUDA(cudaGetLastError());
@@ -809,7 +808,7 @@ int64_t vcycle_kernels(const pf_ctx* ctx) {
 void step_kernel_counts(pf_ctx* ctx, int refresh, int64_t* fixed, int64_t* per_iter) {
   const int64_t vc = ctx->prm.solver == PF_PCG_MG ? vcycle_kernels(ctx) : 0;
   const bool heun = ctx->prm.integrator == PF_HEUN;
-  const int64_t per_solve = (ctx->singular ? 2 : 0) + 2 + vc + (plain_extrap(ctx) ? 1 : 0);
+  const int64_t per_solve = (ctx->singular ? 2 : 0) + 2 + (plain_extrap(ctx) ? 1 : 0);
   const bool loop = cg_loop_of(ctx);
   *per_iter = loop ? 0 : 2 + vc;
   // graph-captured multigrid solves run their first iteration (compensated
@@ -821,9 +820,12 @@ void step_kernel_counts(pf_ctx* ctx, int refresh, int64_t* fixed, int64_t* per_i
 // Append one whole time step of film ctx, reading P from buffer cur, to
 // graph after the nodes deps (empty: a root); on return deps holds the
 // step's last node.  With refresh = 1 the potential is solved:
-//   solve(P)   [b mean] r0 = b - A phi (+ first V-cycle); while { CG
-//              iteration (+ V-cycle) } with the condition set by the kernels;
-//              last x update [mean removal]
+//   solve(P)   [b mean] r0 = b - A phi; while { (V-cycle +) CG iteration }
+//              with the condition set by the kernels; last x update [mean
+//              removal].  Every iteration begins with its own V-cycle, so a
+//              solve that has converged launches none after its last one (a
+//              V-cycle at the end of the iteration ran as launches that
+//              return at once, 1.1 to 1.5 of them a step).
 //   Euler      solve(P_n); TDGL update into buffer cur ^ 1
 //   Heun       solve(P_n); predictor into buffer cur ^ 1; solve(P^p);
 //              corrector back into buffer cur
@@ -879,11 +881,10 @@ cudaError_t append_step(pf_ctx* ctx, cudaGraph_t graph, std::vector<cudaGraphNod
         vcycle<T>(ctx, 0);
         pf::launch_cg_p<T>(ctx->L, g, d, mg, 1);
         pf::launch_cg_r<T>(ctx->L, g, d, mg, h, 1);
-        vcycle<T>(ctx, 1);
         if (peel_second(ctx)) {  // and so does the second (x still 0, not read)
+          vcycle<T>(ctx, 1);
           pf::launch_cg_p<T>(ctx->L, g, d, mg, 0, 1);
           pf::launch_cg_r<T>(ctx->L, g, d, mg, h, 1);
-          vcycle<T>(ctx, 2);
         }
       }
     });
@@ -900,9 +901,9 @@ cudaError_t append_step(pf_ctx* ctx, cudaGraph_t graph, std::vector<cudaGraphNod
     cudaGraph_t body = cp.conditional.phGraph_out[0];
     e = cudaStreamBeginCaptureToGraph(st, body, nullptr, nullptr, 0, mode);
     if (e != cudaSuccess) return;
+    if (mg) vcycle<T>(ctx, 1);
     pf::launch_cg_p<T>(ctx->L, g, d, mg);
     pf::launch_cg_r<T>(ctx->L, g, d, mg, h, 1);
-    if (mg) vcycle<T>(ctx, 1);
     e = cudaStreamEndCapture(st, &body);
     deps.assign(1, cnode);
     segment([&] {
