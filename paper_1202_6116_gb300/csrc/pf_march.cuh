@@ -654,17 +654,18 @@ __device__ __forceinline__ Stencil7<T> pick(const Stencil7<Raw<T, NH>>& s, int k
 
 // (A v)_c for eps = 1 with homogeneous boundary data: faces summed in the
 // order x-, x+, y-, y+, z-, z+; a boundary face adds 2 v_c at an electrode
-// and nothing at an open surface.
+// and nothing at an open surface.  The plus faces enter as - (v_+ - v_c), the
+// same number as + (v_c - v_+): the difference across the face between two
+// cells of a vector is then one expression for both, formed once.
 template <typename T>
 __device__ __forceinline__ T apply_field(const Stencil7<T>& s, int dlo, int dhi, T ih2) {
-  T acc = T(0);
-  acc += s.c - s.xm;
-  acc += s.c - s.xp;
+  T acc = s.c - s.xm;
+  acc -= s.xp - s.c;
   acc += s.c - s.ym;
-  acc += s.c - s.yp;
+  acc -= s.yp - s.c;
   if (s.zb >= 0) acc += s.c - s.zm;
   else if (dlo) acc += T(2) * s.c;
-  if (s.za >= 0) acc += s.c - s.zp;
+  if (s.za >= 0) acc -= s.zp - s.c;
   else if (dhi) acc += T(2) * s.c;
   return acc * ih2;
 }
@@ -684,22 +685,23 @@ __device__ __forceinline__ T field_value(T f) { return f; }
 template <typename T>
 __device__ __forceinline__ T field_value(const EpsVal<T>& f) { return f.v; }
 
+// Harmonic mean, symmetric in a and b as written, so that a face between two
+// cells of a vector costs one division.
 template <typename T>
 __device__ __forceinline__ T hmean2(T a, T b) {
-  return T(2) * a * b / (a + b);
+  return T(2) * (a * b) / (a + b);
 }
 
 template <typename T>
 __device__ __forceinline__ T apply_field(const Stencil7<EpsVal<T>>& s, int dlo, int dhi, T ih2) {
   const T ec = s.c.e, vc = s.c.v;
-  T acc = T(0);
-  acc += hmean2(ec, s.xm.e) * (vc - s.xm.v);
-  acc += hmean2(ec, s.xp.e) * (vc - s.xp.v);
+  T acc = hmean2(ec, s.xm.e) * (vc - s.xm.v);
+  acc -= hmean2(ec, s.xp.e) * (s.xp.v - vc);
   acc += hmean2(ec, s.ym.e) * (vc - s.ym.v);
-  acc += hmean2(ec, s.yp.e) * (vc - s.yp.v);
+  acc -= hmean2(ec, s.yp.e) * (s.yp.v - vc);
   if (s.zb >= 0) acc += hmean2(ec, s.zm.e) * (vc - s.zm.v);
   else if (dlo) acc += T(2) * ec * vc;
-  if (s.za >= 0) acc += hmean2(ec, s.zp.e) * (vc - s.zp.v);
+  if (s.za >= 0) acc -= hmean2(ec, s.zp.e) * (s.zp.v - vc);
   else if (dhi) acc += T(2) * ec * vc;
   return acc * ih2;
 }

@@ -146,7 +146,13 @@ __global__ void __launch_bounds__(MTX* MTY) k_rhs(Geo g, Bc<T> bc, const T* __re
     T dir = T(0);
     if (dlo) dir += T(2) * ec * bc.vlo[xy];
     if (dhi) dir += T(2) * ec * bc.vhi[xy];
-    const T b = -divergence(st, dlo, dhi) * ih + dir * ih2 - mb;
+    T b;
+    if constexpr (sizeof(T) == 8) {                      // fewer FP64 operations: the factors folded
+      if (!B) b = fma(T(-0.5) * ih, (st.xp.v[0] - st.xm.v[0]) + (st.yp.v[1] - st.ym.v[1]) + (st.zp.v[2] - st.zm.v[2]), -mb);
+      else b = -divergence(st, dlo, dhi) * ih + dir * ih2 - mb;
+    } else {
+      b = -divergence(st, dlo, dhi) * ih + dir * ih2 - mb;
+    }
     if (MEAN) {
       abb.add(b, T(1));
       return T(0);
@@ -428,9 +434,12 @@ __global__ void __launch_bounds__(MTX* MTY, RW_D == 1 ? 3 : 2) k_rhs_w(Geo g, Bc
   rhs_close<3, false, true>(g, part, S, mc.ntiles, cond, use_cond, smem);
 }
 
+// Coefficients of an increment dt L (-df/dP + g Lap P + E), with dt L and the
+// grid factors folded in (formed in FP64, rounded once):
+//   P_i (c1 + c12 (P_x^2 + P_y^2 + P_z^2) + cd P_i^2) + gl (neighbour differences) + el (phi difference).
 template <typename T>
 struct Coef {
-  T c1, c11, c12, g, dtL;        // c1 = 2 a1, c11 = 4 a11, c12 = 2 a12 (exact scalings)
+  T c1, c12, cd, gl, el;         // -2 a1, -2 a12, -(4 a11 - 2 a12), g/dx^2, -1/(2 dx), each times dt L
   T amp;                         // thermal random force: sigma sqrt(dt) (0: off)
   unsigned long long seed;
   long long* step;               // device step counter (steps since pf_bind)
@@ -500,36 +509,53 @@ __device__ __forceinline__ void two_sum(T a, T b, T& s, T& e) {
 }
 
 // dt L (-df/dP + g Lap P + E) at one cell from its stencil (P in v[0..2], phi
-// in v[3]); zb / za < 0 mark a z face (Neumann P, the face value of phi).
+// in v[3]); zb / za < 0 mark a z face (Neumann P, the face value of phi: mean
+// inside, V at an electrode, phi_cell at an open face, so that the difference
+// of the two face values is formed doubled, 2 V or 2 phi_cell at a face).
+// 52 operations a cell in FP32 where the terms written out took 84: FP32 is
+// bound by issue, FP64 by its unit.  The FP32 Laplacian sums differences (they
+// are nearly exact, and the compensated state keeps what they resolve; a
+// difference between two cells of a vector serves both); the FP64 one takes
+// the neighbour sum less 6 P, whose rounding is 0.03 of that of the updated P.
 template <typename T>
 __device__ __forceinline__ void tdgl_inc(const Stencil7<Raw<T, 4>>& st, int xy, int z, const Geo& g,
                                          const Bc<T>& bc, const Coef<T>& k, T (&inc)[3]) {
-  const T h = T(0.5), ih = T(g.ih), ih2 = T(g.ih2);
-  // E = -grad phi from face values (mean inside, V at an electrode, phi_cell at an open face)
   const T fc = st.c.v[3];
-  T E[3];
-  E[0] = -(h * (st.xp.v[3] - st.xm.v[3])) * ih;      // the face values' phi_c cancels
-  E[1] = -(h * (st.yp.v[3] - st.ym.v[3])) * ih;
-  T flo, fhi;
-  if (st.zb >= 0) flo = h * (fc + st.zm.v[3]);
-  else flo = bc.tlo[xy] ? bc.vlo[xy] : fc;
-  if (st.za >= 0) fhi = h * (fc + st.zp.v[3]);
-  else fhi = bc.thi[xy] ? bc.vhi[xy] : fc;
-  E[2] = -(fhi - flo) * ih;
+  T dphi[3];
+  dphi[0] = st.xp.v[3] - st.xm.v[3];                 // the face values' phi_c cancels
+  dphi[1] = st.yp.v[3] - st.ym.v[3];
+  if (st.zb >= 0 && st.za >= 0) {
+    dphi[2] = st.zp.v[3] - st.zm.v[3];
+  } else {
+    const T flo = st.zb >= 0 ? fc + st.zm.v[3] : T(2) * (bc.tlo[xy] ? bc.vlo[xy] : fc);
+    const T fhi = st.za >= 0 ? fc + st.zp.v[3] : T(2) * (bc.thi[xy] ? bc.vhi[xy] : fc);
+    dphi[2] = fhi - flo;
+  }
+  const bool lo = st.zb >= 0, hi = st.za >= 0 && (z + 1 < g.zair || g.zair == g.nz);   // free surface under air
   const T p[3] = {st.c.v[0], st.c.v[1], st.c.v[2]};
+  const T p2[3] = {p[0] * p[0], p[1] * p[1], p[2] * p[2]};
+  const T a = k.c1 + k.c12 * (p2[0] + p2[1] + p2[2]);
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
-    const int j = (i + 1) % 3, l = (i + 2) % 3;
-    const T hi = k.c1 * p[i] + k.c11 * p[i] * p[i] * p[i] + k.c12 * p[i] * (p[j] * p[j] + p[l] * p[l]);
-    T lap = T(0);
-    lap += st.xm.v[i] - p[i];
-    lap += st.xp.v[i] - p[i];
-    lap += st.ym.v[i] - p[i];
-    lap += st.yp.v[i] - p[i];
-    if (st.zb >= 0) lap += st.zm.v[i] - p[i];
-    if (st.za >= 0 && (z + 1 < g.zair || g.zair == g.nz)) lap += st.zp.v[i] - p[i];   // free surface under air
-    lap *= ih2;
-    inc[i] = k.dtL * (-hi + k.g * lap + E[i]);
+    T lap;
+    if constexpr (sizeof(T) == 8) {
+      lap = (st.xm.v[i] + st.xp.v[i]) + (st.ym.v[i] + st.yp.v[i]);
+      if (lo && hi) {
+        lap = fma(T(-6), p[i], lap + (st.zm.v[i] + st.zp.v[i]));
+      } else {
+        lap = fma(T(-4), p[i], lap);
+        if (lo) lap += st.zm.v[i] - p[i];
+        if (hi) lap += st.zp.v[i] - p[i];
+      }
+    } else {
+      lap = st.xp.v[i] - p[i];
+      lap -= p[i] - st.xm.v[i];
+      lap += st.yp.v[i] - p[i];
+      lap -= p[i] - st.ym.v[i];
+      if (lo) lap += st.zm.v[i] - p[i];
+      if (hi) lap += st.zp.v[i] - p[i];
+    }
+    inc[i] = p[i] * (a + k.cd * p2[i]) + (k.gl * lap + k.el * dphi[i]);
   }
 }
 
@@ -963,8 +989,16 @@ static void tdgl_v(const LaunchCfg& L, const Geo& g, const Dev<T>& d, const T* P
 template <typename T>
 void launch_tdgl(const LaunchCfg& L, const Geo& g, const Dev<T>& d, const T* P, T* Pn, const double* coef,
                  int corr, const Noise& nz) {
-  Coef<T> k{T(2) * T(coef[0]), T(4) * T(coef[1]), T(2) * T(coef[2]), T(coef[3]), T(coef[4]), T(nz.amp), nz.seed,
-            nz.step, nz.advance};
+  const double dtL = coef[4];
+  const Coef<T> k{T(-2.0 * coef[0] * dtL),
+                  T(-2.0 * coef[2] * dtL),
+                  T((2.0 * coef[2] - 4.0 * coef[1]) * dtL),
+                  T(coef[3] * g.ih2 * dtL),
+                  T(-0.5 * g.ih * dtL),
+                  T(nz.amp),
+                  nz.seed,
+                  nz.step,
+                  nz.advance};
   const bool noise = nz.amp != 0.0;
   if (corr) {
     if (noise) tdgl_v<T, true, true>(L, g, d, P, Pn, k);
