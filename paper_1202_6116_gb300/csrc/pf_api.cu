@@ -733,10 +733,11 @@ pf_status solve(pf_ctx* ctx, const T* P, bool adj = false, bool step_solve = fal
       if (mg) vcycle<T>(ctx, it - 1);
       before_launch(ctx);
       pf::launch_cg_p<T>(ctx->L, g, d, mg, it == 1, comp && mg && e == 0.0 && it == 2);
-      // the multigrid first iteration stages z alone (p = z), except with eps
-      // the second iteration of a compensated multigrid solve reads no x (still 0)
-      const double cgp = (comp && mg && e == 0.0 && it == 2 ? 5 : 6 + 2 * e) * N * w;
-      after_launch(ctx, F_CG_P, cgp, 1, it, (mg && e == 0.0) ? 3 * N * w : (6 + 2 * e) * N * w);
+      // the multigrid first iteration stages z (and eps) alone (p = z); the
+      // second one of a compensated multigrid solve reads no x (still 0)
+      const double ce = mg ? e : 2 * e;
+      const double cgp = (comp && mg && e == 0.0 && it == 2 ? 5 : 6 + ce) * N * w;
+      after_launch(ctx, F_CG_P, cgp, 1, it, (mg ? 3 + e : 6 + ce) * N * w);
       pf::launch_cg_r<T>(ctx->L, g, d, mg, 0, 0);
       after_launch(ctx, F_CG_R, (3 + e) * N * w, 1, it);
     }

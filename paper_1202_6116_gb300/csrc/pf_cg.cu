@@ -21,11 +21,13 @@ using CgPipe = Pipe<T, typename FieldOf<T, EPS>::type, MTX, MTY, VX, EPS ? 4 : 2
 
 // MG = false: z = r/diag (Jacobi), r is the staged input.  MG = true: z comes
 // from the V-cycle and is the staged input.
-// DIRECT (multigrid, eps = 1): the stencil of p = z + beta p_old is formed
-// from the staged planes of z and p_old at each of the seven cells (no field
-// buffer); otherwise p goes through the march's shared field buffer.
+// DIRECT (multigrid): the stencil of p = z + beta p_old is formed from the
+// staged planes of z and p_old at each of the seven cells (no field buffer);
+// otherwise p goes through the march's shared field buffer.  With a
+// permittivity field eps is staged beside them, and 1/diag, which only the
+// Jacobi z = r/diag needs, is not: two blocks per SM instead of one.
 // FIRST (direct form, launched for a solve's first iteration only): p = z,
-// and neither p_old nor x is read (1 word read, 2 written per cell).
+// and neither p_old nor x is read (1 word read, 2 written per cell; eps 1 more).
 // SECOND (direct form, launched for a compensated solve's second iteration
 // only): the correction x is still 0, so the deferred update writes alpha
 // p_old without staging or reading x (2 words read, 3 written per cell).
@@ -37,7 +39,7 @@ __global__ void __launch_bounds__(MTX* MTY, (sizeof(T) == 4 && !EPS) ? 3 : 2) k_
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ long long tile_slot;
   using F = typename FieldOf<T, EPS>::type;
-  constexpr int NH = EPS ? 4 : 2;          // r or z, p_old (, eps, 1/diag) with halo
+  constexpr int NH = EPS ? (DIRECT ? 3 : 4) : 2;   // r or z, p_old (, eps (, 1/diag)) with halo
   static_assert(!FIRST || DIRECT, "the first-iteration form is the direct one");
   static_assert(!SECOND || (DIRECT && !FIRST), "the second-iteration form is the direct one");
   if (S->done) return;
@@ -56,10 +58,8 @@ __global__ void __launch_bounds__(MTX* MTY, (sizeof(T) == 4 && !EPS) ? 3 : 2) k_
   const T* hsrc[NH];
   hsrc[0] = r;
   hsrc[1] = pold;
-  if constexpr (EPS) {
-    hsrc[2] = eps;
-    hsrc[3] = invd;
-  }
+  if constexpr (EPS) hsrc[2] = eps;
+  if constexpr (EPS && !DIRECT) hsrc[3] = invd;
   const T* osrc[1] = {x};
   struct Out {
     T x, p, q;
@@ -72,7 +72,7 @@ __global__ void __launch_bounds__(MTX* MTY, (sizeof(T) == 4 && !EPS) ? 3 : 2) k_
       zz = h[0];
     } else {
       T inv;
-      if constexpr (EPS) inv = h[3];
+      if constexpr (EPS) inv = h[NH - 1];
       else inv = bt ? inv_diag_unit(g, bc, xy, z, inv6) : inv6;
       zz = h[0] * inv;
     }
@@ -103,10 +103,15 @@ __global__ void __launch_bounds__(MTX* MTY, (sizeof(T) == 4 && !EPS) ? 3 : 2) k_
     store_n<T, VX>(pnew + c, ps);
     store_n<T, VX>(q + c, qs);
   };
-  // direct form: p at a cell from the raw (z, p_old) pair
-  auto pval = [&](const Raw<T, NH>& rw) -> T { return first ? rw.v[0] : rw.v[0] + beta * rw.v[1]; };
-  auto emit_d = [&](int xy, int, const Stencil7<Raw<T, NH>>& sr, const T (&o)[1], const bool bt) -> Out {
-    Stencil7<T> st;
+  // direct form: p at a cell from the raw (z, p_old) pair (FIRST: z alone), as
+  // the stencil field with eps when there is one
+  auto pval = [&](const auto& rw) -> F {
+    const T v = first ? rw.v[0] : rw.v[0] + beta * rw.v[1];
+    if constexpr (EPS) return F{v, rw.v[FIRST ? 1 : 2]};
+    else return v;
+  };
+  auto emit_d = [&](int xy, int, const auto& sr, const T (&o)[1], const bool bt) -> Out {
+    Stencil7<F> st;
     st.c = pval(sr.c);
     st.xm = pval(sr.xm);
     st.xp = pval(sr.xp);
@@ -120,28 +125,23 @@ __global__ void __launch_bounds__(MTX* MTY, (sizeof(T) == 4 && !EPS) ? 3 : 2) k_
     const int dlo = (B && st.zb < 0) ? (int)bc.tlo[xy] : 0;
     const int dhi = (B && st.za < 0) ? (int)bc.thi[xy] : 0;
     const T qv = apply_bt(st, dlo, dhi, ih2, bt);
-    apq.add(st.c, qv);
-    return Out{first ? o[0] : (xz ? alpha * sr.c.v[1] : o[0] + alpha * sr.c.v[1]), st.c, qv};
+    const T pc = field_value<T>(st.c);
+    apq.add(pc, qv);
+    if constexpr (FIRST) return Out{T(0), pc, qv};
+    else return Out{first ? o[0] : (xz ? alpha * sr.c.v[1] : o[0] + alpha * sr.c.v[1]), pc, qv};
   };
   const TileSched ts{&S->sched_next, &S->sched_done, mc.ntiles};
   for (long long t = sched_first(ts, &tile_slot); t < mc.ntiles; t = sched_next(ts, &tile_slot)) {
     s = tile_geo<MTX, MTY, VX>(g, t, mc);
     apq = Acc<T>();
     if constexpr (DIRECT && FIRST) {
-      const T* const hs1[1] = {r};
+      const T* hs1[EPS ? 2 : 1];
+      hs1[0] = r;
+      if constexpr (EPS) hs1[1] = eps;
       const T* const os1[1] = {nullptr};
-      auto emit_f = [&](int xy, int, const Stencil7<Raw<T, 1>>& sr, const T (&)[1], const bool bt) -> Out {
-        Stencil7<T> st = pick(sr, 0);
-        const bool B = bt;
-        const int dlo = (B && st.zb < 0) ? (int)bc.tlo[xy] : 0;
-        const int dhi = (B && st.za < 0) ? (int)bc.thi[xy] : 0;
-        const T qv = apply_bt(st, dlo, dhi, ih2, bt);
-        apq.add(st.c, qv);
-        return Out{T(0), st.c, qv};
-      };
-      march_direct<T, Out, MTX, MTY, VX, 1, 0, CGD_D>(g, s, smem, hs1, os1, emit_f, post);
+      march_direct<T, Out, MTX, MTY, VX, EPS ? 2 : 1, 0, CGD_D>(g, s, smem, hs1, os1, emit_d, post);
     } else if constexpr (DIRECT) {
-      static_assert(MG && !EPS, "the direct form is the multigrid search direction with eps = 1");
+      static_assert(MG, "the direct form is the multigrid search direction");
       if constexpr (SECOND) {          // x is not read: stage z and p_old alone
         const T* const os0[1] = {nullptr};
         march_direct<T, Out, MTX, MTY, VX, NH, 0, CGD_D>(g, s, smem, hsrc, os0, emit_d, post);
@@ -197,27 +197,37 @@ __global__ void __launch_bounds__(FLAT_THREADS) k_cg_r(Geo g, Bc<T> bc, const T*
   Acc<T> arr, arz;
   const long long nvec = g.n / NV;
   const long long stride = (long long)gridDim.x * FLAT_THREADS;
-  int cnt = 0;
+  // vectors in flight (a 4M-cell FP32 film: 15.2 us with four, 15.8 with two,
+  // 17.3 with one; FP64 27 with one, 28 with two)
+  constexpr int U = sizeof(T) == 8 ? 1 : MG ? 4 : 2;
   auto one = [&](long long e, T& rv, T qv) {
     rv = rv - alpha * qv;
     arr.add(rv, rv);
     if (!MG) arz.add(rv, rv * (EPS ? invd[e] : inv_flat(g, bc, e, inv6)));
   };
-  for (long long i = blockIdx.x * (long long)FLAT_THREADS + threadIdx.x; i < nvec; i += stride) {
-    V rv = reinterpret_cast<const V*>(r)[i];
-    const V qv = reinterpret_cast<const V*>(q)[i];
-    T* rs = reinterpret_cast<T*>(&rv);
-    const T* qs = reinterpret_cast<const T*>(&qv);
+  for (long long i0 = blockIdx.x * (long long)FLAT_THREADS + threadIdx.x; i0 < nvec; i0 += U * stride) {
+    V rv[U], qv[U];
 #pragma unroll
-    for (int k = 0; k < NV; ++k) one(i * NV + k, rs[k], qs[k]);
-    reinterpret_cast<V*>(r)[i] = rv;
-    arr.run();
-    arz.run();
-    if (++cnt == 16) {
-      arr.flush();
-      arz.flush();
-      cnt = 0;
+    for (int u = 0; u < U; ++u)
+      if (i0 + u * stride < nvec) {
+        rv[u] = reinterpret_cast<const V*>(r)[i0 + u * stride];
+        qv[u] = reinterpret_cast<const V*>(q)[i0 + u * stride];
+      }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const long long i = i0 + u * stride;
+      if (i < nvec) {
+        T* rs = reinterpret_cast<T*>(&rv[u]);
+        const T* qs = reinterpret_cast<const T*>(&qv[u]);
+#pragma unroll
+        for (int k = 0; k < NV; ++k) one(i * NV + k, rs[k], qs[k]);
+        reinterpret_cast<V*>(r)[i] = rv[u];
+        arr.run();
+        arz.run();
+      }
     }
+    arr.flush();
+    arz.flush();
   }
   for (long long e = nvec * NV + blockIdx.x * (long long)FLAT_THREADS + threadIdx.x; e < g.n; e += stride) {
     T rv = r[e];
@@ -259,8 +269,8 @@ __global__ void __launch_bounds__(FLAT_THREADS) k_cg_r(Geo g, Bc<T> bc, const T*
 
 template <typename T, bool EPS, bool MG, int VX, bool FIRST, bool SECOND>
 static void launch_cg_p_t(const LaunchCfg& L, const Geo& g, const Dev<T>& d) {
-  constexpr bool DIRECT = MG && !EPS;
-  using PD = Pipe<T, void, MTX, MTY, VX, FIRST ? 1 : 2, (FIRST || SECOND) ? 0 : 1, CGD_D>;
+  constexpr bool DIRECT = MG;
+  using PD = Pipe<T, void, MTX, MTY, VX, (FIRST ? 1 : 2) + (EPS ? 1 : 0), (FIRST || SECOND) ? 0 : 1, CGD_D>;
   const size_t bytes = DIRECT ? PD::bytes() : CgPipe<T, EPS, VX>::bytes();
   static bool once = false;
   if (!once) {
@@ -282,9 +292,8 @@ static void launch_cg_p_v(const LaunchCfg& L, const Geo& g, const Dev<T>& d) {
 
 template <typename T>
 void launch_cg_p(const LaunchCfg& L, const Geo& g, const Dev<T>& d, int mg, int first, int second) {
-  // with a permittivity field the multigrid form stages eps too (field-buffer
-  // march; its first iteration reads the first-iteration flag of the solver)
-  if (mg && d.eps) launch_cg_p_v<T, true, true>(L, g, d);
+  if (mg && d.eps && first) launch_cg_p_v<T, true, true, true>(L, g, d);
+  else if (mg && d.eps) launch_cg_p_v<T, true, true>(L, g, d);
   else if (mg && first) launch_cg_p_v<T, false, true, true>(L, g, d);
   else if (mg && second) launch_cg_p_v<T, false, true, false, true>(L, g, d);
   else if (mg) launch_cg_p_v<T, false, true>(L, g, d);
