@@ -8,6 +8,9 @@
 // only where it is interior or periodic), so each face counts once.
 // Sums: per-tile partials gathered in a fixed order; FP32 terms go through
 // the compensated accumulator.  Traffic per cell: reads 4 words, writes none.
+#include <cmath>
+#include <limits>
+
 #include "pf_internal.h"
 #include "pf_march.cuh"
 
@@ -22,8 +25,20 @@ using DiagPipe = Pipe<T, void, MTX, MTY, VX, 4, 0, DIAG_D>;
 template <typename T>
 struct DiagCoef {
   T a1, a11, a12;
-  double thr;          // compared with P_x in FP64
+  // P_x > threshold in FP64: for a float P_x that is P_x > thr, the largest
+  // float not above the threshold (in FP64 the conversion and comparison of
+  // every cell kept the FP64 unit busy for 64 of the 146 us that 512 x 512 x 64 took)
+  T thr;
 };
+
+// The largest T not above v.
+template <typename T>
+static T round_down(double v) {
+  T f = (T)v;
+  if ((double)f > v) f = std::nextafter(f, -std::numeric_limits<T>::infinity());
+  return f;
+}
+
 
 template <typename T, int VX>
 __global__ void __launch_bounds__(MTX* MTY) k_diag(Geo g, Bc<T> bc, const T* __restrict__ P,
@@ -52,7 +67,7 @@ __global__ void __launch_bounds__(MTX* MTY) k_diag(Geo g, Bc<T> bc, const T* __r
     acc[0].add(p[0], T(1));
     acc[1].add(p[1], T(1));
     acc[2].add(p[2], T(1));
-    acc[3].add((double)p[0] > k.thr ? T(1) : T(0), T(1));
+    acc[3].add(p[0] > k.thr ? T(1) : T(0), T(1));
     acc[4].add(k.a1, x2 + y2 + z2);
     acc[4].add(k.a11, x2 * x2 + y2 * y2 + z2 * z2);
     acc[4].add(k.a12, x2 * y2 + y2 * z2 + z2 * x2);
@@ -110,7 +125,7 @@ static void diag_t(const LaunchCfg& L, const Geo& g, const Dev<T>& d, const T* P
 
 template <typename T>
 void launch_diag(const LaunchCfg& L, const Geo& g, const Dev<T>& d, const T* P, const double* coef, double* out) {
-  const DiagCoef<T> k{T(coef[0]), T(coef[1]), T(coef[2]), coef[3]};
+  const DiagCoef<T> k{T(coef[0]), T(coef[1]), T(coef[2]), round_down<T>(coef[3])};
   constexpr int V = 16 / sizeof(T);
   if (L.march.vx == V) diag_t<T, V>(L, g, d, P, k, out);
   else diag_t<T, 1>(L, g, d, P, k, out);
