@@ -638,12 +638,19 @@ void comp_view(pf_ctx* ctx, pf::Dev<T>& d) {
   d.phi = (T*)(ws + ctx->lay.cx);
 }
 
-// Does a graph-captured step solve run its second iteration outside the
-// Krylov loop too, with the form that reads no correction (compensated
-// multigrid solves with eps = 1)?
-bool peel_second(const pf_ctx* ctx) {
-  return compensated(ctx) && ctx->prm.solver == PF_PCG_MG && !ctx->prm.has_eps;
+// Does a graph-captured multigrid solve run its first iteration before the
+// Krylov loop (with the form that reads neither p_old nor x)?  On films of two
+// million cells and more; on smaller ones the launches of a solve that needs no
+// iteration, which return at once, cost more than the words saved (a batch of
+// 30 films of 0.03 to 1 million cells, 0.8 iterations a solve: 0.93 ms a step
+// with them, 0.89 without).
+bool peel_first(const pf_ctx* ctx) {
+  return ctx->prm.solver == PF_PCG_MG && ctx->geo.n >= (1LL << 21);
 }
+
+// Does it run its second iteration outside the Krylov loop too, with the form
+// that reads no correction (compensated solves with eps = 1)?
+bool peel_second(const pf_ctx* ctx) { return peel_first(ctx) && compensated(ctx) && !ctx->prm.has_eps; }
 
 // Does a step solve start with k_extrap?  (Compensated series form their
 // start at the end of the solve before.)
@@ -812,9 +819,9 @@ void step_kernel_counts(pf_ctx* ctx, int refresh, int64_t* fixed, int64_t* per_i
   const int64_t per_solve = (ctx->singular ? 2 : 0) + 2 + (plain_extrap(ctx) ? 1 : 0);
   const bool loop = cg_loop_of(ctx);
   *per_iter = loop ? 0 : 2 + vc;
-  // graph-captured multigrid solves run their first iteration (compensated
-  // ones their first two) outside the loop
-  const int64_t peeled = vc ? *per_iter * (peel_second(ctx) ? 2 : 1) : 0;
+  // graph-captured multigrid solves of large films run their first iteration
+  // (compensated ones their first two) outside the loop
+  const int64_t peeled = peel_first(ctx) ? *per_iter * (peel_second(ctx) ? 2 : 1) : 0;
   *fixed = (refresh ? (heun ? 2 : 1) * (per_solve + peeled + (loop ? 1 : 0)) : 0) + (heun ? 2 : 1);
 }
 
@@ -878,7 +885,7 @@ cudaError_t append_step(pf_ctx* ctx, cudaGraph_t graph, std::vector<cudaGraphNod
         pf::launch_cg_finish<T>(ctx->L, g, d, ctx->singular);
         if (ctx->singular) pf::launch_sub_mean<T>(ctx->L, g, d);
       }
-      if (mg) {                  // the first iteration (p = z) runs outside the loop
+      if (peel_first(ctx)) {     // the first iteration (p = z) runs outside the loop
         vcycle<T>(ctx, 0);
         pf::launch_cg_p<T>(ctx->L, g, d, mg, 1);
         pf::launch_cg_r<T>(ctx->L, g, d, mg, h, 1);
@@ -1234,8 +1241,7 @@ pf_status finish_info(pf_ctx* ctx, int nsteps, pf_step_info* info) {
     // graph-launched steps: kernels = fixed part + one loop body per iteration
     // (multigrid: per iteration after the first, which is in the fixed part)
     // loop bodies: the iterations past the peeled ones, sum of max(0, iters - peeled)
-    const int64_t mg = ctx->prm.solver == PF_PCG_MG;
-    const int64_t bodies = !mg ? s.total_iters
+    const int64_t bodies = !peel_first(ctx) ? s.total_iters
                            : peel_second(ctx)
                                ? s.total_iters - 2 * ctx->graph_solves + s.zero_solves + s.short_solves
                                : s.total_iters + s.zero_solves - ctx->graph_solves;
