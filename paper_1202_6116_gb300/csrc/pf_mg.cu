@@ -66,39 +66,53 @@ __device__ __forceinline__ double rn_sub(double a, double b) { return __dsub_rn(
 __device__ __forceinline__ double rn_mul(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ double rn_fma(double a, double b, double c) { return __fma_rn(a, b, c); }
 
+//
+// The operator is taken as d c - S, d the diagonal (constant away from the z
+// faces) and S the weighted sum of the neighbours, with a sweep's constants
+// folded into the weights: seven to eight operations a cell and sweep instead
+// of 14 to 18.  FP64 sweeps are bound by the FP64 unit (one warp instruction in
+// 19 cycles per SM) and the fused FP32 passes by issue; neither by memory.
+// (Its rounding is of the size u |d c|, which storing c has cost already.)
 template <typename T>
-__device__ __forceinline__ T apply_int(T c, T xm, T xp, T ym, T yp, T zm, T zp, T ax, T ay, T az) {
-  const T sx = rn_add(rn_sub(c, xm), rn_sub(c, xp));
-  const T sy = rn_add(rn_sub(c, ym), rn_sub(c, yp));
-  const T sz = rn_add(rn_sub(c, zm), rn_sub(c, zp));
-  return rn_fma(ax, sx, rn_fma(ay, sy, rn_mul(az, sz)));
+__device__ __forceinline__ T nb_int(T xm, T xp, T ym, T yp, T zm, T zp, T kx, T ky, T kz, T base) {
+  return rn_fma(kx, rn_add(xm, xp), rn_fma(ky, rn_add(ym, yp), rn_fma(kz, rn_add(zm, zp), base)));
 }
 
-// FP64 sweeps are bound by the FP64 unit (one warp instruction in 19 cycles
-// per SM), not by memory: on the planes away from the z faces they take the
-// operator as d c - S, d the diagonal and S the weighted neighbour sum, and
-// fold the sweep's constants into the weights.  Seven to nine FP64 operations
-// a cell instead of 18 to 24; the finest level of a 256 x 256 x 64 film took
-// 179 (pre), 154 (rr), 188 (post1) and 145 us (post2) before.
-__device__ __forceinline__ double nb_sum(const Stencil7<double>& s, double kx, double ky, double kz, double base) {
-  return fma(kx, s.xm + s.xp, fma(ky, s.ym + s.yp, fma(kz, s.zm + s.zp, base)));
+// A sweep out = c + w D^-1 (f - A c) with D constant: out = kc c + kf f + S(kx, ky, kz).
+template <typename T>
+struct SweepK {
+  T kc, kf, kx, ky, kz;
+  // w: the weight over the diagonal
+  __device__ __forceinline__ SweepK(T w, T ax, T ay, T az)
+      : kc(rn_fma(-w, T(2) * (ax + ay + az), T(1))), kf(w), kx(w * ax), ky(w * ay), kz(w * az) {}
+};
+template <typename T>
+__device__ __forceinline__ T sweep_int(const SweepK<T>& k, T f, T c, T xm, T xp, T ym, T yp, T zm, T zp) {
+  return nb_int(xm, xp, ym, yp, zm, zp, k.kx, k.ky, k.kz, rn_fma(k.kf, f, rn_mul(k.kc, c)));
+}
+template <typename T>
+__device__ __forceinline__ T sweep_int(const SweepK<T>& k, T f, const Stencil7<T>& s) {
+  return sweep_int(k, f, s.c, s.xm, s.xp, s.ym, s.yp, s.zm, s.zp);
 }
 
-// e = e1 + w2 D^-1 (f - A e1), e1 = w1 D^-1 f, with D constant (w1 = omega1 / d,
-// w2d = omega2 / d): A e1 = w1 A f.
+// f - A c.
 template <typename T>
-__device__ __forceinline__ T pre_int(T c, T xm, T xp, T ym, T yp, T zm, T zp, T ax, T ay, T az, T w1, T w2d) {
-  const T Ae1 = rn_mul(w1, apply_int(c, xm, xp, ym, yp, zm, zp, ax, ay, az));
-  return rn_fma(w2d, rn_sub(c, Ae1), rn_mul(w1, c));
+__device__ __forceinline__ T res_int(T f, T c, T xm, T xp, T ym, T yp, T zm, T zp, T ax, T ay, T az, T d) {
+  return nb_int(xm, xp, ym, yp, zm, zp, ax, ay, az, rn_fma(-d, c, f));
 }
 
-// c + w (f - A c) on a plane away from the z faces, FP64 (see nb_sum).
+// Two sweeps from zero: e1 = w1 f, e = e1 + w2d (f - A e1) with D constant
+// (w1 = omega1 / d, w2d = omega2 / d): e = (w1 + w2d - w1 w2d d) f + w1 w2d S(f).
 template <typename T>
-__device__ __forceinline__ T sweep_int(const Stencil7<T>& s, T f, T w, T ax, T ay, T az) {
-  if constexpr (sizeof(T) == 8)
-    return nb_sum(s, w * ax, w * ay, w * az, fma(w, f, (T(1) - w * (T(2) * (ax + ay + az))) * s.c));
-  else
-    return T(0);
+struct PreK {
+  T kf, kx, ky, kz;
+  __device__ __forceinline__ PreK(T w1, T w2d, T ax, T ay, T az)
+      : kf(rn_fma(-rn_mul(w1, w2d), T(2) * (ax + ay + az), rn_add(w1, w2d))), kx(rn_mul(w1, w2d) * ax),
+        ky(rn_mul(w1, w2d) * ay), kz(rn_mul(w1, w2d) * az) {}
+};
+template <typename T>
+__device__ __forceinline__ T pre_int(const PreK<T>& k, T c, T xm, T xp, T ym, T yp, T zm, T zp) {
+  return nb_int(xm, xp, ym, yp, zm, zp, k.kx, k.ky, k.kz, rn_mul(k.kf, c));
 }
 
 template <typename T>
@@ -168,6 +182,7 @@ __global__ void __launch_bounds__(MTX* MTY, (sizeof(T) == 4 && !EPS) ? (INT ? 5 
   constexpr int NH = EPS ? 3 : 1;          // f (, eps, 1/diag)
   const T om1 = mg_omega1<T>(), om2 = mg_omega2<T>(), inv_int = mg_inv_int(L);
   const T w1 = rn_mul(om1, inv_int), w2d = rn_mul(om2, inv_int);
+  const PreK<T> pk(w1, w2d, L.ax, L.ay, L.az);
   const T* hsrc[NH];
   hsrc[0] = L.f;
   if constexpr (EPS) {
@@ -196,14 +211,7 @@ __global__ void __launch_bounds__(MTX* MTY, (sizeof(T) == 4 && !EPS) ? (INT ? 5 
       return e1.c.v + om2 * sr.c.v[2] * (f.c - Ae1);
     } else {
       const bool near = !INT && zfaces && (z == 1 || z == nz - 2);
-      if (!bt && !near) {
-        if constexpr (sizeof(T) == 8) {
-          const T k1 = w1 * w2d, d = T(2) * (L.ax + L.ay + L.az);
-          return nb_sum(f, k1 * L.ax, k1 * L.ay, k1 * L.az, (w1 + w2d - k1 * d) * f.c);
-        } else {
-          return pre_int(f.c, f.xm, f.xp, f.ym, f.yp, f.zm, f.zp, L.ax, L.ay, L.az, w1, w2d);
-        }
-      }
+      if (!bt && !near) return pre_int(pk, f.c, f.xm, f.xp, f.ym, f.yp, f.zm, f.zp);
       Stencil7<T> e1;
       const T ic = mg_inv(L, xy, z, inv_int);
       e1.c = om1 * ic * f.c;
@@ -246,7 +254,7 @@ __global__ void __launch_bounds__(MTX* MTY, (sizeof(T) == 4 && !EPS) ? (INT ? 5 
 // 2k+1 share a warp: lane ^ 16), 2 columns (inside the thread's vector, or
 // lane ^ 1 when a thread owns one cell).
 template <typename T, int VX, bool EPS>
-__global__ void __launch_bounds__(MTX* MTY) k_mg_rr(MgView<T> L, MgView<T> C, Scalars* S) {
+__global__ void __launch_bounds__(MTX* MTY, (sizeof(T) == 4 && !EPS) ? 4 : 2) k_mg_rr(MgView<T> L, MgView<T> C, Scalars* S) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ long long tile_slot;
   static_assert(MTX == 16, "row pairs share a warp");
@@ -256,7 +264,7 @@ __global__ void __launch_bounds__(MTX* MTY) k_mg_rr(MgView<T> L, MgView<T> C, Sc
   hsrc[0] = L.e;
   if constexpr (EPS) hsrc[1] = L.eps;
   const T* osrc[1] = {L.f};
-  const T scale = T(1) / T(L.fx * L.fy * L.fz);
+  const T scale = T(1) / T(L.fx * L.fy * L.fz), dg = T(2) * (L.ax + L.ay + L.az);
   TileGeo<MTX, MTY, VX> s;
   T racc[VX];
 #pragma unroll
@@ -270,10 +278,7 @@ __global__ void __launch_bounds__(MTX* MTY) k_mg_rr(MgView<T> L, MgView<T> C, Sc
     } else {
       if (!bt) {
         const Stencil7<T> e = pick(sr, 0);
-        if constexpr (sizeof(T) == 8)
-          return nb_sum(e, L.ax, L.ay, L.az, fma(T(-2) * (L.ax + L.ay + L.az), e.c, o[0]));
-        else
-          return rn_sub(o[0], apply_int(e.c, e.xm, e.xp, e.ym, e.yp, e.zm, e.zp, L.ax, L.ay, L.az));
+        return res_int(o[0], e.c, e.xm, e.xp, e.ym, e.yp, e.zm, e.zp, L.ax, L.ay, L.az, dg);
       }
       return o[0] - apply_aniso(pick(sr, 0), dlo, dhi, L.ax, L.ay, L.az, bt);
     }
@@ -330,7 +335,7 @@ __global__ void __launch_bounds__(MTX* MTY) k_mg_rr(MgView<T> L, MgView<T> C, Sc
 // face, which belong to the face slabs: there it is the face-slab
 // pre-smoother's output, read back (that launch runs first; the face-slab
 // residual runs after this one).  The arithmetic per cell is pre_int and
-// apply_int, as in k_mg_pre and k_mg_rr, so the results are bit-identical.
+// res_int, as in k_mg_pre and k_mg_rr, so the results are bit-identical.
 // One barrier per plane: the e plane a tile writes at plane u (buffer u mod 2)
 // was last read for the residual of plane u - 2, and stage u + 4 mod 5 last
 // held plane u - 1; both reads end before the barrier of plane u.
@@ -354,8 +359,8 @@ __global__ void __launch_bounds__(MTX* MTY, 4) k_mg_prr(MgView<float> L, MgView<
   const int nx = L.g.nx, ny = L.g.ny, nz = L.g.nz;
   const long long nxy = L.g.nxy;
   const float om1 = mg_omega1<float>(), om2 = mg_omega2<float>(), inv_int = mg_inv_int(L);
-  const float w1 = rn_mul(om1, inv_int), w2d = rn_mul(om2, inv_int);
-  const float ax = L.ax, ay = L.ay, az = L.az;
+  const PreK<float> pk(rn_mul(om1, inv_int), rn_mul(om2, inv_int), L.ax, L.ay, L.az);
+  const float ax = L.ax, ay = L.ay, az = L.az, dg = 2.f * (ax + ay + az);
   const float scale = 1.0f / float(L.fx * L.fy * L.fz);
   const int tx = threadIdx.x, ty = threadIdx.y, tid = tx + ty * MTX;
   const int c0 = 4 + 4 * tx;               // column of the own vector in a stage or e plane
@@ -413,7 +418,7 @@ __global__ void __launch_bounds__(MTX* MTY, 4) k_mg_prr(MgView<float> L, MgView<
     // e at a staged cell from the f planes below, at and above it
     auto e_at = [&](const float* sm, const float* sc, const float* sp, int off) -> float {
       const float* q = sc + off;
-      return pre_int(q[0], q[-1], q[1], q[-PRR_RS], q[PRR_RS], sm[off], sp[off], ax, ay, az, w1, w2d);
+      return pre_int(pk, q[0], q[-1], q[1], q[-PRR_RS], q[PRR_RS], sm[off], sp[off]);
     };
     float em2[4], em1[4], e0[4], racc[4];
 #pragma unroll
@@ -444,8 +449,7 @@ __global__ void __launch_bounds__(MTX* MTY, 4) k_mg_prr(MgView<float> L, MgView<
         if (tx == MTX - 1) fr = sc[so + 4];
 #pragma unroll
         for (int i = 0; i < 4; ++i)
-          e0[i] = pre_int(fc[i], i == 0 ? fl : fc[i - 1], i == 3 ? fr : fc[i + 1], fym[i], fyp[i], fm[i], fp[i], ax,
-                          ay, az, w1, w2d);
+          e0[i] = pre_int(pk, fc[i], i == 0 ? fl : fc[i - 1], i == 3 ? fr : fc[i + 1], fym[i], fyp[i], fm[i], fp[i]);
       }
       // planes whose residual this tile forms: e on the own vector and the ring
       if (u >= 1 && u <= nt) {
@@ -465,8 +469,8 @@ __global__ void __launch_bounds__(MTX* MTY, 4) k_mg_prr(MgView<float> L, MgView<
         if (tx == MTX - 1) er = ebm[eo + 4];
 #pragma unroll
         for (int i = 0; i < 4; ++i)
-          rv[i] = rn_sub(fv[i], apply_int(ec[i], i == 0 ? el : ec[i - 1], i == 3 ? er : ec[i + 1], eym[i], eyp[i],
-                                          em2[i], e0[i], ax, ay, az));
+          rv[i] = res_int(fv[i], ec[i], i == 0 ? el : ec[i - 1], i == 3 ? er : ec[i + 1], eym[i], eyp[i], em2[i],
+                          e0[i], ax, ay, az, dg);
         const int zr = z - 1;
         *reinterpret_cast<float4*>(L.e + (long long)zr * nxy + s.xy) = make_float4(ec[0], ec[1], ec[2], ec[3]);
         // restriction: 2 planes in registers, 2 rows by lane ^ 16, 2 columns in the vector
@@ -541,8 +545,8 @@ __global__ void __launch_bounds__(MTX* MTY, 3) k_mg_pp(MgView<float> L, MgView<f
   const int nx = L.g.nx, ny = L.g.ny, nz = L.g.nz, cnx = C.g.nx, cny = C.g.ny;
   const long long nxy = L.g.nxy, cnxy = C.g.nxy;
   const float inv_int = mg_inv_int(L);
-  const float w2d = rn_mul(mg_omega2<float>(), inv_int), w1d = rn_mul(mg_omega1<float>(), inv_int);
-  const float ax = L.ax, ay = L.ay, az = L.az;
+  const SweepK<float> k2(rn_mul(mg_omega2<float>(), inv_int), L.ax, L.ay, L.az);
+  const SweepK<float> k1(rn_mul(mg_omega1<float>(), inv_int), L.ax, L.ay, L.az);
   const int tx = threadIdx.x, ty = threadIdx.y, tid = tx + ty * MTX;
   const int c0 = 4 + 4 * tx;
   const int so = (ty + 2) * PRR_RS + c0;   // own vector in a staged field plane
@@ -625,10 +629,8 @@ __global__ void __launch_bounds__(MTX* MTY, 3) k_mg_pp(MgView<float> L, MgView<f
     };
     // e' at staged cell (r, c) from the stages of the planes below, at and above it
     auto ep_at = [&](const float* sm, const float* sc, const float* sp, int r, int c) -> float {
-      const float uc = u_at(sc, r, c);
-      const float Au = apply_int(uc, u_at(sc, r, c - 1), u_at(sc, r, c + 1), u_at(sc, r - 1, c), u_at(sc, r + 1, c),
-                                 u_at(sm, r, c), u_at(sp, r, c), ax, ay, az);
-      return rn_fma(w2d, rn_sub(sc[PRR_STAGE + r * PRR_RS + c], Au), uc);
+      return sweep_int(k2, sc[PRR_STAGE + r * PRR_RS + c], u_at(sc, r, c), u_at(sc, r, c - 1), u_at(sc, r, c + 1),
+                       u_at(sc, r - 1, c), u_at(sc, r + 1, c), u_at(sm, r, c), u_at(sp, r, c));
     };
     float em2[4], e0[4];
 #pragma unroll
@@ -673,8 +675,7 @@ __global__ void __launch_bounds__(MTX* MTY, 3) k_mg_pp(MgView<float> L, MgView<f
         for (int i = 0; i < 4; ++i) {
           const float ym = eym[i] + (i < 2 ? pYM.x : pYM.y), yp = eyp[i] + (i < 2 ? pYP.x : pYP.y);
           const float zm = ezm[i] + (i < 2 ? pZM.x : pZM.y), zp = ezp[i] + (i < 2 ? pZP.x : pZP.y);
-          const float Au = apply_int(uc[i], i == 0 ? uL : uc[i - 1], i == 3 ? uR : uc[i + 1], ym, yp, zm, zp, ax, ay, az);
-          e0[i] = rn_fma(w2d, rn_sub(fc[i], Au), uc[i]);
+          e0[i] = sweep_int(k2, fc[i], uc[i], i == 0 ? uL : uc[i - 1], i == 3 ? uR : uc[i + 1], ym, yp, zm, zp);
         }
       }
       if (u >= 1 && u <= nt) {
@@ -695,9 +696,8 @@ __global__ void __launch_bounds__(MTX* MTY, 3) k_mg_pp(MgView<float> L, MgView<f
         if (tx == MTX - 1) er = ebm[eo + 4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-          const float Ae = apply_int(ec[i], i == 0 ? el : ec[i - 1], i == 3 ? er : ec[i + 1], eym[i], eyp[i], em2[i],
-                                     e0[i], ax, ay, az);
-          ev[i] = rn_fma(w1d, rn_sub(fv[i], Ae), ec[i]);
+          ev[i] = sweep_int(k1, fv[i], ec[i], i == 0 ? el : ec[i - 1], i == 3 ? er : ec[i + 1], eym[i], eyp[i], em2[i],
+                            e0[i]);
           arz.add(fv[i], ev[i]);
         }
         arz.run();
@@ -727,6 +727,7 @@ __global__ void __launch_bounds__(MTX* MTY, (sizeof(T) == 4 && !EPS) ? 3 : 2) k_
   constexpr int NH = EPS ? 2 : 1;          // e (, eps); the parents come as field NH
   constexpr int NO = EPS ? 2 : 1;          // f (, 1/diag)
   const T om = mg_omega2<T>(), inv_int = mg_inv_int(L);
+  const SweepK<T> sk(rn_mul(om, inv_int), L.ax, L.ay, L.az);
   const T* hsrc[NH];
   hsrc[0] = L.e;
   if constexpr (EPS) hsrc[1] = L.eps;
@@ -761,9 +762,7 @@ __global__ void __launch_bounds__(MTX* MTY, (sizeof(T) == 4 && !EPS) ? 3 : 2) k_
       const T Ae = apply_aniso_eps(se, dlo, dhi, L.ax, L.ay, L.az, bt);
       return st.c + om * o[1] * (o[0] - Ae);
     } else {
-      if constexpr (sizeof(T) == 8) {
-        if (!bt) return sweep_int(st, o[0], om * inv_int, L.ax, L.ay, L.az);
-      }
+      if (!bt) return sweep_int(sk, o[0], st);
       const T Ae = apply_aniso(st, dlo, dhi, L.ax, L.ay, L.az, bt);
       return st.c + om * mg_inv_bt(L, xy, z, inv_int, bt) * (o[0] - Ae);
     }
@@ -791,6 +790,7 @@ __global__ void __launch_bounds__(MTX* MTY, (sizeof(T) == 4 && !EPS) ? (INT ? 5 
   constexpr int NH = EPS ? 2 : 1;          // et (, eps)
   constexpr int NO = EPS ? 2 : 1;          // f (, 1/diag)
   const T om = mg_omega1<T>(), inv_int = mg_inv_int(L);
+  const SweepK<T> sk(rn_mul(om, inv_int), L.ax, L.ay, L.az);
   const T* hsrc[NH];
   hsrc[0] = L.et;
   if constexpr (EPS) hsrc[1] = L.eps;
@@ -809,8 +809,8 @@ __global__ void __launch_bounds__(MTX* MTY, (sizeof(T) == 4 && !EPS) ? (INT ? 5 
       e = sr.c.v[0] + om * o[1] * (o[0] - Ae);
     } else {
       const Stencil7<T> st = pick(sr, 0);
-      if (sizeof(T) == 8 && !bt) {
-        e = sweep_int(st, o[0], om * inv_int, L.ax, L.ay, L.az);
+      if (!bt) {
+        e = sweep_int(sk, o[0], st);
       } else {
         const T Ae = apply_aniso(st, dlo, dhi, L.ax, L.ay, L.az, bt);
         e = st.c + om * mg_inv_bt(L, xy, z, inv_int, bt) * (o[0] - Ae);
