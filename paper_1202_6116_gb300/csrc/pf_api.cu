@@ -431,6 +431,7 @@ pf::Dev<T> dev_view(pf_ctx* ctx) {
   d.bc.thi = (const int8_t*)(ws + L.thi);
   d.bc.vlo = (const T*)(ws + L.vlo);
   d.bc.vhi = (const T*)(ws + L.vhi);
+  pf::diag_table<T>(ctx->geo.ih2, d.bc.itab);
   d.part = (double*)(ws + L.part);
   d.S = (Scalars*)(ws + L.S);
   d.plo = comp_state(&ctx->prm) ? (unsigned short*)(ws + L.plo) : nullptr;
@@ -476,6 +477,7 @@ pf::MgView<T> mg_view(pf_ctx* ctx, size_t k) {
     v.invd = (const T*)(ctx->ws + (k == 0 ? ctx->lay.invd : l.invd));
   }
   v.mc = l.mc;
+  pf::sweep_constants(v);
   v.split = !ctx->mg_whole && pf::mg_split_level(l.n(), l.nz, ctx->prm.periodic_z, ctx->prm.has_eps) ? 1 : 0;
   return v;
 }
@@ -1156,9 +1158,10 @@ std::vector<char> tail_blob(pf_ctx* ctx, const std::vector<std::vector<int8_t>>&
     d.ay = v.ay;
     d.az = v.az;
     for (int i = 0; i < 9; ++i) {
-      auto faces = [](int kind) { return kind == 0 ? 1 : 2 * (kind - 1); };
-      d.tab[i] = T(1) / (T(2) * v.ax + T(2) * v.ay + T(faces(i / 3) + faces(i % 3)) * v.az);
+      d.tab[i] = v.k.tab[i];
+      d.diag[i] = T(2) * (v.ax + v.ay) + T(pf::faces_of(i / 3) + pf::faces_of(i % 3)) * v.az;
     }
+    d.scale = v.k.scale;
     d.f = v.f;
     d.e = v.e;
     d.et = v.et;

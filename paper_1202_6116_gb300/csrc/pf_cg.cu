@@ -52,7 +52,7 @@ __global__ void __launch_bounds__(MTX* MTY, (sizeof(T) == 4 && !EPS) ? 3 : 2) k_
   const int pb = S->pbuf;
   const T* pold = pb ? p1 : p0;
   T* __restrict__ pnew = pb ? p0 : p1;
-  const T inv6 = T(1) / (T(6) * T(g.ih2));
+  const T inv6 = bc.itab[0];
   const T ih2 = T(g.ih2);
   Acc<T> apq;
   const T* hsrc[NH];
@@ -193,7 +193,7 @@ __global__ void __launch_bounds__(FLAT_THREADS) k_cg_r(Geo g, Bc<T> bc, const T*
   using V = typename Vec16<T>::type;
   constexpr int NV = 16 / sizeof(T);
   const T alpha = T(S->alpha);
-  const T inv6 = T(1) / (T(6) * T(g.ih2));
+  const T inv6 = bc.itab[0];
   Acc<T> arr, arz;
   const long long nvec = g.n / NV;
   const long long stride = (long long)gridDim.x * FLAT_THREADS;

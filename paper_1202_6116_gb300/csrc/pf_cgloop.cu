@@ -111,24 +111,14 @@ k_cg_loop(Geo g, Bc<T> bc, T* r, T* p0, T* p1, T* q, T* x, double* part, Scalars
   using Sum = typename SumOf<T>::type;
   __shared__ Sum scratch[2 * NT];
   __shared__ double tot[2], alpha_s, beta_s, rel_s;
-  __shared__ T itab[9];
   __shared__ int verdict, ok;           // verdict: 0 go on, 1 converged, 2 maxit, 3 breakdown, 4 non-finite
   if (S->done) return;                  // written by this kernel only after the last barrier
   const int tx = threadIdx.x, ty = threadIdx.y, tid = tx + 16 * ty + 256 * threadIdx.z;
-  const int nb = gridDim.x, nx = g.nx, ny = g.ny, nz = g.nz;
+  const int nb = gridDim.x, nx = g.nx, ny = g.ny;
   const long long nxy = g.nxy;
   const T ih2 = T(g.ih2);
-  // 1/diag by the kind of the z faces: 0 interior, 1 open, 2 electrode
-  if (tid < 9) {
-    const int lo = tid / 3, hi = tid % 3;
-    itab[tid] = T(1) / (T(4 + (lo == 0 ? 1 : 2 * (lo - 1)) + (hi == 0 ? 1 : 2 * (hi - 1))) * ih2);
-  }
-  __syncthreads();
-  const T inv6 = itab[0];
-  auto inv_at = [&](int xy, int z) -> T {
-    if (g.periodic_z || (z > 0 && z < nz - 1)) return inv6;
-    return itab[3 * (z > 0 ? 0 : 1 + (int)bc.tlo[xy]) + (z < nz - 1 ? 0 : 1 + (int)bc.thi[xy])];
-  };
+  const T inv6 = bc.itab[0];
+  auto inv_at = [&](int xy, int z) -> T { return inv_diag_unit(g, bc, xy, z, inv6); };
   const double rtol = S->rtol, bnorm = S->bnorm;
   const int maxit = S->maxit;
   double rz = S->rz, rr = 0.0, rel = S->last_rel, alpha = 0.0;

@@ -53,14 +53,20 @@ __device__ __forceinline__ int small_div(int a, int d, float r) {
   return q;
 }
 
+// Where a cell's diagonal stands in a level's tables.
+template <typename T>
+__device__ __forceinline__ int sub_kind(const SubDesc<T>& L, const int8_t* lo, const int8_t* hi, int x, int y, int z) {
+  if (L.per || (z > 0 && z < L.nz - 1)) return 0;
+  const int xy = y * L.nx + x;
+  return 3 * (z > 0 ? 0 : 1 + (int)lo[xy]) + (z < L.nz - 1 ? 0 : 1 + (int)hi[xy]);
+}
+
 // 1/diag at cell (x, y, z) with linear index c; lo, hi: the level's face masks.
 template <typename T, bool EPS>
 __device__ __forceinline__ T sub_inv(const SubDesc<T>& L, const int8_t* lo, const int8_t* hi, int c, int x, int y,
                                      int z) {
   if constexpr (EPS) return L.invd[c];
-  if (L.per || (z > 0 && z < L.nz - 1)) return L.tab[0];
-  const int xy = y * L.nx + x;
-  return L.tab[3 * (z > 0 ? 0 : 1 + (int)lo[xy]) + (z < L.nz - 1 ? 0 : 1 + (int)hi[xy])];
+  return L.tab[sub_kind(L, lo, hi, x, y, z)];
 }
 
 // VX cells in a row from (x, y, z) on: linear index, neighbour rows and planes
@@ -86,12 +92,14 @@ struct SubRow {
   }
 };
 
-// A v at VX cells in a row.  vec(index, x, y, z, o) gives the field at the VX
-// cells from there on, one(index, x, y, z) at one cell; vc: the field at the
-// cells themselves.
+// f - A v at VX cells in a row.  vec(index, x, y, z, o) gives v at the VX cells
+// from there on, one(index, x, y, z) at one cell; vc: v at the cells
+// themselves.  With eps = 1 as f - d v + S (d the diagonal, S the weighted sum
+// of the neighbours): 7 FP64 operations a cell, 13 as differences.
 template <typename T, bool EPS, int VX, class Vec, class One>
-__device__ __forceinline__ void sub_apply(const SubDesc<T>& L, const int8_t* lo, const int8_t* hi,
-                                          const SubRow<T, VX>& s, const T (&vc)[VX], T (&out)[VX], Vec vec, One one) {
+__device__ __forceinline__ void sub_res(const SubDesc<T>& L, const int8_t* lo, const int8_t* hi,
+                                          const SubRow<T, VX>& s, const T (&fc)[VX], const T (&vc)[VX], T (&out)[VX],
+                                        Vec vec, One one) {
   const int xl = s.x == 0 ? L.nx - 1 : s.x - 1, xr = s.x + VX == L.nx ? 0 : s.x + VX;
   const int cl = s.c - s.x + xl, cr = s.c - s.x + xr;
   const int cym = s.c + (s.ym - s.y) * L.nx, cyp = s.c + (s.yp - s.y) * L.nx;
@@ -104,8 +112,8 @@ __device__ __forceinline__ void sub_apply(const SubDesc<T>& L, const int8_t* lo,
   for (int i = 0; i < VX; ++i) zm[i] = zp[i] = T(0);
   if (s.zm >= 0) vec(czm, s.x, s.y, s.zm, zm);
   if (s.zp >= 0) vec(czp, s.x, s.y, s.zp, zp);
-  const int xy = s.y * L.nx + s.x;
   if constexpr (EPS) {
+    const int xy = s.y * L.nx + s.x;
     T ec[VX], eym[VX], eyp[VX], ezm[VX], ezp[VX];
     load_n<T, VX>(L.eps + s.c, ec);
     load_n<T, VX>(L.eps + cym, eym);
@@ -126,20 +134,15 @@ __device__ __forceinline__ void sub_apply(const SubDesc<T>& L, const int8_t* lo,
       else if (lo[xy + i]) sz += T(2) * e * v;
       if (s.zp >= 0) sz += hmean2(e, ezp[i]) * (v - zp[i]);
       else if (hi[xy + i]) sz += T(2) * e * v;
-      out[i] = L.ax * sx + L.ay * sy + L.az * sz;
+      out[i] = fc[i] - (L.ax * sx + L.ay * sy + L.az * sz);
     }
   } else {
 #pragma unroll
     for (int i = 0; i < VX; ++i) {
-      const T v = vc[i];
-      const T sx = (v - (i == 0 ? vl : vc[i - 1])) - ((i == VX - 1 ? vr : vc[i + 1]) - v);
-      const T sy = (v - ym[i]) - (yp[i] - v);
-      T sz = T(0);
-      if (s.zm >= 0) sz += v - zm[i];
-      else if (lo[xy + i]) sz += T(2) * v;
-      if (s.zp >= 0) sz += v - zp[i];
-      else if (hi[xy + i]) sz += T(2) * v;
-      out[i] = L.ax * sx + L.ay * sy + L.az * sz;
+      T r = fc[i] - L.diag[sub_kind(L, lo, hi, s.x + i, s.y, s.z)] * vc[i];
+      r += L.az * (zm[i] + zp[i]);
+      r += L.ay * (ym[i] + yp[i]);
+      out[i] = r + L.ax * ((i == 0 ? vl : vc[i - 1]) + (i == VX - 1 ? vr : vc[i + 1]));
     }
   }
 }
@@ -154,7 +157,7 @@ __device__ __forceinline__ void sub_pre(const SubDesc<T>& L, const int8_t* lo, c
   const T om1 = mg_omega1<T>(), om2 = mg_omega2<T>();
   for (int i = i0; i < L.n / VX; i += stride) {
     const SubRow<T, VX> s(L, i);
-    T fc[VX], ec[VX], inv[VX], Ae[VX];
+    T fc[VX], ec[VX], inv[VX], res[VX];
     load_n<T, VX>(f + s.c, fc);
 #pragma unroll
     for (int k = 0; k < VX; ++k) inv[k] = sub_inv<T, EPS>(L, lo, hi, s.c + k, s.x + k, s.y, s.z);
@@ -165,8 +168,8 @@ __device__ __forceinline__ void sub_pre(const SubDesc<T>& L, const int8_t* lo, c
       };
 #pragma unroll
       for (int k = 0; k < VX; ++k) ec[k] = om1 * inv[k] * fc[k];
-      sub_apply<T, EPS, VX>(
-          L, lo, hi, s, ec, Ae,
+      sub_res<T, EPS, VX>(
+          L, lo, hi, s, fc, ec, res,
           [&](int j, int x, int y, int z, T (&o)[VX]) {
             load_n<T, VX>(f + j, o);
 #pragma unroll
@@ -175,12 +178,12 @@ __device__ __forceinline__ void sub_pre(const SubDesc<T>& L, const int8_t* lo, c
           [&](int j, int x, int y, int z) -> T { return w(j, x, y, z) * f[j]; });
     } else {
       load_n<T, VX>(e1 + s.c, ec);
-      sub_apply<T, EPS, VX>(
-          L, lo, hi, s, ec, Ae, [&](int j, int, int, int, T (&o)[VX]) { load_n<T, VX>(e1 + j, o); },
+      sub_res<T, EPS, VX>(
+          L, lo, hi, s, fc, ec, res, [&](int j, int, int, int, T (&o)[VX]) { load_n<T, VX>(e1 + j, o); },
           [&](int j, int, int, int) -> T { return e1[j]; });
     }
 #pragma unroll
-    for (int k = 0; k < VX; ++k) ec[k] += om2 * inv[k] * (fc[k] - Ae[k]);
+    for (int k = 0; k < VX; ++k) ec[k] += om2 * inv[k] * res[k];
     store_n<T, VX>(e + s.c, ec);
   }
 }
@@ -192,7 +195,7 @@ template <typename T, bool EPS, int VX>
 __device__ __forceinline__ void sub_restrict(const SubDesc<T>& L, const int8_t* lo, const int8_t* hi, const T* f,
                                              const T* e, const SubDesc<T>& C, const int8_t* clo, const int8_t* chi,
                                              T* fc, T* e1c, int i0, int stride) {
-  const T scale = T(1) / T(L.fx * L.fy * L.fz);
+  const T scale = L.scale;
   const int cv = VX == 1 ? 1 : VX / L.fx;                          // coarse cells of a group
   const int gs = L.fy * L.fz, sh = gs >> 1, total = C.n / cv * gs; // gs = 1, 2, 4: shift 0, 1, 2
   const int lane = threadIdx.x & 31, nv = C.nx / cv;
@@ -210,11 +213,9 @@ __device__ __forceinline__ void sub_restrict(const SubDesc<T>& L, const int8_t* 
         T ec[VX], fv[VX];
         load_n<T, VX>(e + s.c, ec);
         load_n<T, VX>(f + s.c, fv);
-        sub_apply<T, EPS, VX>(
-            L, lo, hi, s, ec, o, [&](int j, int, int, int, T (&v)[VX]) { load_n<T, VX>(e + j, v); },
+        sub_res<T, EPS, VX>(
+            L, lo, hi, s, fv, ec, o, [&](int j, int, int, int, T (&v)[VX]) { load_n<T, VX>(e + j, v); },
             [&](int j, int, int, int) -> T { return e[j]; });
-#pragma unroll
-        for (int k = 0; k < VX; ++k) o[k] = fv[k] - o[k];
       };
       res(X * L.fx, acc);
       if (L.fx == 2) {
@@ -259,15 +260,15 @@ __device__ __forceinline__ void sub_post1(const SubDesc<T>& L, const int8_t* lo,
   };
   for (int i = i0; i < L.n / VX; i += stride) {
     const SubRow<T, VX> s(L, i);
-    T uc[VX], fc[VX], Au[VX];
+    T uc[VX], fc[VX], res[VX];
     vec(s.c, s.x, s.y, s.z, uc);
     load_n<T, VX>(f + s.c, fc);
-    sub_apply<T, EPS, VX>(L, lo, hi, s, uc, Au, vec, [&](int j, int x, int y, int z) -> T {
+    sub_res<T, EPS, VX>(L, lo, hi, s, fc, uc, res, vec, [&](int j, int x, int y, int z) -> T {
       return e[j] + ec[((z >> sz) * cny + (y >> sy)) * cnx + (x >> sx)];
     });
 #pragma unroll
     for (int k = 0; k < VX; ++k)
-      uc[k] += om * sub_inv<T, EPS>(L, lo, hi, s.c + k, s.x + k, s.y, s.z) * (fc[k] - Au[k]);
+      uc[k] += om * sub_inv<T, EPS>(L, lo, hi, s.c + k, s.x + k, s.y, s.z) * res[k];
     store_n<T, VX>(et + s.c, uc);
   }
 }
@@ -278,15 +279,15 @@ __device__ __forceinline__ void sub_post2(const SubDesc<T>& L, const int8_t* lo,
   const T om = mg_omega1<T>();
   for (int i = i0; i < L.n / VX; i += stride) {
     const SubRow<T, VX> s(L, i);
-    T vc[VX], fc[VX], Av[VX];
+    T vc[VX], fc[VX], res[VX];
     load_n<T, VX>(et + s.c, vc);
     load_n<T, VX>(f + s.c, fc);
-    sub_apply<T, EPS, VX>(
-        L, lo, hi, s, vc, Av, [&](int j, int, int, int, T (&o)[VX]) { load_n<T, VX>(et + j, o); },
+    sub_res<T, EPS, VX>(
+        L, lo, hi, s, fc, vc, res, [&](int j, int, int, int, T (&o)[VX]) { load_n<T, VX>(et + j, o); },
         [&](int j, int, int, int) -> T { return et[j]; });
 #pragma unroll
     for (int k = 0; k < VX; ++k) {
-      vc[k] += om * sub_inv<T, EPS>(L, lo, hi, s.c + k, s.x + k, s.y, s.z) * (fc[k] - Av[k]);
+      vc[k] += om * sub_inv<T, EPS>(L, lo, hi, s.c + k, s.x + k, s.y, s.z) * res[k];
       arz.add(fc[k], vc[k]);
     }
     arz.run();

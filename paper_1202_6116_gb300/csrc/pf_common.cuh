@@ -52,7 +52,18 @@ struct Bc {
   const int8_t* thi;
   const T* vlo;
   const T* vhi;
+  T itab[9];               // 1/diag(A) with eps = 1, by 3 (kind of the lower z face) + kind of the upper one
+                           // (0 interior, 1 open, 2 electrode); see diag_table
 };
+
+// faces_of: the weight of a z face of each kind in the diagonal.  The nine
+// values are formed on the host: a division is 20 FP64 operations, and one per
+// thread at the start of a kernel is 6 us on an SM's FP64 unit.
+inline int faces_of(int kind) { return kind == 0 ? 1 : 2 * (kind - 1); }
+template <typename T>
+inline void diag_table(double ih2, T (&tab)[9]) {
+  for (int i = 0; i < 9; ++i) tab[i] = T(1) / (T(4 + faces_of(i / 3) + faces_of(i % 3)) * T(ih2));
+}
 
 // 16-byte vector type of a field element type.
 template <typename T>
@@ -68,13 +79,12 @@ struct Vec16<double> {
 
 // 1/diag(A) at column xy of plane z when eps = 1.  The diagonal is
 // (interior faces + 2 x electrode faces)/dx^2: 6/dx^2 away from the z faces.
-// Every kernel forms it through this one expression, so z = r/diag agrees
-// bit for bit between kernels.
+// Every kernel takes it from the one table, so z = r/diag agrees bit for bit
+// between kernels.
 template <typename T>
 __device__ __forceinline__ T inv_diag_unit(const Geo& g, const Bc<T>& bc, long long xy, int z, T inv6) {
   if (g.periodic_z || (z > 0 && z < g.nz - 1)) return inv6;
-  const int k = 4 + (z > 0 ? 1 : 2 * (int)bc.tlo[xy]) + (z < g.nz - 1 ? 1 : 2 * (int)bc.thi[xy]);
-  return T(1) / (T(k) * T(g.ih2));
+  return bc.itab[3 * (z > 0 ? 0 : 1 + (int)bc.tlo[xy]) + (z < g.nz - 1 ? 0 : 1 + (int)bc.thi[xy])];
 }
 
 // Same, addressed by the linear cell index e.

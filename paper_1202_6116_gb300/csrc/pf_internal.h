@@ -86,6 +86,40 @@ struct Dev {
   unsigned short* plo;   // remainder of a compensated FP32 polarization state (3N bf16), or nullptr
 };
 
+// Jacobi weights of the two smoothing sweeps: the reciprocals of the roots of
+// the degree-2 Chebyshev polynomial on [b/4, b], b = 1.9, which bound the
+// spectrum of diag(A)^-1 A (in [0, 2] for this M-matrix) from below b/4 up,
+// i.e. 1/lambda_k with lambda_k = (b + a)/2 + (b - a)/2 cos((2k - 1) pi / 4),
+// a = b/4.  The pair damps the upper three quarters of the spectrum (the part
+// the coarse grid cannot represent) by |(1 - w1 l)(1 - w2 l)| <= 0.35 on
+// [b/4, 2]; weighted Jacobi with 6/7 twice leaves up to 0.51 there.  The
+// pre-smoother applies w1 then w2, the post-smoother w2 then w1.
+constexpr double MG_OMEGA1 = 0.5912564121058501;
+constexpr double MG_OMEGA2 = 1.462658863889015;
+
+// Constants of a level's sweeps with eps = 1, formed on the host: per thread
+// they are a division and a dozen operations, and as many again per phase of
+// the small levels, on the FP64 unit of each SM (the adjoint of 128 x 128 x 32:
+// 55.3 -> 46.0 ms with these and the small levels' d c - S; FP64 256 x 256 x 64
+// 8.13 -> 7.68 ms per 4 steps).  On the
+// planes away from the z faces the operator is d c - S, d the diagonal and S
+// the weighted sum of the neighbours, and a sweep's constants fold into the
+// weights:
+//   both pre-sweeps from zero  e   = p.kf f + S(p.kx, p.ky, p.kz)
+//   one sweep of weight w      out = kc c + kf f + S(kx, ky, kz)
+template <typename T>
+struct LevelK {
+  struct Pre {
+    T kf, kx, ky, kz;
+  } pre;
+  struct Sweep {
+    T kc, kf, kx, ky, kz;
+  } s1, s2;                // weights omega1, omega2
+  T d;                     // the diagonal
+  T tab[9];                // 1/diag by the kinds of the z faces (as Bc::itab)
+  T scale;                 // 1 / children of a coarse cell
+};
+
 // One multigrid level as the kernels see it.
 template <typename T>
 struct MgView {
@@ -99,9 +133,23 @@ struct MgView {
   T* et;              // second buffer of the Jacobi sweeps
   const T* eps;       // cell permittivity of this level (nullptr: eps = 1)
   const T* invd;      // 1/diag of this level's operator (with eps only)
+  LevelK<T> k;
   MarchCfg mc;
   int split;          // 1: its split sweeps run as interior + face-slab launches (mg_split_level)
 };
+
+template <typename T>
+inline void sweep_constants(MgView<T>& v) {
+  LevelK<T>& k = v.k;
+  for (int i = 0; i < 9; ++i)
+    k.tab[i] = T(1) / (T(2) * v.ax + T(2) * v.ay + T(faces_of(i / 3) + faces_of(i % 3)) * v.az);
+  k.d = T(2) * (v.ax + v.ay + v.az);
+  k.scale = T(1) / T(v.fx * v.fy * v.fz);
+  const T w1 = T(MG_OMEGA1) * k.tab[0], w2 = T(MG_OMEGA2) * k.tab[0], w12 = w1 * w2;
+  k.pre = {w1 + w2 - w12 * k.d, w12 * v.ax, w12 * v.ay, w12 * v.az};
+  k.s1 = {T(1) - w1 * k.d, w1, w1 * v.ax, w1 * v.ay, w1 * v.az};
+  k.s2 = {T(1) - w2 * k.d, w2, w2 * v.ax, w2 * v.ay, w2 * v.az};
+}
 
 // The small levels of the V-cycle, handled by one cluster (pf_coarse.cu): nl
 // levels, those from solo on by the cluster's first block, the coarsest of
@@ -120,8 +168,8 @@ struct SubDesc {
   int off, moff;              // shared memory: element offset of the fields, byte offset of the masks (solo levels)
   float rnx, rny;             // 1 / nx, 1 / ny
   T ax, ay, az;
-  T tab[9];                   // 1/diag with eps = 1, by 3 (kind of the lower z face) + kind of the upper one
-                              // (0 interior, 1 open, 2 electrode)
+  T tab[9], diag[9];          // 1/diag and diag with eps = 1, by the kinds of the z faces (as Bc::itab)
+  T scale;                    // 1 / (fx fy fz)
   T *f, *e, *et;
   const int8_t *tlo, *thi;
   const T *eps, *invd;

@@ -58,15 +58,12 @@ __device__ __forceinline__ T apply_aniso(const Stencil7<T>& s, int dlo, int dhi,
 // the same cell -- the pre-smoother, the residual and their fused form on a
 // split level -- then agree bit for bit.
 __device__ __forceinline__ float rn_add(float a, float b) { return __fadd_rn(a, b); }
-__device__ __forceinline__ float rn_sub(float a, float b) { return __fsub_rn(a, b); }
 __device__ __forceinline__ float rn_mul(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ float rn_fma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double rn_add(double a, double b) { return __dadd_rn(a, b); }
-__device__ __forceinline__ double rn_sub(double a, double b) { return __dsub_rn(a, b); }
 __device__ __forceinline__ double rn_mul(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ double rn_fma(double a, double b, double c) { return __fma_rn(a, b, c); }
 
-//
 // The operator is taken as d c - S, d the diagonal (constant away from the z
 // faces) and S the weighted sum of the neighbours, with a sweep's constants
 // folded into the weights: seven to eight operations a cell and sweep instead
@@ -78,46 +75,23 @@ __device__ __forceinline__ T nb_int(T xm, T xp, T ym, T yp, T zm, T zp, T kx, T 
   return rn_fma(kx, rn_add(xm, xp), rn_fma(ky, rn_add(ym, yp), rn_fma(kz, rn_add(zm, zp), base)));
 }
 
-// A sweep out = c + w D^-1 (f - A c) with D constant: out = kc c + kf f + S(kx, ky, kz).
+// A sweep, both pre-sweeps and the residual there (constants: LevelK).
 template <typename T>
-struct SweepK {
-  T kc, kf, kx, ky, kz;
-  // w: the weight over the diagonal
-  __device__ __forceinline__ SweepK(T w, T ax, T ay, T az)
-      : kc(rn_fma(-w, T(2) * (ax + ay + az), T(1))), kf(w), kx(w * ax), ky(w * ay), kz(w * az) {}
-};
-template <typename T>
-__device__ __forceinline__ T sweep_int(const SweepK<T>& k, T f, T c, T xm, T xp, T ym, T yp, T zm, T zp) {
+__device__ __forceinline__ T sweep_int(const typename LevelK<T>::Sweep& k, T f, T c, T xm, T xp, T ym, T yp, T zm,
+                                       T zp) {
   return nb_int(xm, xp, ym, yp, zm, zp, k.kx, k.ky, k.kz, rn_fma(k.kf, f, rn_mul(k.kc, c)));
 }
 template <typename T>
-__device__ __forceinline__ T sweep_int(const SweepK<T>& k, T f, const Stencil7<T>& s) {
-  return sweep_int(k, f, s.c, s.xm, s.xp, s.ym, s.yp, s.zm, s.zp);
+__device__ __forceinline__ T sweep_int(const typename LevelK<T>::Sweep& k, T f, const Stencil7<T>& s) {
+  return sweep_int<T>(k, f, s.c, s.xm, s.xp, s.ym, s.yp, s.zm, s.zp);
 }
-
-// f - A c.
+template <typename T>
+__device__ __forceinline__ T pre_int(const typename LevelK<T>::Pre& k, T c, T xm, T xp, T ym, T yp, T zm, T zp) {
+  return nb_int(xm, xp, ym, yp, zm, zp, k.kx, k.ky, k.kz, rn_mul(k.kf, c));
+}
 template <typename T>
 __device__ __forceinline__ T res_int(T f, T c, T xm, T xp, T ym, T yp, T zm, T zp, T ax, T ay, T az, T d) {
   return nb_int(xm, xp, ym, yp, zm, zp, ax, ay, az, rn_fma(-d, c, f));
-}
-
-// Two sweeps from zero: e1 = w1 f, e = e1 + w2d (f - A e1) with D constant
-// (w1 = omega1 / d, w2d = omega2 / d): e = (w1 + w2d - w1 w2d d) f + w1 w2d S(f).
-template <typename T>
-struct PreK {
-  T kf, kx, ky, kz;
-  __device__ __forceinline__ PreK(T w1, T w2d, T ax, T ay, T az)
-      : kf(rn_fma(-rn_mul(w1, w2d), T(2) * (ax + ay + az), rn_add(w1, w2d))), kx(rn_mul(w1, w2d) * ax),
-        ky(rn_mul(w1, w2d) * ay), kz(rn_mul(w1, w2d) * az) {}
-};
-template <typename T>
-__device__ __forceinline__ T pre_int(const PreK<T>& k, T c, T xm, T xp, T ym, T yp, T zm, T zp) {
-  return nb_int(xm, xp, ym, yp, zm, zp, k.kx, k.ky, k.kz, rn_mul(k.kf, c));
-}
-
-template <typename T>
-__device__ __forceinline__ T mg_inv_bt(const MgView<T>& L, int xy, int z, T inv_int, const bool bt) {
-  return bt ? mg_inv(L, xy, z, inv_int) : inv_int;
 }
 
 // A v at a level with cell permittivities (v and eps carried together).
@@ -180,9 +154,7 @@ __global__ void __launch_bounds__(MTX* MTY, (sizeof(T) == 4 && !EPS) ? (INT ? 5 
   __shared__ long long tile_slot;
   if (S->done) return;
   constexpr int NH = EPS ? 3 : 1;          // f (, eps, 1/diag)
-  const T om1 = mg_omega1<T>(), om2 = mg_omega2<T>(), inv_int = mg_inv_int(L);
-  const T w1 = rn_mul(om1, inv_int), w2d = rn_mul(om2, inv_int);
-  const PreK<T> pk(w1, w2d, L.ax, L.ay, L.az);
+  const T om1 = mg_omega1<T>(), om2 = mg_omega2<T>(), w1 = L.k.s1.kf;
   const T* hsrc[NH];
   hsrc[0] = L.f;
   if constexpr (EPS) {
@@ -211,27 +183,27 @@ __global__ void __launch_bounds__(MTX* MTY, (sizeof(T) == 4 && !EPS) ? (INT ? 5 
       return e1.c.v + om2 * sr.c.v[2] * (f.c - Ae1);
     } else {
       const bool near = !INT && zfaces && (z == 1 || z == nz - 2);
-      if (!bt && !near) return pre_int(pk, f.c, f.xm, f.xp, f.ym, f.yp, f.zm, f.zp);
+      if (!bt && !near) return pre_int<T>(L.k.pre, f.c, f.xm, f.xp, f.ym, f.yp, f.zm, f.zp);
       Stencil7<T> e1;
-      const T ic = mg_inv(L, xy, z, inv_int);
+      const T ic = mg_inv(L, xy, z);
       e1.c = om1 * ic * f.c;
       if (bt) {
         const int x = xy % nx, rb = xy - x;
         const int xm = rb + (x == 0 ? nx - 1 : x - 1), xp = rb + (x == nx - 1 ? 0 : x + 1);
         const int y = xy / nx;
         const int ym = (y == 0 ? L.g.ny - 1 : y - 1) * nx + x, yp = (y == L.g.ny - 1 ? 0 : y + 1) * nx + x;
-        e1.xm = om1 * mg_inv(L, xm, z, inv_int) * f.xm;
-        e1.xp = om1 * mg_inv(L, xp, z, inv_int) * f.xp;
-        e1.ym = om1 * mg_inv(L, ym, z, inv_int) * f.ym;
-        e1.yp = om1 * mg_inv(L, yp, z, inv_int) * f.yp;
+        e1.xm = om1 * mg_inv(L, xm, z) * f.xm;
+        e1.xp = om1 * mg_inv(L, xp, z) * f.xp;
+        e1.ym = om1 * mg_inv(L, ym, z) * f.ym;
+        e1.yp = om1 * mg_inv(L, yp, z) * f.yp;
       } else {
         e1.xm = w1 * f.xm;
         e1.xp = w1 * f.xp;
         e1.ym = w1 * f.ym;
         e1.yp = w1 * f.yp;
       }
-      e1.zm = f.zb >= 0 ? om1 * mg_inv(L, xy, z - 1, inv_int) * f.zm : T(0);
-      e1.zp = f.za >= 0 ? om1 * mg_inv(L, xy, z + 1, inv_int) * f.zp : T(0);
+      e1.zm = f.zb >= 0 ? om1 * mg_inv(L, xy, z - 1) * f.zm : T(0);
+      e1.zp = f.za >= 0 ? om1 * mg_inv(L, xy, z + 1) * f.zp : T(0);
       e1.zb = f.zb;
       e1.za = f.za;
       const int dlo = (bt && f.zb < 0) ? (int)L.tlo[xy] : 0;
@@ -264,7 +236,7 @@ __global__ void __launch_bounds__(MTX* MTY, (sizeof(T) == 4 && !EPS) ? 4 : 2) k_
   hsrc[0] = L.e;
   if constexpr (EPS) hsrc[1] = L.eps;
   const T* osrc[1] = {L.f};
-  const T scale = T(1) / T(L.fx * L.fy * L.fz), dg = T(2) * (L.ax + L.ay + L.az);
+  const T scale = L.k.scale, dg = L.k.d;
   TileGeo<MTX, MTY, VX> s;
   T racc[VX];
 #pragma unroll
@@ -358,10 +330,9 @@ __global__ void __launch_bounds__(MTX* MTY, 4) k_mg_prr(MgView<float> L, MgView<
   float* const eb = stg + PRR_NS * PRR_STAGE;
   const int nx = L.g.nx, ny = L.g.ny, nz = L.g.nz;
   const long long nxy = L.g.nxy;
-  const float om1 = mg_omega1<float>(), om2 = mg_omega2<float>(), inv_int = mg_inv_int(L);
-  const PreK<float> pk(rn_mul(om1, inv_int), rn_mul(om2, inv_int), L.ax, L.ay, L.az);
-  const float ax = L.ax, ay = L.ay, az = L.az, dg = 2.f * (ax + ay + az);
-  const float scale = 1.0f / float(L.fx * L.fy * L.fz);
+  const LevelK<float>::Pre pk = L.k.pre;
+  const float ax = L.ax, ay = L.ay, az = L.az, dg = L.k.d;
+  const float scale = L.k.scale;
   const int tx = threadIdx.x, ty = threadIdx.y, tid = tx + ty * MTX;
   const int c0 = 4 + 4 * tx;               // column of the own vector in a stage or e plane
   const int so = (ty + 2) * PRR_RS + c0;   // own vector in a stage
@@ -418,7 +389,7 @@ __global__ void __launch_bounds__(MTX* MTY, 4) k_mg_prr(MgView<float> L, MgView<
     // e at a staged cell from the f planes below, at and above it
     auto e_at = [&](const float* sm, const float* sc, const float* sp, int off) -> float {
       const float* q = sc + off;
-      return pre_int(pk, q[0], q[-1], q[1], q[-PRR_RS], q[PRR_RS], sm[off], sp[off]);
+      return pre_int<float>(pk, q[0], q[-1], q[1], q[-PRR_RS], q[PRR_RS], sm[off], sp[off]);
     };
     float em2[4], em1[4], e0[4], racc[4];
 #pragma unroll
@@ -449,7 +420,7 @@ __global__ void __launch_bounds__(MTX* MTY, 4) k_mg_prr(MgView<float> L, MgView<
         if (tx == MTX - 1) fr = sc[so + 4];
 #pragma unroll
         for (int i = 0; i < 4; ++i)
-          e0[i] = pre_int(pk, fc[i], i == 0 ? fl : fc[i - 1], i == 3 ? fr : fc[i + 1], fym[i], fyp[i], fm[i], fp[i]);
+          e0[i] = pre_int<float>(pk, fc[i], i == 0 ? fl : fc[i - 1], i == 3 ? fr : fc[i + 1], fym[i], fyp[i], fm[i], fp[i]);
       }
       // planes whose residual this tile forms: e on the own vector and the ring
       if (u >= 1 && u <= nt) {
@@ -544,9 +515,7 @@ __global__ void __launch_bounds__(MTX* MTY, 3) k_mg_pp(MgView<float> L, MgView<f
   float* const eb = stg + PP_NS * PP_STAGE;
   const int nx = L.g.nx, ny = L.g.ny, nz = L.g.nz, cnx = C.g.nx, cny = C.g.ny;
   const long long nxy = L.g.nxy, cnxy = C.g.nxy;
-  const float inv_int = mg_inv_int(L);
-  const SweepK<float> k2(rn_mul(mg_omega2<float>(), inv_int), L.ax, L.ay, L.az);
-  const SweepK<float> k1(rn_mul(mg_omega1<float>(), inv_int), L.ax, L.ay, L.az);
+  const LevelK<float>::Sweep k1 = L.k.s1, k2 = L.k.s2;
   const int tx = threadIdx.x, ty = threadIdx.y, tid = tx + ty * MTX;
   const int c0 = 4 + 4 * tx;
   const int so = (ty + 2) * PRR_RS + c0;   // own vector in a staged field plane
@@ -629,7 +598,7 @@ __global__ void __launch_bounds__(MTX* MTY, 3) k_mg_pp(MgView<float> L, MgView<f
     };
     // e' at staged cell (r, c) from the stages of the planes below, at and above it
     auto ep_at = [&](const float* sm, const float* sc, const float* sp, int r, int c) -> float {
-      return sweep_int(k2, sc[PRR_STAGE + r * PRR_RS + c], u_at(sc, r, c), u_at(sc, r, c - 1), u_at(sc, r, c + 1),
+      return sweep_int<float>(k2, sc[PRR_STAGE + r * PRR_RS + c], u_at(sc, r, c), u_at(sc, r, c - 1), u_at(sc, r, c + 1),
                        u_at(sc, r - 1, c), u_at(sc, r + 1, c), u_at(sm, r, c), u_at(sp, r, c));
     };
     float em2[4], e0[4];
@@ -675,7 +644,7 @@ __global__ void __launch_bounds__(MTX* MTY, 3) k_mg_pp(MgView<float> L, MgView<f
         for (int i = 0; i < 4; ++i) {
           const float ym = eym[i] + (i < 2 ? pYM.x : pYM.y), yp = eyp[i] + (i < 2 ? pYP.x : pYP.y);
           const float zm = ezm[i] + (i < 2 ? pZM.x : pZM.y), zp = ezp[i] + (i < 2 ? pZP.x : pZP.y);
-          e0[i] = sweep_int(k2, fc[i], uc[i], i == 0 ? uL : uc[i - 1], i == 3 ? uR : uc[i + 1], ym, yp, zm, zp);
+          e0[i] = sweep_int<float>(k2, fc[i], uc[i], i == 0 ? uL : uc[i - 1], i == 3 ? uR : uc[i + 1], ym, yp, zm, zp);
         }
       }
       if (u >= 1 && u <= nt) {
@@ -696,7 +665,7 @@ __global__ void __launch_bounds__(MTX* MTY, 3) k_mg_pp(MgView<float> L, MgView<f
         if (tx == MTX - 1) er = ebm[eo + 4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-          ev[i] = sweep_int(k1, fv[i], ec[i], i == 0 ? el : ec[i - 1], i == 3 ? er : ec[i + 1], eym[i], eyp[i], em2[i],
+          ev[i] = sweep_int<float>(k1, fv[i], ec[i], i == 0 ? el : ec[i - 1], i == 3 ? er : ec[i + 1], eym[i], eyp[i], em2[i],
                             e0[i]);
           arz.add(fv[i], ev[i]);
         }
@@ -726,8 +695,7 @@ __global__ void __launch_bounds__(MTX* MTY, (sizeof(T) == 4 && !EPS) ? 3 : 2) k_
   if (S->done) return;
   constexpr int NH = EPS ? 2 : 1;          // e (, eps); the parents come as field NH
   constexpr int NO = EPS ? 2 : 1;          // f (, 1/diag)
-  const T om = mg_omega2<T>(), inv_int = mg_inv_int(L);
-  const SweepK<T> sk(rn_mul(om, inv_int), L.ax, L.ay, L.az);
+  const T om = mg_omega2<T>();
   const T* hsrc[NH];
   hsrc[0] = L.e;
   if constexpr (EPS) hsrc[1] = L.eps;
@@ -762,9 +730,9 @@ __global__ void __launch_bounds__(MTX* MTY, (sizeof(T) == 4 && !EPS) ? 3 : 2) k_
       const T Ae = apply_aniso_eps(se, dlo, dhi, L.ax, L.ay, L.az, bt);
       return st.c + om * o[1] * (o[0] - Ae);
     } else {
-      if (!bt) return sweep_int(sk, o[0], st);
+      if (!bt) return sweep_int<T>(L.k.s2, o[0], st);
       const T Ae = apply_aniso(st, dlo, dhi, L.ax, L.ay, L.az, bt);
-      return st.c + om * mg_inv_bt(L, xy, z, inv_int, bt) * (o[0] - Ae);
+      return st.c + om * mg_inv(L, xy, z) * (o[0] - Ae);
     }
   };
   auto post = [&](int z, const T (&ov)[VX]) { store_n<T, VX>(L.et + (long long)z * L.g.nxy + s.xy, ov); };
@@ -789,8 +757,7 @@ __global__ void __launch_bounds__(MTX* MTY, (sizeof(T) == 4 && !EPS) ? (INT ? 5 
   if (S->done) return;
   constexpr int NH = EPS ? 2 : 1;          // et (, eps)
   constexpr int NO = EPS ? 2 : 1;          // f (, 1/diag)
-  const T om = mg_omega1<T>(), inv_int = mg_inv_int(L);
-  const SweepK<T> sk(rn_mul(om, inv_int), L.ax, L.ay, L.az);
+  const T om = mg_omega1<T>();
   const T* hsrc[NH];
   hsrc[0] = L.et;
   if constexpr (EPS) hsrc[1] = L.eps;
@@ -810,10 +777,10 @@ __global__ void __launch_bounds__(MTX* MTY, (sizeof(T) == 4 && !EPS) ? (INT ? 5 
     } else {
       const Stencil7<T> st = pick(sr, 0);
       if (!bt) {
-        e = sweep_int(sk, o[0], st);
+        e = sweep_int<T>(L.k.s1, o[0], st);
       } else {
         const T Ae = apply_aniso(st, dlo, dhi, L.ax, L.ay, L.az, bt);
-        e = st.c + om * mg_inv_bt(L, xy, z, inv_int, bt) * (o[0] - Ae);
+        e = st.c + om * mg_inv(L, xy, z) * (o[0] - Ae);
       }
     }
     if (LAST) arz.add(o[0], e);
@@ -1004,14 +971,16 @@ static void post2_l(const LaunchCfg& L, const MgView<T>& lv, double* part, Scala
 // so it is never split.
 template <typename T, bool LAST, int VX, bool E>
 static int post2_v(const LaunchCfg& L, const MgView<T>& lv, double* part, Scalars* S) {
-  MgView<T> vi, vb;
-  if (LAST || !split_views(lv, vi, vb)) {
-    post2_l<T, LAST, VX, E, false>(L, lv, part, S);
-    return 1;
+  if constexpr (!LAST) {
+    MgView<T> vi, vb;
+    if (split_views(lv, vi, vb)) {
+      post2_l<T, LAST, VX, E, true>(L, vi, part, S);
+      post2_l<T, LAST, VX, E, false>(L, vb, part, S);
+      return 2;
+    }
   }
-  post2_l<T, LAST, VX, E, true>(L, vi, part, S);
-  post2_l<T, LAST, VX, E, false>(L, vb, part, S);
-  return 2;
+  post2_l<T, LAST, VX, E, false>(L, lv, part, S);
+  return 1;
 }
 
 constexpr int vec_of(size_t bytes) { return (int)(16 / bytes); }

@@ -123,6 +123,7 @@ pf_status solve(const pf_params* prm, cudaStream_t st, char* base, const Layout&
   d.bc.thi = (const int8_t*)(base + Ly.thi);
   d.bc.vlo = (const T*)(base + Ly.vlo);
   d.bc.vhi = (const T*)(base + Ly.vhi);
+  pf::diag_table<T>(g.ih2, d.bc.itab);
   d.part = (double*)(base + Ly.part);
   d.S = (pf::Scalars*)(base + Ly.S);
 

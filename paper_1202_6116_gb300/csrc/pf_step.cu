@@ -126,7 +126,7 @@ __global__ void __launch_bounds__(MTX* MTY) k_rhs(Geo g, Bc<T> bc, const T* __re
   constexpr int NO = EPS ? 1 : 0;     // (1/diag)
   constexpr int NV = MEAN ? 1 : 3;
   const T mb = MEAN ? T(0) : T(S->mean_b);
-  const T inv6 = T(1) / (T(6) * T(g.ih2));
+  const T inv6 = bc.itab[0];
   const T ih = T(g.ih), ih2 = T(g.ih2);
   const T* hsrc[NH];
   hsrc[0] = P;
@@ -250,7 +250,7 @@ __global__ void __launch_bounds__(MTX* MTY, RW_D == 1 ? 3 : 2) k_rhs_w(Geo g, Bc
   const float* const Py = P + g.n;
   const float* const Pz = P + 2 * g.n;
   const float mb = float(S->mean_b);
-  const float inv6 = 1.0f / (6.0f * float(g.ih2));
+  const float inv6 = bc.itab[0];
   const float ih = float(g.ih), ih2 = float(g.ih2);
   const int tx = threadIdx.x, ty = threadIdx.y, tid = tx + ty * MTX;
   // own vector in each region of a stage
