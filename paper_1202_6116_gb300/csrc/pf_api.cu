@@ -164,6 +164,7 @@ void mg_tail_layout(Layout& L, size_t word) {
   L.tail0 = k0;
   L.tail.nl = (int)(nl - k0);
   L.tail.solo = (int)(b0 - k0);
+  L.tail.cells = (int)L.mg[k0].n();
   L.tail.coarse = (int)L.mg[nl - 1].n();
   L.tail.blob_bytes = (int)up16((nl - k0) * desc + mb);
   L.tail.smem_bytes = L.tail.blob_bytes + (int)fb;

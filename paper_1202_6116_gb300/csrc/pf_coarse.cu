@@ -576,7 +576,14 @@ static cudaError_t mg_sub_t(const LaunchCfg& L, const MgTail& t, const void* blo
     }
     cluster = c;
   }
-  const int nc = (t.solo > 0 || t.coarse > SUB_ROWS) ? cluster : 1;
+  int nc = (t.solo > 0 || t.coarse > SUB_ROWS) ? cluster : 1;
+  // FP32: no more blocks than its first level has 16-byte vectors for, but at
+  // least 8.  A block holds its SM's registers while the first one runs the
+  // solo levels: a batch of 30 films 17.15 ms with 16 blocks for every film,
+  // 16.65 so (and 16.14 with 8 for every film, but then a film alone whose first
+  // level has 65 536 cells pays 6 %).  FP64 levels are bound by the SMs' FP64
+  // units: 8 blocks for 16 384 cells were 3 % slower.
+  while (sizeof(T) == 4 && nc > 8 && t.cells <= (nc / 2) * NT * (int)(16 / sizeof(T))) nc /= 2;
   cfg.gridDim = dim3(nc);
   at.val.clusterDim.x = nc;
   cfg.dynamicSmemBytes = t.smem_bytes;

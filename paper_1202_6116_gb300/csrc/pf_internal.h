@@ -156,6 +156,7 @@ inline void sweep_constants(MgView<T>& v) {
 // coarse cells.
 struct MgTail {
   int nl, solo, coarse;
+  int cells;                  // of the first one
   int blob_bytes;             // descriptors and solo masks, a multiple of 16
   int smem_bytes;             // the blob, then the solo levels' f, e, e_tmp
 };
