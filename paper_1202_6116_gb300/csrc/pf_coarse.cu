@@ -126,8 +126,15 @@ __device__ __forceinline__ void sub_res(const SubDesc<T>& L, const int8_t* lo, c
 #pragma unroll
     for (int i = 0; i < VX; ++i) {
       const T v = vc[i], e = ec[i];
-      const T sx = hmean2(e, i == 0 ? el : ec[i - 1]) * (v - (i == 0 ? vl : vc[i - 1])) -
-                   hmean2(e, i == VX - 1 ? er : ec[i + 1]) * ((i == VX - 1 ? vr : vc[i + 1]) - v);
+      const T eb = i == 0 ? el : ec[i - 1], ea = i == VX - 1 ? er : ec[i + 1];
+      const T vb = i == 0 ? vl : vc[i - 1], va = i == VX - 1 ? vr : vc[i + 1];
+      if (s.zm >= 0 && s.zp >= 0 &&
+          (eb == e) & (ea == e) & (eym[i] == e) & (eyp[i] == e) & (ezm[i] == e) & (ezp[i] == e)) {   // see one_eps
+        out[i] = fc[i] - e * (L.ax * ((v - vb) - (va - v)) + L.ay * ((v - ym[i]) - (yp[i] - v)) +
+                              L.az * ((v - zm[i]) - (zp[i] - v)));
+        continue;
+      }
+      const T sx = hmean2(e, eb) * (v - vb) - hmean2(e, ea) * (va - v);
       const T sy = hmean2(e, eym[i]) * (v - ym[i]) - hmean2(e, eyp[i]) * (yp[i] - v);
       T sz = T(0);
       if (s.zm >= 0) sz += hmean2(e, ezm[i]) * (v - zm[i]);

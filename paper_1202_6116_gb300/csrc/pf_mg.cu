@@ -99,6 +99,9 @@ template <typename T>
 __device__ __forceinline__ T apply_aniso_eps(const Stencil7<EpsVal<T>>& s, int dlo, int dhi, T ax, T ay, T az,
                                              const bool bt) {
   const T ec = s.c.e, vc = s.c.v;
+  if (!bt && one_eps(s))
+    return ec * (ax * ((vc - s.xm.v) - (s.xp.v - vc)) + ay * ((vc - s.ym.v) - (s.yp.v - vc)) +
+                 az * ((vc - s.zm.v) - (s.zp.v - vc)));
   const T sx = hmean2(ec, s.xm.e) * (vc - s.xm.v) - hmean2(ec, s.xp.e) * (s.xp.v - vc);
   const T sy = hmean2(ec, s.ym.e) * (vc - s.ym.v) - hmean2(ec, s.yp.e) * (s.yp.v - vc);
   T sz = T(0);

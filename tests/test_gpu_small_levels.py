@@ -95,3 +95,31 @@ def test_cg_loop_matches_the_two_kernel_iteration(precision, shape, faces):
     assert abs(info["last_iters"] - info_ref["last_iters"]) <= max(2, info_ref["last_iters"] // 50)
     # the whole loop is one launch
     assert info["kernel_launches"] <= 5 < info_ref["kernel_launches"] or shape == (1, 1, 1)
+
+
+@pytest.mark.parametrize("shape", [(32, 32, 16), (32, 32, 32), (64, 64, 32), (64, 64, 36)])
+def test_small_levels_fp32_by_cluster_size(shape):
+    """First levels of 16 384 cells (8 blocks) and just above (16), as the finest level and below it: potentials
+    within the FP32 parity bar of the oracle."""
+    w = mixed_workload(*shape, 65, precision="fp32", rtol=1e-7).with_(solver="mg", maxit=300)
+    phio, st, _, _ = O.solve_potential(oracle_grid(w), w.P0, rtol=1e-14)
+    assert st == O.OK
+    phi, info = solve(w)
+    assert relerr(phi, phio) <= 1e-4
+    assert info["last_iters"] <= 30
+
+
+@pytest.mark.parametrize("solver", ["pcg", "mg"])
+@pytest.mark.parametrize("shape", [(32, 24, 13), (37, 22, 11), (64, 32, 16)])
+def test_patchwork_permittivity_matches_oracle(solver, shape):
+    """Blocks of two permittivities: cells whose six neighbours share theirs (no harmonic mean formed) beside cells
+    whose neighbours do not, within one warp.  FP64 bar 1e-10 as in the parity tests."""
+    if solver == "mg" and shape[0] % 2:
+        shape = (40, 24, 12)
+    w = mixed_workload(*shape, 66).with_(solver=solver, maxit=3000, rtol=1e-13)
+    z, y, x = np.meshgrid(*(np.arange(n) for n in w.shape), indexing="ij")
+    w = w.with_(eps=np.where((x // 7 + y // 5 + z // 4) % 2, 30.0, 1.0))
+    phio, st, _, _ = O.solve_potential(oracle_grid(w), w.P0, rtol=1e-14)
+    assert st == O.OK
+    phi, _ = solve(w)
+    assert relerr(phi, phio) <= 1e-10
