@@ -118,7 +118,7 @@ k_cg_loop(Geo g, Bc<T> bc, T* r, T* p0, T* p1, T* q, T* x, double* part, Scalars
   const long long nxy = g.nxy;
   const T ih2 = T(g.ih2);
   const T inv6 = bc.itab[0];
-  auto inv_at = [&](int xy, int z) -> T { return inv_diag_unit(g, bc, xy, z, inv6); };
+  auto inv_at = [&](int xy, int z) -> T { return inv_diag_tab(g, bc, xy, z, inv6); };
   const double rtol = S->rtol, bnorm = S->bnorm;
   const int maxit = S->maxit;
   double rz = S->rz, rr = 0.0, rel = S->last_rel, alpha = 0.0;
