@@ -20,9 +20,13 @@ constexpr int MG_MAX_LEVELS = 24;
 constexpr int MG_MAX_COARSE = 1024;   // cells of the coarsest multigrid level (solved by its inverse)
 // The V-cycle's small levels run as one cluster launch (pf_coarse.cu): from
 // the first level of at most mg_sub_cells on; its levels of at most
-// mg_solo_cells in one block of the cluster.
+// mg_solo_cells in one block of the cluster.  FP32 from 131 072 cells on: no
+// faster on films, from 524 288 much slower (16 SMs); solo from 4096 / 1024 / 256
+// cells: the air film of 512 x 512 x 37 15.86 / 15.69 / 15.76 ms per 4 steps,
+// 336 x 216 x 32 predictor-corrector 6.95 / 6.88 / 6.89, a batch of 30 films 16.68
+// / 16.58 / 16.66.
 inline long long mg_sub_cells(size_t word) { return word == 4 ? 65536 : 16384; }
-inline long long mg_solo_cells(size_t word) { return word == 4 ? 4096 : 256; }
+inline long long mg_solo_cells(size_t word) { return word == 4 ? 1024 : 256; }
 constexpr int MG_TAIL_LEVELS = 24;
 constexpr int MG_TAIL_SMEM = 192 * 1024;   // shared-memory limit of the solo levels' arrays (bytes)
 // A multigrid sweep over a large level whose z faces are not periodic runs as
