@@ -355,7 +355,13 @@ inline MarchCfg march_cfg(int nx, int ny, int nz, int nsm, int occ, int tzmax, b
   for (int tz = std::min(tzmax, nz); tz >= 1; --tz) {
     if (even_tz && (tz & 1)) continue;
     const int chunks = (nz + tz - 1) / tz;
-    if (chunks > 128) break;
+    if (chunks > 128) {          // march_cost is a sum over the chunks: very tall grids take a plain rule
+      if (best == 0.0) {
+        m.tz = tz;
+        while (m.tz > 2 && cols * ((nz + m.tz - 1) / m.tz) < 3LL * nsm * occ) m.tz = m.tz / 4 * 2;
+      }
+      break;
+    }
     // of the depths with this many chunks: the deepest, the even split, multiples of 8
     if (chunks == last && (nz + chunks - 1) / chunks != tz && tz % 8 != 0) continue;
     last = chunks;

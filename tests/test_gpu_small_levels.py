@@ -11,7 +11,7 @@ from paper_1202_6116_gb300 import build as B
 from paper_1202_6116_gb300 import pf
 from paper_1202_6116_gb300.film import Film
 
-from helpers import mixed_workload, oracle_grid, relerr
+from helpers import mixed_workload, oracle_grid, oracle_params, relerr
 
 pytestmark = pytest.mark.gpu
 
@@ -123,3 +123,22 @@ def test_patchwork_permittivity_matches_oracle(solver, shape):
     assert st == O.OK
     phi, _ = solve(w)
     assert relerr(phi, phio) <= 1e-10
+
+
+@pytest.mark.parametrize("precision,tol", [("fp64", 1e-12), ("fp32", 1e-5)])
+@pytest.mark.parametrize("nz", [8192, 8193])
+def test_tall_grids_match_oracle(nz, precision, tol):
+    """More than 128 tiles of the largest depth in z (64 planes), and just fewer: the plain rule of the
+    tile depth.  Sums over the grid with the bars of the diagnostics' tests."""
+    w = mixed_workload(4, 4, nz, 67, precision=precision, amp=0.7)
+    f = Film(w)
+    f.phi.copy_(0.3 * f.P[0] + 0.1 * f.P[2])
+    P, phi = f.numpy()
+    d = f.diagnostics(0.3)
+    f.close()
+    o = O.diagnostics(oracle_grid(w), oracle_params(w), P, phi, 0.3)
+    assert d["switched_fraction"] == o["switched_fraction"]
+    for k in ("mean_px", "mean_py", "mean_pz"):
+        assert abs(d[k] - o[k]) <= tol * np.abs(P).max()
+    for k in ("f_landau", "f_grad", "f_elec"):
+        assert abs(d[k] - o[k]) <= tol * abs(o[k])
