@@ -54,6 +54,7 @@ struct LaunchCfg {
                        // (tiled = 1), or the default of the CG operator
   int tiled;           // 1: a tiling was set (pf_set_tiling); 0: every kernel plans its own
   int nsm, word, nx, ny, nz;
+  int loop_share = 1;  // virtual blocks per block of the persistent Jacobi-PCG loop (films of a batch: see pf_cgloop.cu)
   mutable MarchCfg plan[2][PLAN_OCC];   // planned tilings (ntiles = 0: not yet), see kernel_tiling
   int flat_grid;       // flat vector kernels (FLAT_THREADS blocks, grid-stride)
   cudaStream_t stream;
