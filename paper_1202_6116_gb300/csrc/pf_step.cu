@@ -434,12 +434,19 @@ __global__ void __launch_bounds__(MTX* MTY, RW_D == 1 ? 3 : 2) k_rhs_w(Geo g, Bc
   rhs_close<3, false, true>(g, part, S, mc.ntiles, cond, use_cond, smem);
 }
 
-// Coefficients of an increment dt L (-df/dP + g Lap P + E), with dt L and the
-// grid factors folded in (formed in FP64, rounded once):
-//   P_i (c1 + c12 (P_x^2 + P_y^2 + P_z^2) + cd P_i^2) + gl (neighbour differences) + el (phi difference).
+// Coefficients of an increment dt L (-df/dP + g Lap P + E), formed in FP64 and
+// rounded once:
+//   m (P_i (c1 + c12 (P_x^2 + P_y^2 + P_z^2) + cd P_i^2) + gl (neighbour differences) + el (phi difference)).
+// FP64 folds dt L into them (m = 1, not applied).  FP32 keeps m = dt L apart,
+// for three products a cell: its rounding scales time by 3e-8 and no more, while
+// folded coefficients are each off by as much, which shifts the energy's balance
+// (-2 a1 and the like are mostly exact).  A 256 x 256 x 64 strip film over 5000
+// steps peaked at 1.5e-4 from FP64 with folded coefficients, at 5e-5 with every
+// term written out and dt L apart.
 template <typename T>
 struct Coef {
-  T c1, c12, cd, gl, el;         // -2 a1, -2 a12, -(4 a11 - 2 a12), g/dx^2, -1/(2 dx), each times dt L
+  T c1, c12, cd, gl, el;         // -2 a1, -2 a12, -(4 a11 - 2 a12), g/dx^2, -1/(2 dx) (FP64: each times dt L)
+  T m;                           // dt L
   T amp;                         // thermal random force: sigma sqrt(dt) (0: off)
   unsigned long long seed;
   long long* step;               // device step counter (steps since pf_bind)
@@ -512,7 +519,7 @@ __device__ __forceinline__ void two_sum(T a, T b, T& s, T& e) {
 // in v[3]); zb / za < 0 mark a z face (Neumann P, the face value of phi: mean
 // inside, V at an electrode, phi_cell at an open face, so that the difference
 // of the two face values is formed doubled, 2 V or 2 phi_cell at a face).
-// 52 operations a cell in FP32 where the terms written out took 84: FP32 is
+// 55 operations a cell in FP32 where the terms written out took 84: FP32 is
 // bound by issue, FP64 by its unit.  The FP32 Laplacian sums differences (they
 // are nearly exact, and the compensated state keeps what they resolve; a
 // difference between two cells of a vector serves both); the FP64 one takes
@@ -556,6 +563,7 @@ __device__ __forceinline__ void tdgl_inc(const Stencil7<Raw<T, 4>>& st, int xy, 
       if (hi) lap += st.zp.v[i] - p[i];
     }
     inc[i] = p[i] * (a + k.cd * p2[i]) + (k.gl * lap + k.el * dphi[i]);
+    if constexpr (sizeof(T) == 4) inc[i] *= k.m;
   }
 }
 
@@ -989,12 +997,13 @@ static void tdgl_v(const LaunchCfg& L, const Geo& g, const Dev<T>& d, const T* P
 template <typename T>
 void launch_tdgl(const LaunchCfg& L, const Geo& g, const Dev<T>& d, const T* P, T* Pn, const double* coef,
                  int corr, const Noise& nz) {
-  const double dtL = coef[4];
+  const double dtL = sizeof(T) == 8 ? coef[4] : 1.0;
   const Coef<T> k{T(-2.0 * coef[0] * dtL),
                   T(-2.0 * coef[2] * dtL),
                   T((2.0 * coef[2] - 4.0 * coef[1]) * dtL),
                   T(coef[3] * g.ih2 * dtL),
                   T(-0.5 * g.ih * dtL),
+                  T(coef[4]),
                   T(nz.amp),
                   nz.seed,
                   nz.step,
