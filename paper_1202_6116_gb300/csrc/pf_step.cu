@@ -436,16 +436,21 @@ __global__ void __launch_bounds__(MTX* MTY, RW_D == 1 ? 3 : 2) k_rhs_w(Geo g, Bc
 
 // Coefficients of an increment dt L (-df/dP + g Lap P + E), formed in FP64 and
 // rounded once:
-//   m (P_i (c1 + c12 (P_x^2 + P_y^2 + P_z^2) + cd P_i^2) + gl (neighbour differences) + el (phi difference)).
+//   m (P_i (c1 + c11 P_i^2 + c12 (P_j^2 + P_k^2)) + gl (neighbour differences) + el (phi difference)).
+// -2 a1, -4 a11 and the like are mostly exact and stay apart, and so does the sum
+// of the other two squares: taken as c12 (P_x^2 + P_y^2 + P_z^2) + cd P_i^2, three
+// operations a cell fewer, the quartic coefficient along an axis is the sum of
+// two rounded numbers.  In FP32 that left a mean error of 3e-8 in the force near
+// a pole (4e-10 as written here), which the compensated state collects step after
+// step: a 256 x 256 x 64 strip film over 5000 steps peaked at 1.8e-4 from FP64 that
+// way and at 4.2e-5 this way (medians over eleven solve tolerances from 0.7e-8 to
+// 1.5e-8: 1.5e-4 and 6e-5).
 // FP64 folds dt L into them (m = 1, not applied).  FP32 keeps m = dt L apart,
 // for three products a cell: its rounding scales time by 3e-8 and no more, while
-// folded coefficients are each off by as much, which shifts the energy's balance
-// (-2 a1 and the like are mostly exact).  A 256 x 256 x 64 strip film over 5000
-// steps peaked at 1.5e-4 from FP64 with folded coefficients, at 5e-5 with every
-// term written out and dt L apart.
+// folded coefficients are each off by as much.
 template <typename T>
 struct Coef {
-  T c1, c12, cd, gl, el;         // -2 a1, -2 a12, -(4 a11 - 2 a12), g/dx^2, -1/(2 dx) (FP64: each times dt L)
+  T c1, c11, c12, gl, el;        // -2 a1, -4 a11, -2 a12, g/dx^2, -1/(2 dx) (FP64: each times dt L)
   T m;                           // dt L
   T amp;                         // thermal random force: sigma sqrt(dt) (0: off)
   unsigned long long seed;
@@ -519,7 +524,7 @@ __device__ __forceinline__ void two_sum(T a, T b, T& s, T& e) {
 // in v[3]); zb / za < 0 mark a z face (Neumann P, the face value of phi: mean
 // inside, V at an electrode, phi_cell at an open face, so that the difference
 // of the two face values is formed doubled, 2 V or 2 phi_cell at a face).
-// 55 operations a cell in FP32 where the terms written out took 84: FP32 is
+// 58 operations a cell in FP32 where the terms written out took 84: FP32 is
 // bound by issue, FP64 by its unit.  The FP32 Laplacian sums differences (they
 // are nearly exact, and the compensated state keeps what they resolve; a
 // difference between two cells of a vector serves both); the FP64 one takes
@@ -541,9 +546,10 @@ __device__ __forceinline__ void tdgl_inc(const Stencil7<Raw<T, 4>>& st, int xy, 
   const bool lo = st.zb >= 0, hi = st.za >= 0 && (z + 1 < g.zair || g.zair == g.nz);   // free surface under air
   const T p[3] = {st.c.v[0], st.c.v[1], st.c.v[2]};
   const T p2[3] = {p[0] * p[0], p[1] * p[1], p[2] * p[2]};
-  const T a = k.c1 + k.c12 * (p2[0] + p2[1] + p2[2]);
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
+    const int j = (i + 1) % 3, l = (i + 2) % 3;
+    const T a = fma(k.c12, fma(p[j], p[j], p2[l]), fma(k.c11, p2[i], k.c1));
     T lap;
     if constexpr (sizeof(T) == 8) {
       lap = (st.xm.v[i] + st.xp.v[i]) + (st.ym.v[i] + st.yp.v[i]);
@@ -562,7 +568,7 @@ __device__ __forceinline__ void tdgl_inc(const Stencil7<Raw<T, 4>>& st, int xy, 
       if (lo) lap += st.zm.v[i] - p[i];
       if (hi) lap += st.zp.v[i] - p[i];
     }
-    inc[i] = p[i] * (a + k.cd * p2[i]) + (k.gl * lap + k.el * dphi[i]);
+    inc[i] = p[i] * a + (k.gl * lap + k.el * dphi[i]);
     if constexpr (sizeof(T) == 4) inc[i] *= k.m;
   }
 }
@@ -999,8 +1005,8 @@ void launch_tdgl(const LaunchCfg& L, const Geo& g, const Dev<T>& d, const T* P, 
                  int corr, const Noise& nz) {
   const double dtL = sizeof(T) == 8 ? coef[4] : 1.0;
   const Coef<T> k{T(-2.0 * coef[0] * dtL),
+                  T(-4.0 * coef[1] * dtL),
                   T(-2.0 * coef[2] * dtL),
-                  T((2.0 * coef[2] - 4.0 * coef[1]) * dtL),
                   T(coef[3] * g.ih2 * dtL),
                   T(-0.5 * g.ih * dtL),
                   T(coef[4]),

@@ -1,0 +1,62 @@
+"""Rounding of one TDGL update against the same step in extended precision,
+on states whose potential is exactly zero: each component of P depends on the
+two coordinates across it, so div P = 0 in every cell of a periodic film."""
+import numpy as np
+import pytest
+import torch
+
+from paper_1202_6116_gb300 import build as B
+from paper_1202_6116_gb300 import pf
+from paper_1202_6116_gb300 import workloads as W
+from paper_1202_6116_gb300.film import Film
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    B.build()
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    pf.lib()
+
+
+def divergence_free(nx, ny, nz, mean, amp, seed, dtype):
+    """mean + amp U[-1, 1] per component, constant along its own axis, representable in dtype."""
+    rng = np.random.default_rng(seed)
+    u = [rng.uniform(-1, 1, s) for s in ((nz, ny, 1), (nz, 1, nx), (1, ny, nx))]
+    return np.stack([np.broadcast_to((m + amp * v).astype(dtype), (nz, ny, nx)) for m, v in zip(mean, u)]).astype(float)
+
+
+def one_step(P0, precision, **coeffs):
+    _, nz, ny, nx = P0.shape
+    z8, z = np.zeros((ny, nx), np.int8), np.zeros((ny, nx))
+    w = W.Workload("update", nx, ny, nz, P0, z8, z, z8, z, precision=precision, periodic_z=True, rtol=1e-7, **coeffs)
+    f = Film(w)
+    f.step(1)
+    P, phi = f.numpy()
+    f.close()
+    assert (phi == 0.0).all()
+    return P
+
+
+def landau(P, a1, a11, a12):
+    p2 = P * P
+    return -(2 * a1 * P + 4 * a11 * P * p2 + 2 * a12 * P * (p2.sum(0) - p2))
+
+
+@pytest.mark.parametrize("axis", [0, 1, 2])
+def test_fp32_landau_force_has_no_bias_at_a_pole(axis):
+    """Mean error of the force over thousands of states next to P = 1 along one
+    axis, with dt L = 1024 so that the updated P shows the force itself.  One
+    value's error is at most a few half-ulps of the terms of size 2 (rms 6e-8),
+    plus the rounding of P of size 40 / 1024: its mean over 4096 independent
+    values scatters by 1e-9.  A coefficient off by one rounding shifts it by 3e-8."""
+    mean = [0.0] * 3
+    mean[axis] = 1.0
+    n = [64, 64, 64]
+    n[axis] = 4                                     # the biased component varies over the other two axes
+    P0 = divergence_free(*n, mean, 0.01, 5 + axis, np.float32)
+    P = one_step(P0, "fp32", g=0.0, dt=1024.0)
+    err = (P[axis] - P0[axis]) / 1024.0 - landau(P0, -1.0, 0.5, 0.8)[axis]
+    assert abs(err.mean()) <= 1e-8
+    assert np.abs(err).max() <= 5e-7
