@@ -445,13 +445,13 @@ __global__ void __launch_bounds__(MTX* MTY, RW_D == 1 ? 3 : 2) k_rhs_w(Geo g, Bc
 // step: a 256 x 256 x 64 strip film over 5000 steps peaked at 1.8e-4 from FP64 that
 // way and at 4.2e-5 this way (medians over eleven solve tolerances from 0.7e-8 to
 // 1.5e-8: 1.5e-4 and 6e-5).
-// FP64 folds dt L into them (m = 1, not applied).  FP32 keeps m = dt L apart,
-// for three products a cell: its rounding scales time by 3e-8 and no more, while
-// folded coefficients are each off by as much.
+// m = dt L stays apart too: its rounding scales time and no more, while
+// coefficients that hold it are each off by as much.
 template <typename T>
 struct Coef {
-  T c1, c11, c12, gl, el;        // -2 a1, -4 a11, -2 a12, g/dx^2, -1/(2 dx) (FP64: each times dt L)
+  T c1, c11, c12, gl, el;        // -2 a1, -4 a11, -2 a12, g/dx^2, -1/(2 dx)
   T m;                           // dt L
+  int sum6;                      // 1: 6 g dt L/dx^2 <= 1/16 (see tdgl_inc)
   T amp;                         // thermal random force: sigma sqrt(dt) (0: off)
   unsigned long long seed;
   long long* step;               // device step counter (steps since pf_bind)
@@ -525,10 +525,14 @@ __device__ __forceinline__ void two_sum(T a, T b, T& s, T& e) {
 // inside, V at an electrode, phi_cell at an open face, so that the difference
 // of the two face values is formed doubled, 2 V or 2 phi_cell at a face).
 // 58 operations a cell in FP32 where the terms written out took 84: FP32 is
-// bound by issue, FP64 by its unit.  The FP32 Laplacian sums differences (they
-// are nearly exact, and the compensated state keeps what they resolve; a
-// difference between two cells of a vector serves both); the FP64 one takes
-// the neighbour sum less 6 P, whose rounding is 0.03 of that of the updated P.
+// bound by issue, FP64 by its unit.  The Laplacian sums differences: they are
+// nearly exact, the compensated state keeps what they resolve, and a difference
+// between two cells of a vector serves both.  In FP64 with small steps (sum6) it
+// takes the neighbour sum less 6 P, five operations fewer a component (448 us for
+// 256 x 256 x 64, 482 with differences): that sum is rounded at the size of 6 P, and
+// the step adds c = 6 g dt L/dx^2 of this to the rounding of P itself.  (c = 0.03: the
+// updated P scatters by 0.2892 units in the last place, 0.2887 with differences;
+// 0.9, near the explicit scheme's limit: 0.55 and 0.29.)
 template <typename T>
 __device__ __forceinline__ void tdgl_inc(const Stencil7<Raw<T, 4>>& st, int xy, int z, const Geo& g,
                                          const Bc<T>& bc, const Coef<T>& k, T (&inc)[3]) {
@@ -551,7 +555,7 @@ __device__ __forceinline__ void tdgl_inc(const Stencil7<Raw<T, 4>>& st, int xy, 
     const int j = (i + 1) % 3, l = (i + 2) % 3;
     const T a = fma(k.c12, fma(p[j], p[j], p2[l]), fma(k.c11, p2[i], k.c1));
     T lap;
-    if constexpr (sizeof(T) == 8) {
+    if (sizeof(T) == 8 && k.sum6) {
       lap = (st.xm.v[i] + st.xp.v[i]) + (st.ym.v[i] + st.yp.v[i]);
       if (lo && hi) {
         lap = fma(T(-6), p[i], lap + (st.zm.v[i] + st.zp.v[i]));
@@ -568,8 +572,7 @@ __device__ __forceinline__ void tdgl_inc(const Stencil7<Raw<T, 4>>& st, int xy, 
       if (lo) lap += st.zm.v[i] - p[i];
       if (hi) lap += st.zp.v[i] - p[i];
     }
-    inc[i] = p[i] * a + (k.gl * lap + k.el * dphi[i]);
-    if constexpr (sizeof(T) == 4) inc[i] *= k.m;
+    inc[i] = k.m * (p[i] * a + (k.gl * lap + k.el * dphi[i]));
   }
 }
 
@@ -1003,13 +1006,13 @@ static void tdgl_v(const LaunchCfg& L, const Geo& g, const Dev<T>& d, const T* P
 template <typename T>
 void launch_tdgl(const LaunchCfg& L, const Geo& g, const Dev<T>& d, const T* P, T* Pn, const double* coef,
                  int corr, const Noise& nz) {
-  const double dtL = sizeof(T) == 8 ? coef[4] : 1.0;
-  const Coef<T> k{T(-2.0 * coef[0] * dtL),
-                  T(-4.0 * coef[1] * dtL),
-                  T(-2.0 * coef[2] * dtL),
-                  T(coef[3] * g.ih2 * dtL),
-                  T(-0.5 * g.ih * dtL),
+  const Coef<T> k{T(-2.0 * coef[0]),
+                  T(-4.0 * coef[1]),
+                  T(-2.0 * coef[2]),
+                  T(coef[3] * g.ih2),
+                  T(-0.5 * g.ih),
                   T(coef[4]),
+                  std::fabs(6.0 * coef[3] * coef[4] * g.ih2) <= 0.0625,
                   T(nz.amp),
                   nz.seed,
                   nz.step,
