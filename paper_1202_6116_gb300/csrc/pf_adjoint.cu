@@ -29,11 +29,13 @@ constexpr int ADJ_NV = 4;
 template <typename T, int VX>
 using AdjPipe = Pipe<T, void, MTX, MTY, VX, 4, 3, ADJ_D>;
 
-// The Hessian's and the stencils' factors times dt L (formed in FP64, rounded once).
+// The Hessian's and the stencils' factors (formed in FP64, rounded once) and, apart
+// from them as in the forward update, dt L.
 template <typename T>
 struct AdjCoef {
-  T h1, h12, hd, hx;             // -2 a1, -2 a12, -(12 a11 - 2 a12), -4 a12
+  T h1, h11, h12, hx;            // -2 a1, -12 a11, -2 a12, -4 a12
   T gl, el;                      // g/dx^2, -1/(2 dx)
+  T m;                           // dt L
   double dtL;
 };
 
@@ -70,32 +72,32 @@ __global__ void __launch_bounds__(MTX* MTY) k_tdgl_adj(Geo g, Bc<T> bc, const T*
     }
     const T p[3] = {o[0], o[1], o[2]};
     const T l[3] = {st.c.v[0], st.c.v[1], st.c.v[2]};
-    // With s = sum P_j^2 and d = sum P_j lam_j, (H lam)_i = lam_i (2 a1 + 2 a12 s +
-    // (12 a11 - 2 a12) P_i^2) + 4 a12 P_i (d - P_i lam_i), and the sensitivities
-    // sum over i to 2 d, 4 sum P_i^3 lam_i and 2 (s d - sum P_i^3 lam_i): 83 FP64
-    // operations a cell where the terms written out took 196.
+    // (H lam)_i = lam_i (2 a1 + 12 a11 P_i^2 + 2 a12 q_i) + 4 a12 P_i d_i with q_i the
+    // sum of the other two P_j^2 and d_i that of the other two P_j lam_j; the products
+    // serve the sensitivities too: 87 FP64 operations a cell where the terms written
+    // out took 196.  (Sums over all three, less the own one, are four operations fewer
+    // and round twice: in FP32 the quartic coefficient along an axis is 1e-7 off.)
     T p2[3], pl[3], out[3];
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
       p2[i] = p[i] * p[i];
       pl[i] = p[i] * l[i];
     }
-    const T s2 = p2[0] + p2[1] + p2[2], d = pl[0] + pl[1] + pl[2];
-    const T t3 = p2[0] * pl[0] + p2[1] * pl[1] + p2[2] * pl[2];
-    const T a = k.h1 + k.h12 * s2;
-    acc[0].add(d, T(1));
-    acc[1].add(t3, T(1));
-    acc[2].add(s2 * d - t3, T(1));
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
+      const int j = (i + 1) % 3, q = (i + 2) % 3;
       T lap = st.xp.v[i] - l[i];
       lap -= l[i] - st.xm.v[i];
       lap += st.yp.v[i] - l[i];
       lap -= l[i] - st.ym.v[i];
       if (st.zb >= 0) lap += st.zm.v[i] - l[i];
       if (st.za >= 0) lap += st.zp.v[i] - l[i];
-      const T Hl = l[i] * (a + k.hd * p2[i]) + k.hx * (p[i] * (d - pl[i]));
-      out[i] = l[i] + (k.gl * lap + (k.el * dpsi[i] + Hl));
+      const T pq = fma(p[j], p[j], p2[q]);
+      const T Hl = fma(l[i], fma(k.h12, pq, fma(k.h11, p2[i], k.h1)), k.hx * p[i] * fma(p[j], l[j], pl[q]));
+      out[i] = l[i] + k.m * (k.gl * lap + (k.el * dpsi[i] + Hl));
+      acc[0].add(l[i], p[i]);
+      acc[1].add(p2[i], pl[i]);
+      acc[2].add(pl[i], pq);
       acc[3].add(p[i], lap);
     }
     if (bt) {
@@ -166,12 +168,13 @@ template <typename T>
 void launch_tdgl_adj(const LaunchCfg& L, const Geo& g, const Dev<T>& d, const T* lam, T* lam_out, const T* psi,
                      const T* P, const double* coef, double* grad, double* gv_lo, double* gv_hi) {
   const double dtL = coef[4];
-  const AdjCoef<T> k{T(-2.0 * coef[0] * dtL),
-                     T(-2.0 * coef[2] * dtL),
-                     T((2.0 * coef[2] - 12.0 * coef[1]) * dtL),
-                     T(-4.0 * coef[2] * dtL),
-                     T(coef[3] * g.ih2 * dtL),
-                     T(-0.5 * g.ih * dtL),
+  const AdjCoef<T> k{T(-2.0 * coef[0]),
+                     T(-12.0 * coef[1]),
+                     T(-2.0 * coef[2]),
+                     T(-4.0 * coef[2]),
+                     T(coef[3] * g.ih2),
+                     T(-0.5 * g.ih),
+                     T(dtL),
                      dtL};
   constexpr int V = 16 / sizeof(T);
   if (L.march.vx == V) adj_t<T, V>(L, g, d, lam, lam_out, psi, P, k, grad, gv_lo, gv_hi);

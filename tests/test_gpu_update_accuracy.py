@@ -73,3 +73,36 @@ def test_fp64_gradient_term(dt):
     lap = sum(np.roll(X, s, d) - X for d in (1, 2, 3) for s in (1, -1))
     err = (P.astype(np.longdouble) - (X + np.longdouble(dt) * np.longdouble(0.5) * lap)) * 2.0 ** 53
     assert float(np.sqrt((err * err).mean())) <= 0.35
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+def test_adjoint_hessian_has_no_bias_at_a_pole(precision):
+    """(lam_out - lam) / dt L = -H(P) lam where P and lam have no divergence
+    (psi = 0) and g = 0, dt L = 1024.  Each value of size 4 is off by a few of its
+    half-ulps u = 2^-24 or 2^-53 (rms 4 u); the mean over 4096 independent ones
+    scatters by u / 16.  Coefficients that do not add up to 12 a11 shift it by 2 u.
+    The sensitivities come from the same products."""
+    dt = np.float32 if precision == "fp32" else np.float64
+    u = 2.0 ** -24 if precision == "fp32" else 2.0 ** -53
+    n = (64, 64, 4)
+    P0 = divergence_free(*n, [0.0, 0.0, 1.0], 0.01, 21, dt)
+    lam0 = divergence_free(*n, [0.0, 0.0, 1.0], 0.01, 22, dt)
+    z8, z = np.zeros((64, 64), np.int8), np.zeros((64, 64))
+    w = W.Workload("adjoint", *n, P0, z8, z, z8, z, precision=precision, periodic_z=True, rtol=1e-7, g=0.0, dt=1024.0)
+    f = Film(w, flags=pf.PF_FLAG_ADJOINT)
+    lam = torch.as_tensor(lam0, dtype=f.dtype, device="cuda").contiguous()
+    out, grad = torch.empty_like(lam), torch.zeros(4, dtype=torch.float64, device="cuda")
+    pf.pf_adjoint_step(f.ctx, lam, out, grad)
+    got = out.double().cpu().numpy()
+    f.close()
+    X, Y = P0.astype(np.longdouble), lam0.astype(np.longdouble)
+    p2, pl = X * X, X * Y
+    H = Y * (-2 + 6 * p2 + np.longdouble(1.6) * (p2.sum(0) - p2)) + np.longdouble(3.2) * X * (pl.sum(0) - pl)
+    # lam_out has size 4096: its own rounding is one part in 1024 of the force's
+    err = ((got.astype(np.longdouble) - Y) / 1024 + H)[2]
+    assert abs(float(err.mean())) <= u / 2
+    assert float(np.abs(err).max()) <= 32 * u
+    ref = [-1024 * float((2 * pl).sum()), -1024 * float((4 * p2 * pl).sum()),
+           -1024 * float((2 * pl * (p2.sum(0) - p2)).sum()),
+           1024 * float((X * sum(np.roll(Y, s, d) - Y for d in (1, 2, 3) for s in (1, -1))).sum())]
+    assert np.abs(grad.cpu().numpy() - ref).max() <= 16 * u * max(map(abs, ref))
