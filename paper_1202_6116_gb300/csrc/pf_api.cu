@@ -790,7 +790,7 @@ void drop_graphs(pf_ctx* ctx) {
 
 // Does a solve run its Krylov loop as one persistent launch?
 bool cg_loop_of(pf_ctx* ctx) {
-  if (ctx->prm.solver != PF_PCG_JACOBI || ctx->prm.has_eps) return false;
+  if (ctx->prm.solver != PF_PCG_JACOBI || ctx->prm.has_eps || ctx->L.loop_halves) return false;
   return ctx->prm.precision == PF_FP32 ? pf::launch_cg_loop<float>(ctx->L, ctx->geo, pf::Dev<float>{}, true)
                                        : pf::launch_cg_loop<double>(ctx->L, ctx->geo, pf::Dev<double>{}, true);
 }
@@ -913,8 +913,12 @@ cudaError_t append_step(pf_ctx* ctx, cudaGraph_t graph, std::vector<cudaGraphNod
     e = cudaStreamBeginCaptureToGraph(st, body, nullptr, nullptr, 0, mode);
     if (e != cudaSuccess) return;
     if (mg) vcycle<T>(ctx, 1);
-    pf::launch_cg_p<T>(ctx->L, g, d, mg);
-    pf::launch_cg_r<T>(ctx->L, g, d, mg, h, 1);
+    if (ctx->L.loop_halves) {
+      pf::launch_cg_halves<T>(ctx->L, g, d, h);
+    } else {
+      pf::launch_cg_p<T>(ctx->L, g, d, mg);
+      pf::launch_cg_r<T>(ctx->L, g, d, mg, h, 1);
+    }
     e = cudaStreamEndCapture(st, &body);
     deps.assign(1, cnode);
     segment([&] {
@@ -1764,6 +1768,43 @@ pf_status batch_upload_table(pf_batch* b) {
   return PF_OK;
 }
 
+// How the films of a batch run their Jacobi-PCG loops, for as long as this
+// object lives.  While all the films' loops have a few blocks per SM together, each
+// as it does alone.  Beyond that, small films (pf_cgloop.cu) as two launches an
+// iteration: ms a step with loops / launches for 10 films of 32^3 in FP32 0.41 / 0.59,
+// 8 of 64 x 64 x 32 0.69 / 0.59; in FP64 5 of 48 x 40 x 24 0.64 / 0.53, 4 of 64 x 64
+// x 32 0.84 / 0.77.  Films that fill the GPU by themselves keep the loop, in FP32 from
+// 32 films on with an eighth of the blocks each, so that fewer of them share the L2:
+// 64 of 96 x 96 x 48 13.2 against 22.1 with two plane marches (16 films: 5.1 on all
+// blocks, 5.5; FP64 is slower with an eighth: 29 against 20 for 16 films of mixed sizes).
+struct BatchLoops {
+  pf_batch* b;
+  explicit BatchLoops(pf_batch* batch) : b(batch) {
+    long long blocks = 0;
+    std::vector<int> small(b->films.size(), 0);
+    for (size_t i = 0; i < b->films.size(); ++i) {
+      pf_ctx* c = b->films[i];
+      if (cg_loop_of(c))
+        blocks += c->prm.precision == PF_FP32 ? pf::cg_loop_blocks<float>(c->L, c->geo, &small[i])
+                                              : pf::cg_loop_blocks<double>(c->L, c->geo, &small[i]);
+    }
+    for (size_t i = 0; i < b->films.size(); ++i) {
+      pf_ctx* c = b->films[i];
+      if (!cg_loop_of(c)) continue;
+      const bool fp32 = c->prm.precision == PF_FP32;
+      if (blocks <= (fp32 ? 6LL : 4LL) * c->nsm) continue;
+      if (small[i]) c->L.loop_halves = 1;
+      else if (fp32 && b->films.size() >= 32) c->L.loop_share = 8;
+    }
+  }
+  ~BatchLoops() {
+    for (pf_ctx* c : b->films) {
+      c->L.loop_share = 1;
+      c->L.loop_halves = 0;
+    }
+  }
+};
+
 // One batch step as a graph: the ramp kernel, every film's step as an
 // independent branch after it, the loop record after all of them.
 // Append one batch step (ramp, every film's step from buffer cur, loop record)
@@ -1794,14 +1835,8 @@ cudaError_t batch_append(pf_batch* b, cudaGraph_t graph, std::vector<cudaGraphNo
   for (pf_ctx* c : b->films) {
     if (e != cudaSuccess) break;
     std::vector<cudaGraphNode_t> dp = ramp;
-    // FP32 with 64 films of 0.03 to 1 million cells: 17.7 ms a step with an
-    // eighth of the blocks, 23.2 with all; 16 of them 6.8 and 6.7 (FP64: 29.1 and
-    // 20.2).  64 films of 32^3: FP32 2.6 and 3.4, FP64 5.5 and 8.1.
-    const bool small = c->geo.n <= 65536, fp32 = c->prm.precision == PF_FP32;
-    c->L.loop_share = (small && b->films.size() >= 12) || (fp32 && b->films.size() >= 32) ? 8 : 1;
     e = c->prm.precision == PF_FP32 ? append_step<float>(c, graph, dp, cur, refresh, b->cap)
                                     : append_step<double>(c, graph, dp, cur, refresh, b->cap);
-    c->L.loop_share = 1;
     joined.insert(joined.end(), dp.begin(), dp.end());
   }
   const int buf = b->films[0]->prm.integrator == PF_HEUN ? cur : cur ^ 1;
@@ -1994,6 +2029,7 @@ pf_status pf_batch_step(pf_batch* b, int32_t nsteps, pf_step_info* info) {
     if (c->prm.precision == PF_FP32) refresh_operators<float>(c, c->L, false);
     else refresh_operators<double>(c, c->L, false);
   }
+  const BatchLoops loops(b);
   const bool heun = f0->prm.integrator == PF_HEUN;
   auto book = [&](int refresh, long long steps) {    // host bookkeeping of graph-run steps
     for (pf_ctx* c : b->films) {

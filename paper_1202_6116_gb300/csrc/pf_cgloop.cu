@@ -19,14 +19,18 @@
 // L2, and nothing is left to overlap the copies with).
 //
 // Several films at once (a batch): the loop's blocks fill the GPU with few
-// films, each waiting at its barriers, where two kernels an iteration had
-// interleaved all (64 films of 32^3 in FP32: 3.36 ms a step against 2.07).  The
-// work is therefore split into virtual blocks, as many as a film alone has
-// blocks, and a film in a batch runs them on an eighth of the blocks: same
-// partials, same order of the sums, same bits, more films side by side.
+// films, each waiting at its barriers.  Its work is split into virtual blocks, as
+// many as a film alone has blocks, so that a film can run them in other ways with
+// the same partials and the same order of the sums, that is the same bits: as the
+// blocks of two ordinary launches an iteration (k_half_p, k_half_r), which the
+// scheduler interleaves with the other films', or on fewer blocks of the loop, so
+// that fewer films at a time keep their vectors in L2.  Which film does what:
+// BatchLoops in pf_api.cu.
 //
 // The barrier's wait is bounded: a block that gives up marks the solve and
 // leaves, and so do the others, each at its own limit.
+#include <type_traits>
+
 #include "pf_internal.h"
 #include "pf_march.cuh"
 
@@ -39,11 +43,6 @@ constexpr int LOOP_ROWS = 16;           // tile: 16 threads along x by 16 rows
 // x 48, 13.5 MB, 106.7 against 111.7; 256 x 256 x 32, 16 MB, 137.4 against 136.0.)
 constexpr size_t LOOP_BYTES = 15u << 20;
 constexpr unsigned LOOP_SPIN = 1u << 22;   // polls before a barrier gives up (seconds)
-
-template <typename T, int VX>
-struct LoopGroups {                     // tiles a block walks at once (registers: 64 or 128 a thread)
-  static constexpr int value = sizeof(T) * VX <= 4 ? 4 : 2;
-};
 
 // Sums of NV values over the block; value k in lane 0 of warp k.  FP32 pairs:
 // a shuffle tree per warp, then one over the warps (a pair_add is 11 FP32
@@ -81,6 +80,15 @@ __device__ __forceinline__ void loop_partial(const V (&v)[NV], void* scratch, do
   if ((tid & 31) == 0 && (tid >> 5) < NV) set[(tid >> 5) * nvb + vb] = d;
 }
 
+// Sum of the nvb partials at v: the same in every warp that forms it.
+__device__ __forceinline__ double loop_total(const double* v, int nvb, int lane) {
+  double a = 0.0;
+  for (int i = lane; i < nvb; i += 32) a += __ldcg(v + i);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+  return a;
+}
+
 // Sums of NV values over the nvb partials in set, in tot, after a barrier of
 // all the grid's blocks: bar counts arrivals (zeroed by the right-hand side
 // kernel), ph numbers the reductions.  The fence before the arrival orders the
@@ -106,123 +114,172 @@ __device__ __forceinline__ bool loop_reduce(const double* set, unsigned* bar, in
   __syncthreads();
   if (!*ok) return false;
   if (wid < NV) {
-    double a = 0.0;
-    for (int i = lane; i < nvb; i += 32) a += __ldcg(set + wid * nvb + i);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+    const double a = loop_total(set + wid * nvb, nvb, lane);
     if (lane == 0) tot[wid] = a;
   }
   __syncthreads();
   return true;
 }
 
-template <typename T, int VX>
-__global__ void __launch_bounds__(256 * LoopGroups<T, VX>::value)
-k_cg_loop(Geo g, Bc<T> bc, T* r, T* p0, T* p1, T* q, T* x, double* part, Scalars* S, MarchCfg mc, int nvb) {
-  constexpr int G = LoopGroups<T, VX>::value, NT = 256 * G;
+template <typename T>
+struct LoopVecs {
+  T *r, *p0, *p1, *q, *x;
+};
+
+// What an iteration knows when it begins.
+template <typename T>
+struct LoopIter {
+  int first, pb, xz;       // first iteration; p_old is p1 (1) or p0; x is still 0
+  T alpha, beta;           // of the last iteration
+};
+
+// First half of an iteration, over the block's virtual blocks: p = z + beta
+// p_old, q = A p, x += alpha p_old; partials of p.q into set.
+template <typename T, int VX, int G>
+__device__ __forceinline__ void loop_p(const Geo& g, const Bc<T>& bc, const LoopVecs<T>& v, const LoopIter<T>& it,
+                                       const MarchCfg& mc, int nvb, double* set, void* scratch, int tid) {
+  constexpr int NT = 256 * G;
   using Sum = typename SumOf<T>::type;
-  __shared__ Sum scratch[2 * NT];
+  const int tx = threadIdx.x, nx = g.nx, ny = g.ny;
+  const long long nxy = g.nxy;
+  const T ih2 = T(g.ih2), inv6 = bc.itab[0], al = it.alpha, beta = it.beta;
+  const bool first = it.first, xz = it.xz;
+  const T* const r = v.r;
+  const T* const pold = it.pb ? v.p1 : v.p0;
+  T* const pnew = it.pb ? v.p0 : v.p1;
+  auto zat = [&](T rv, int xy, int z) -> T { return rn_mul(rv, inv_diag_tab(g, bc, xy, z, inv6)); };
+  // p at one cell, or at VX cells in a row, of plane z
+  auto p1at = [&](long long zo, int xy, int z) -> T {
+    const T zz = zat(r[zo + xy], xy, z);
+    return first ? zz : rn_fma(beta, pold[zo + xy], zz);
+  };
+  auto pvec = [&](int xy, int z, T (&o)[VX], T (&old)[VX]) {
+    const long long c = (long long)z * nxy + xy;
+    T rv[VX];
+    load_n<T, VX>(r + c, rv);
+    if (!first) load_n<T, VX>(pold + c, old);
+#pragma unroll
+    for (int i = 0; i < VX; ++i) {
+      const T zz = zat(rv[i], xy + i, z);
+      o[i] = first ? zz : rn_fma(beta, old[i], zz);
+    }
+  };
+  for (int vb = blockIdx.x; vb < nvb; vb += gridDim.x) {
+    Acc<T> apq;
+    for (long long t = vb * G + threadIdx.z; t < mc.ntiles; t += (long long)nvb * G) {
+      const TileGeo<16, 16, VX> s = tile_geo<16, 16, VX>(g, t, mc);
+      const bool lin = tx > 0, rin = tx < 15 && (tx + 1) * VX < s.w;
+      const int ym = s.y == 0 ? ny - 1 : s.y - 1, yp = s.y == ny - 1 ? 0 : s.y + 1;
+      const int xl = s.x == 0 ? nx - 1 : s.x - 1, xr = s.x + VX >= nx ? 0 : s.x + VX;
+      T pm[VX], pc[VX], pp[VX], oc[VX], op[VX], t0[VX];
+#pragma unroll
+      for (int i = 0; i < VX; ++i) pm[i] = pc[i] = pp[i] = oc[i] = op[i] = t0[i] = T(0);
+      if (s.act) {
+        const int zb = z_below(g, s.z0);
+        if (zb >= 0) pvec(s.xy, zb, pm, t0);
+        pvec(s.xy, s.z0, pc, oc);
+      }
+      for (int z = s.z0; z < s.z1; ++z) {
+        const int zb = z_below(g, z), za = z_above(g, z);
+        const long long zo = (long long)z * nxy;
+        T pym[VX], pyp[VX], xv[VX];
+        T pl = __shfl_up_sync(0xffffffffu, pc[VX - 1], 1), pr = __shfl_down_sync(0xffffffffu, pc[0], 1);
+        if (s.act) {
+          if (za >= 0) pvec(s.xy, za, pp, op);
+          pvec(ym * nx + s.x, z, pym, t0);
+          pvec(yp * nx + s.x, z, pyp, t0);
+          if (!lin) pl = p1at(zo, s.y * nx + xl, z);
+          if (!rin) pr = p1at(zo, s.y * nx + xr, z);
+          if (!first && !xz) load_n<T, VX>(v.x + zo + s.xy, xv);
+          T qv[VX];
+          const bool bt = zb < 0 || za < 0;
+#pragma unroll
+          for (int i = 0; i < VX; ++i) {
+            Stencil7<T> st;
+            st.c = pc[i];
+            st.xm = i == 0 ? pl : pc[i - 1];
+            st.xp = i == VX - 1 ? pr : pc[i + 1];
+            st.ym = pym[i];
+            st.yp = pyp[i];
+            st.zm = pm[i];
+            st.zp = pp[i];
+            st.zb = zb;
+            st.za = za;
+            const int dlo = (bt && zb < 0) ? (int)bc.tlo[s.xy + i] : 0;
+            const int dhi = (bt && za < 0) ? (int)bc.thi[s.xy + i] : 0;
+            qv[i] = apply_bt(st, dlo, dhi, ih2, bt);
+            apq.add(pc[i], qv[i]);
+            if (!first) xv[i] = xz ? rn_mul(al, oc[i]) : rn_fma(al, oc[i], xv[i]);
+          }
+          apq.run();
+          if (!first) store_n<T, VX>(v.x + zo + s.xy, xv);
+          store_n<T, VX>(pnew + zo + s.xy, pc);
+          store_n<T, VX>(v.q + zo + s.xy, qv);
+        }
+#pragma unroll
+        for (int i = 0; i < VX; ++i) {
+          pm[i] = pc[i];
+          pc[i] = pp[i];
+          oc[i] = op[i];
+        }
+      }
+    }
+    const Sum sum[1] = {apq.sum()};
+    loop_partial<1, NT>(sum, scratch, set, vb, nvb, tid);
+  }
+}
+
+// Second half: r -= alpha q over the same tiles; partials of r.r and r.z.
+template <typename T, int VX, int G>
+__device__ __forceinline__ void loop_r(const Geo& g, const Bc<T>& bc, const LoopVecs<T>& v, T alpha, const MarchCfg& mc,
+                                       int nvb, double* set, void* scratch, int tid) {
+  constexpr int NT = 256 * G;
+  using Sum = typename SumOf<T>::type;
+  const T inv6 = bc.itab[0];
+  for (int vb = blockIdx.x; vb < nvb; vb += gridDim.x) {
+    Acc<T> arr, arz;
+    for (long long t = vb * G + threadIdx.z; t < mc.ntiles; t += (long long)nvb * G) {
+      const TileGeo<16, 16, VX> s = tile_geo<16, 16, VX>(g, t, mc);
+      if (!s.act) continue;
+      for (int z = s.z0; z < s.z1; ++z) {
+        const long long c = (long long)z * g.nxy + s.xy;
+        T rv[VX], qv[VX];
+        load_n<T, VX>(v.r + c, rv);
+        load_n<T, VX>(v.q + c, qv);
+#pragma unroll
+        for (int i = 0; i < VX; ++i) {
+          rv[i] = rn_fma(-alpha, qv[i], rv[i]);
+          arr.add(rv[i], rv[i]);
+          arz.add(rv[i], rn_mul(rv[i], inv_diag_tab(g, bc, s.xy + i, z, inv6)));
+        }
+        arr.run();
+        arz.run();
+        store_n<T, VX>(v.r + c, rv);
+      }
+    }
+    const Sum sum[2] = {arr.sum(), arz.sum()};
+    loop_partial<2, NT>(sum, scratch, set, vb, nvb, tid);
+  }
+}
+
+template <typename T, int VX, int G>
+__global__ void __launch_bounds__(256 * G)
+k_cg_loop(Geo g, Bc<T> bc, LoopVecs<T> v, double* part, Scalars* S, MarchCfg mc, int nvb) {
+  constexpr int NT = 256 * G;
+  __shared__ typename SumOf<T>::type scratch[2 * NT];
   __shared__ double tot[2], alpha_s, beta_s, rel_s;
   __shared__ int verdict, ok;           // verdict: 0 go on, 1 converged, 2 maxit, 3 breakdown, 4 non-finite
   if (S->done) return;                  // written by this kernel only after the last barrier
-  const int tx = threadIdx.x, ty = threadIdx.y, tid = tx + 16 * ty + 256 * threadIdx.z;
-  const int nx = g.nx, ny = g.ny;
-  const long long nxy = g.nxy;
-  const T ih2 = T(g.ih2);
-  const T inv6 = bc.itab[0];
-  auto inv_at = [&](int xy, int z) -> T { return inv_diag_tab(g, bc, xy, z, inv6); };
+  const int tid = threadIdx.x + 16 * threadIdx.y + 256 * threadIdx.z;
   const double rtol = S->rtol, bnorm = S->bnorm;
   const int maxit = S->maxit;
   double rz = S->rz, rr = 0.0, rel = S->last_rel, alpha = 0.0;
-  T beta = T(0);
-  int pb = S->pbuf, iter = 0, xz = S->xzero;
-  int ph = 0;
+  LoopIter<T> it{1, S->pbuf, S->xzero, T(0), T(0)};
+  int iter = 0, ph = 0;
 
   for (;;) {
-    const bool first = iter == 0;
-    const T* const pold = pb ? p1 : p0;
-    T* const pnew = pb ? p0 : p1;
-    const T al = T(alpha);
-    // p at one cell, or at VX cells in a row, of plane z
-    auto p1at = [&](long long zo, int xy, int z) -> T {
-      const T zz = r[zo + xy] * inv_at(xy, z);
-      return first ? zz : zz + beta * pold[zo + xy];
-    };
-    auto pvec = [&](int xy, int z, T (&o)[VX], T (&old)[VX]) {
-      const long long c = (long long)z * nxy + xy;
-      T rv[VX];
-      load_n<T, VX>(r + c, rv);
-      if (!first) load_n<T, VX>(pold + c, old);
-#pragma unroll
-      for (int i = 0; i < VX; ++i) {
-        const T zz = rv[i] * inv_at(xy + i, z);
-        o[i] = first ? zz : zz + beta * old[i];
-      }
-    };
     double* set = part + (size_t)(ph & 1) * 2 * nvb;
-    for (int vb = blockIdx.x; vb < nvb; vb += gridDim.x) {
-      Acc<T> apq;
-      for (long long t = vb * G + threadIdx.z; t < mc.ntiles; t += (long long)nvb * G) {
-        const TileGeo<16, 16, VX> s = tile_geo<16, 16, VX>(g, t, mc);
-        const bool lin = tx > 0, rin = tx < 15 && (tx + 1) * VX < s.w;
-        const int ym = s.y == 0 ? ny - 1 : s.y - 1, yp = s.y == ny - 1 ? 0 : s.y + 1;
-        const int xl = s.x == 0 ? nx - 1 : s.x - 1, xr = s.x + VX >= nx ? 0 : s.x + VX;
-        T pm[VX], pc[VX], pp[VX], oc[VX], op[VX], t0[VX];
-#pragma unroll
-        for (int i = 0; i < VX; ++i) pm[i] = pc[i] = pp[i] = oc[i] = op[i] = t0[i] = T(0);
-        if (s.act) {
-          const int zb = z_below(g, s.z0);
-          if (zb >= 0) pvec(s.xy, zb, pm, t0);
-          pvec(s.xy, s.z0, pc, oc);
-        }
-        for (int z = s.z0; z < s.z1; ++z) {
-          const int zb = z_below(g, z), za = z_above(g, z);
-          const long long zo = (long long)z * nxy;
-          T pym[VX], pyp[VX], xv[VX];
-          T pl = __shfl_up_sync(0xffffffffu, pc[VX - 1], 1), pr = __shfl_down_sync(0xffffffffu, pc[0], 1);
-          if (s.act) {
-            if (za >= 0) pvec(s.xy, za, pp, op);
-            pvec(ym * nx + s.x, z, pym, t0);
-            pvec(yp * nx + s.x, z, pyp, t0);
-            if (!lin) pl = p1at(zo, s.y * nx + xl, z);
-            if (!rin) pr = p1at(zo, s.y * nx + xr, z);
-            if (!first && !xz) load_n<T, VX>(x + zo + s.xy, xv);
-            T qv[VX];
-            const bool bt = zb < 0 || za < 0;
-#pragma unroll
-            for (int i = 0; i < VX; ++i) {
-              Stencil7<T> st;
-              st.c = pc[i];
-              st.xm = i == 0 ? pl : pc[i - 1];
-              st.xp = i == VX - 1 ? pr : pc[i + 1];
-              st.ym = pym[i];
-              st.yp = pyp[i];
-              st.zm = pm[i];
-              st.zp = pp[i];
-              st.zb = zb;
-              st.za = za;
-              const int dlo = (bt && zb < 0) ? (int)bc.tlo[s.xy + i] : 0;
-              const int dhi = (bt && za < 0) ? (int)bc.thi[s.xy + i] : 0;
-              qv[i] = apply_bt(st, dlo, dhi, ih2, bt);
-              apq.add(pc[i], qv[i]);
-              if (!first) xv[i] = xz ? al * oc[i] : xv[i] + al * oc[i];
-            }
-            apq.run();
-            if (!first) store_n<T, VX>(x + zo + s.xy, xv);
-            store_n<T, VX>(pnew + zo + s.xy, pc);
-            store_n<T, VX>(q + zo + s.xy, qv);
-          }
-#pragma unroll
-          for (int i = 0; i < VX; ++i) {
-            pm[i] = pc[i];
-            pc[i] = pp[i];
-            oc[i] = op[i];
-          }
-        }
-      }
-      const Sum v[1] = {apq.sum()};
-      loop_partial<1, NT>(v, scratch, set, vb, nvb, tid);
-    }
+    loop_p<T, VX, G>(g, bc, v, it, mc, nvb, set, scratch, tid);
     // alpha = r.z / p.q
     {
       if (!loop_reduce<1>(set, &S->bar, ph++, nvb, tid, tot, &ok)) {
@@ -236,38 +293,15 @@ k_cg_loop(Geo g, Bc<T> bc, T* r, T* p0, T* p1, T* q, T* x, double* part, Scalars
       }
       __syncthreads();
     }
-    if (!first) xz = 0;
+    if (!it.first) it.xz = 0;
     ++iter;
-    pb ^= 1;
+    it.first = 0;
+    it.pb ^= 1;
     alpha = alpha_s;
     if (verdict) break;                 // breakdown: stop with the current iterate
-    // r -= alpha q over the same tiles, r.r and r.z
-    const T aq = T(alpha);
+    it.alpha = T(alpha);
     set = part + (size_t)(ph & 1) * 2 * nvb;
-    for (int vb = blockIdx.x; vb < nvb; vb += gridDim.x) {
-      Acc<T> arr, arz;
-      for (long long t = vb * G + threadIdx.z; t < mc.ntiles; t += (long long)nvb * G) {
-        const TileGeo<16, 16, VX> s = tile_geo<16, 16, VX>(g, t, mc);
-        if (!s.act) continue;
-        for (int z = s.z0; z < s.z1; ++z) {
-          const long long c = (long long)z * nxy + s.xy;
-          T rv[VX], qv[VX];
-          load_n<T, VX>(r + c, rv);
-          load_n<T, VX>(q + c, qv);
-#pragma unroll
-          for (int i = 0; i < VX; ++i) {
-            rv[i] = rv[i] - aq * qv[i];
-            arr.add(rv[i], rv[i]);
-            arz.add(rv[i], rv[i] * inv_at(s.xy + i, z));
-          }
-          arr.run();
-          arz.run();
-          store_n<T, VX>(r + c, rv);
-        }
-      }
-      const Sum v[2] = {arr.sum(), arz.sum()};
-      loop_partial<2, NT>(v, scratch, set, vb, nvb, tid);
-    }
+    loop_r<T, VX, G>(g, bc, v, it.alpha, mc, nvb, set, scratch, tid);
     {
       if (!loop_reduce<2>(set, &S->bar, ph++, nvb, tid, tot, &ok)) {
         if (tid == 0) S->timeout = 1;
@@ -283,14 +317,14 @@ k_cg_loop(Geo g, Bc<T> bc, T* r, T* p0, T* p1, T* q, T* x, double* part, Scalars
       rr = tot[0];
     }
     if (verdict) break;
-    beta = T(beta_s);
+    it.beta = T(beta_s);
     rz = tot[1];
   }
   if (blockIdx.x != 0 || tid != 0) return;
   S->iter = iter;
-  S->pbuf = pb;
+  S->pbuf = it.pb;
   S->first = 0;
-  S->xzero = xz;
+  S->xzero = it.xz;
   S->alpha = alpha;
   S->rz = rz;
   if (verdict == 1 || verdict == 2 || verdict == 4) {
@@ -301,6 +335,73 @@ k_cg_loop(Geo g, Bc<T> bc, T* r, T* p0, T* p1, T* q, T* x, double* part, Scalars
   if (verdict != 1) S->status = 3;
   if (verdict == 4) S->nonfinite = 1;
   S->done = 1;
+}
+
+// The two halves of an iteration as launches of their own, a virtual block per
+// block: the same partials in the same order, so the same bits as the loop.  (64
+// films of 64 x 64 x 32 in FP32: 59 us an iteration for all of them, 302 MB through
+// L2; two plane marches 66 us.)
+template <typename T, int VX, int G>
+__global__ void __launch_bounds__(256 * G)
+k_half_p(Geo g, Bc<T> bc, LoopVecs<T> v, double* part, Scalars* S, MarchCfg mc) {
+  constexpr int NT = 256 * G;
+  __shared__ typename SumOf<T>::type scratch[2 * NT];
+  if (S->done) return;
+  const int tid = threadIdx.x + 16 * threadIdx.y + 256 * threadIdx.z, nvb = gridDim.x;
+  const LoopIter<T> it{S->first, S->pbuf, S->xzero, T(S->alpha), T(S->beta)};
+  loop_p<T, VX, G>(g, bc, v, it, mc, nvb, part, scratch, tid);
+  if (!last_block<NT>(&S->ticket) || tid >= 32) return;
+  const double a = loop_total(part, nvb, tid);
+  if (tid != 0) return;
+  S->iter += 1;
+  S->pbuf = it.pb ^ 1;
+  if (!it.first) S->xzero = 0;
+  S->first = 0;
+  S->alpha = (a > 0.0) ? S->rz / a : 0.0;
+  if (!(a > 0.0)) {                     // breakdown (or NaN): stop with the current iterate
+    if (!isfinite(a)) S->nonfinite = 1;
+    S->pending = 0;
+    S->status = 3;
+    S->done = 1;
+  }
+  S->ticket = 0;
+}
+
+template <typename T, int VX, int G>
+__global__ void __launch_bounds__(256 * G)
+k_half_r(Geo g, Bc<T> bc, LoopVecs<T> v, double* part, Scalars* S, MarchCfg mc, cudaGraphConditionalHandle cond) {
+  constexpr int NT = 256 * G;
+  __shared__ typename SumOf<T>::type scratch[2 * NT];
+  const int tid = threadIdx.x + 16 * threadIdx.y + 256 * threadIdx.z, nvb = gridDim.x;
+  if (S->done) {                        // a breakdown in k_half_p ends the loop
+    if (blockIdx.x == 0 && tid == 0) cudaGraphSetConditional(cond, 0u);
+    return;
+  }
+  loop_r<T, VX, G>(g, bc, v, T(S->alpha), mc, nvb, part, scratch, tid);
+  if (!last_block<NT>(&S->ticket) || tid >= 32) return;
+  const double rr = loop_total(part, nvb, tid), rz = loop_total(part + nvb, nvb, tid);
+  if (tid != 0) return;
+  const double rel = sqrt(rr) / S->bnorm;
+  S->rr = rr;
+  S->last_rel = rel;
+  if (!isfinite(rr)) {
+    S->nonfinite = 1;
+    S->status = 3;
+    S->pending = 0;
+    S->done = 1;
+  } else if (rel < S->rtol) {
+    S->pending = 1;
+    S->done = 1;
+  } else if (S->iter >= S->maxit) {
+    S->pending = 1;
+    S->status = 3;
+    S->done = 1;
+  } else {
+    S->beta = rz / S->rz;
+    S->rz = rz;
+  }
+  S->ticket = 0;
+  cudaGraphSetConditional(cond, S->done ? 0u : 1u);
 }
 
 // ---------------------------------------------------------------- launchers
@@ -326,46 +427,105 @@ static MarchCfg loop_tiles(const Geo& g, int vx, long long streams) {
   return m;
 }
 
+// Virtual blocks and tiles of a film's loop.
+static int loop_blocks(const LaunchCfg& L, const Geo& g, int vx, int groups, MarchCfg& mc) {
+  mc = loop_tiles(g, vx, (long long)L.nsm * groups);
+  return (int)std::min<long long>(L.nsm, (mc.ntiles + groups - 1) / groups);
+}
+
 // dry: only whether it can be launched here.
-template <typename T, int VX>
+template <typename T, int VX, int G>
 static bool cg_loop_t(const LaunchCfg& L, const Geo& g, const Dev<T>& d, bool dry) {
-  constexpr int G = LoopGroups<T, VX>::value;
-  auto kernel = k_cg_loop<T, VX>;
-  static int blocks = -1;               // blocks of the grid (0: cannot be launched here)
-  if (blocks < 0) {
+  auto kernel = k_cg_loop<T, VX, G>;
+  static int can = -1;
+  if (can < 0) {
     int nb = 0, coop = 0, dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kernel, 256 * G, 0) != cudaSuccess)
       coop = 0;
     cudaGetLastError();
-    blocks = coop && nb > 0 ? L.nsm : 0;
+    can = coop && nb > 0;
   }
-  if (dry || blocks == 0) return blocks > 0;
-  const MarchCfg mc = loop_tiles(g, VX, (long long)blocks * G);
+  if (dry || !can) return can;
+  MarchCfg mc;
+  const int nvb = loop_blocks(L, g, VX, G, mc);
   cudaLaunchConfig_t cfg{};
   cudaLaunchAttribute at{};
   at.id = cudaLaunchAttributeCooperative;
   at.val.cooperative = 1;
-  const int nvb = (int)std::min<long long>(blocks, (mc.ntiles + G - 1) / G);
   cfg.gridDim = dim3((unsigned)((nvb + L.loop_share - 1) / L.loop_share));
   cfg.blockDim = dim3(16, 16, G);
   cfg.stream = L.stream;
   cfg.attrs = &at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, g, d.bc, d.r, d.p0, d.p1, d.q, d.phi, d.part, d.S, mc, nvb) == cudaSuccess;
+  const LoopVecs<T> v{d.r, d.p0, d.p1, d.q, d.phi};
+  return cudaLaunchKernelEx(&cfg, kernel, g, d.bc, v, d.part, d.S, mc, nvb) == cudaSuccess;
+}
+
+template <typename T, int VX, int G>
+static void cg_halves_t(const LaunchCfg& L, const Geo& g, const Dev<T>& d, cudaGraphConditionalHandle cond) {
+  MarchCfg mc;
+  const int nvb = loop_blocks(L, g, VX, G, mc);
+  const dim3 block(16, 16, G);
+  const LoopVecs<T> v{d.r, d.p0, d.p1, d.q, d.phi};
+  k_half_p<T, VX, G><<<nvb, block, 0, L.stream>>>(g, d.bc, v, d.part, d.S, mc);
+  k_half_r<T, VX, G><<<nvb, block, 0, L.stream>>>(g, d.bc, v, d.part, d.S, mc, cond);
+}
+
+// Does a film have a 16-byte vector for every thread that the GPU holds?
+template <typename T>
+static bool loop_fills(const LaunchCfg& L, const Geo& g) {
+  constexpr int V = 16 / sizeof(T);
+  return g.n / V >= (long long)L.nsm * 512;
+}
+
+// Calls f with the cells of a film's threads and the thread groups of its blocks.
+// Films that do not fill the GPU take vectors all the same (half as long where 16 of
+// them are longer than a row) and one group a block: ms a step of a film alone 0.123
+// on 32^3 and 0.127 on 64 x 64 x 32 in FP32, where single cells and four groups took
+// 0.136 and 0.143, and 0.169 against 0.177 on 32^3 in FP64 (vectors with two groups:
+// 0.206); 64 such films as two launches an iteration 1.87, 3.9 and 3.35, where single
+// cells took 2.47, 8.4 and 4.6 and two plane marches take 2.15, 4.34 and 3.78.  Rows of
+// no whole vectors (101 x 75 x 19) keep four groups in FP32, 0.191 against 0.223.
+template <typename T, class F>
+static auto loop_form(const LaunchCfg& L, const Geo& g, F f) {
+  constexpr int V = 16 / sizeof(T), F32 = sizeof(T) == 4;
+  const bool vec = L.march.vx == V;
+  using std::integral_constant;
+  if (loop_fills<T>(L, g)) {
+    if (vec) return f(integral_constant<int, V>(), integral_constant<int, 2>());
+    return f(integral_constant<int, 1>(), integral_constant<int, F32 ? 4 : 2>());
+  }
+  if (vec && 16 * (V / 2) >= g.nx) return f(integral_constant<int, V / 2>(), integral_constant<int, 1>());
+  if (vec) return f(integral_constant<int, V>(), integral_constant<int, 1>());
+  return f(integral_constant<int, 1>(), integral_constant<int, F32 ? 4 : 1>());
 }
 
 template <typename T>
 bool launch_cg_loop(const LaunchCfg& L, const Geo& g, const Dev<T>& d, bool dry) {
-  constexpr int V = 16 / sizeof(T);
   if (d.eps || (size_t)g.n * sizeof(T) > LOOP_BYTES) return false;
-  // vectors when they are enough to occupy every thread
-  const bool vec = L.march.vx == V && g.n / V >= (long long)L.nsm * 256 * LoopGroups<T, V>::value;
-  return vec ? cg_loop_t<T, V>(L, g, d, dry) : cg_loop_t<T, 1>(L, g, d, dry);
+  return loop_form<T>(L, g, [&](auto vx, auto groups) { return cg_loop_t<T, vx, groups>(L, g, d, dry); });
 }
 
-template bool launch_cg_loop<float>(const LaunchCfg&, const Geo&, const Dev<float>&, bool);
-template bool launch_cg_loop<double>(const LaunchCfg&, const Geo&, const Dev<double>&, bool);
+template <typename T>
+int cg_loop_blocks(const LaunchCfg& L, const Geo& g, int* small) {
+  MarchCfg mc;
+  *small = !loop_fills<T>(L, g);
+  return loop_form<T>(L, g, [&](auto vx, auto groups) { return loop_blocks(L, g, vx, groups, mc); });
+}
+
+template <typename T>
+void launch_cg_halves(const LaunchCfg& L, const Geo& g, const Dev<T>& d, cudaGraphConditionalHandle cond) {
+  loop_form<T>(L, g, [&](auto vx, auto groups) { cg_halves_t<T, vx, groups>(L, g, d, cond); });
+}
+
+#define PF_LOOP_INSTANTIATE(T)                                                              \
+  template bool launch_cg_loop<T>(const LaunchCfg&, const Geo&, const Dev<T>&, bool);       \
+  template int cg_loop_blocks<T>(const LaunchCfg&, const Geo&, int*);                       \
+  template void launch_cg_halves<T>(const LaunchCfg&, const Geo&, const Dev<T>&, cudaGraphConditionalHandle);
+
+PF_LOOP_INSTANTIATE(float)
+PF_LOOP_INSTANTIATE(double)
 
 }  // namespace pf

@@ -143,6 +143,15 @@ struct Scalars {
                                    // start and is still 0 (its buffer holds stale values)
 };
 
+// Operations that are not contracted further: for arithmetic that two kernels
+// share bit for bit.
+__device__ __forceinline__ float rn_add(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float rn_mul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float rn_fma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double rn_add(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ double rn_mul(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ double rn_fma(double a, double b, double c) { return __fma_rn(a, b, c); }
+
 // ---------------------------------------------------------------- reductions
 //
 // What a thread sums in FP32 it keeps as an unevaluated pair (hi, lo), and the
@@ -282,7 +291,7 @@ template <int NT>
 __device__ __forceinline__ bool last_block(unsigned* ticket) {
   __shared__ bool last;
   __syncthreads();
-  if (threadIdx.x == 0 && threadIdx.y == 0) {
+  if (threadIdx.x == 0 && threadIdx.y == 0 && threadIdx.z == 0) {
     __threadfence();
     const unsigned t = atomicAdd(ticket, 1u);
     last = (t == gridDim.x - 1);

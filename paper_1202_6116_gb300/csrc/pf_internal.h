@@ -54,7 +54,8 @@ struct LaunchCfg {
                        // (tiled = 1), or the default of the CG operator
   int tiled;           // 1: a tiling was set (pf_set_tiling); 0: every kernel plans its own
   int nsm, word, nx, ny, nz;
-  int loop_share = 1;  // virtual blocks per block of the persistent Jacobi-PCG loop (films of a batch: see pf_cgloop.cu)
+  int loop_share = 1;  // virtual blocks per block of the persistent Jacobi-PCG loop
+  int loop_halves = 0; // 1: that loop as two launches an iteration (both: films of a batch, see pf_cgloop.cu)
   mutable MarchCfg plan[2][PLAN_OCC];   // planned tilings (ntiles = 0: not yet), see kernel_tiling
   int flat_grid;       // flat vector kernels (FLAT_THREADS blocks, grid-stride)
   cudaStream_t stream;
@@ -200,6 +201,13 @@ void launch_cg_r(const LaunchCfg& L, const Geo& g, const Dev<T>& d, int mg, cuda
 // possible here; dry: only whether it is.
 template <typename T>
 bool launch_cg_loop(const LaunchCfg& L, const Geo& g, const Dev<T>& d, bool dry);
+// One iteration of that loop as two launches, with the same bits (in a graph's
+// conditional loop); and the blocks of a film's loop when it runs alone (*small: 1
+// when the film does not fill the GPU).
+template <typename T>
+void launch_cg_halves(const LaunchCfg& L, const Geo& g, const Dev<T>& d, cudaGraphConditionalHandle cond);
+template <typename T>
+int cg_loop_blocks(const LaunchCfg& L, const Geo& g, int* small);
 template <typename T>
 void launch_cg_finish(const LaunchCfg& L, const Geo& g, const Dev<T>& d, int singular);
 template <typename T>

@@ -57,13 +57,7 @@ __device__ __forceinline__ T apply_aniso(const Stencil7<T>& s, int dlo, int dhi,
 // out (no contraction left to the compiler): the kernels that form them on
 // the same cell -- the pre-smoother, the residual and their fused form on a
 // split level -- then agree bit for bit.
-__device__ __forceinline__ float rn_add(float a, float b) { return __fadd_rn(a, b); }
-__device__ __forceinline__ float rn_mul(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ float rn_fma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
-__device__ __forceinline__ double rn_add(double a, double b) { return __dadd_rn(a, b); }
-__device__ __forceinline__ double rn_mul(double a, double b) { return __dmul_rn(a, b); }
-__device__ __forceinline__ double rn_fma(double a, double b, double c) { return __fma_rn(a, b, c); }
-
+//
 // The operator is taken as d c - S, d the diagonal (constant away from the z
 // faces) and S the weighted sum of the neighbours, with a sweep's constants
 // folded into the weights: seven to eight operations a cell and sweep instead
