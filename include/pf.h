@@ -405,12 +405,15 @@ typedef struct {
                                 tolerance). */
 } pf_tiling;
 
-/* Current tiling (the default picks vx = 16 bytes when nx allows it and the
- * deepest tz that still gives about three tiles per resident block). */
+/* Current tiling.  By default vx is 16 bytes when nx allows it and every kernel
+ * plans its own tile depth for its own occupancy; tz is then the depth planned
+ * for the CG operator, and blocks_per_sm 0. */
 pf_status pf_get_tiling(const pf_ctx* ctx, pf_tiling* out);
 
-/* Replace the tiling; results are unchanged up to the order of the reduction
- * sums (dot products and norms are summed per tile).  Drops captured graphs. */
+/* Replace the tiling: every kernel takes this one, except that the default's
+ * values of vx, tz and blocks_per_sm (with either mg_whole) put the planned
+ * depths back.  Results are unchanged up to the order of the reduction sums (dot
+ * products and norms are summed per tile).  Drops captured graphs. */
 pf_status pf_set_tiling(pf_ctx* ctx, const pf_tiling* tiling);
 
 /* ------------------------------------------------------------------- batch

@@ -7,6 +7,9 @@ objective is device time per Krylov iteration (CUDA events on the film's
 stream), so candidates are compared fairly even when the iteration counts of
 the timed steps differ.  Results are cached per (shape, precision, solver,
 permittivity) in memory and, optionally, in a JSON file.
+
+The default is timed first and wins ties: setting its values gives every kernel
+its own planned depth, which no other candidate does.
 """
 from __future__ import annotations
 

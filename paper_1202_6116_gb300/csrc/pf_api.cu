@@ -1669,8 +1669,10 @@ pf_status pf_set_tiling(pf_ctx* ctx, const pf_tiling* t) {
   m.grid = (int)std::min<long long>(m.ntiles, std::min<long long>(pf::MAX_GRID, (long long)bps * ctx->nsm));
   m.bps = t->blocks_per_sm;
   drop_graphs(ctx);
-  ctx->L.march = m;
-  ctx->L.tiled = 1;
+  // the default's values, as pf_get_tiling reports them, put the planned tilings back
+  const pf::MarchCfg& dflt = ctx->L.dflt;
+  ctx->L.tiled = m.vx != dflt.vx || m.tz != dflt.tz || m.bps != 0;
+  ctx->L.march = ctx->L.tiled ? m : dflt;
   ctx->tile_bps = t->blocks_per_sm;
   ctx->mg_whole = t->mg_whole;
   ctx->gen += 1;

@@ -51,8 +51,10 @@ struct LaunchCfg {
   int grid;            // simple per-cell kernels (TX x TY blocks over tiles)
   dim3 block;
   MarchCfg march;      // plane-march kernels (MTX x MTY blocks): the tiling asked for
-                       // (tiled = 1), or the default of the CG operator
-  int tiled;           // 1: a tiling was set (pf_set_tiling); 0: every kernel plans its own
+                       // (tiled = 1), or dflt
+  MarchCfg dflt;       // the planned tiling of the CG operator: what a context reports and
+                       // takes as "every kernel plans its own" (tiled = 0)
+  int tiled;           // 1: another tiling was set (pf_set_tiling)
   int nsm, word, nx, ny, nz;
   int loop_share = 1;  // virtual blocks per block of the persistent Jacobi-PCG loop
   int loop_halves = 0; // 1: that loop as two launches an iteration (both: films of a batch, see pf_cgloop.cu)
@@ -442,6 +444,7 @@ inline void setup_launch(const pf_params* p, int nsm, cudaStream_t stream, Geo& 
   L.ny = g.ny;
   L.nz = g.nz;
   L.march = march_cfg(g.nx, g.ny, g.nz, nsm, std::min(PLAN_OCC, march_blocks_per_sm(fp32, p->has_eps)), 64, false, L.word);
+  L.dflt = L.march;
   const long long nvec = (g.n + 3) / 4;
   L.flat_grid = (int)std::max<long long>(
       1, std::min<long long>((nvec + FLAT_THREADS - 1) / FLAT_THREADS, std::min(MAX_GRID, 4 * nsm)));
