@@ -284,6 +284,7 @@ struct pf_ctx {
   bool loop_broken = false;          // the loop graph cannot be built here: one launch per step
   int graph_key = -1;             // singular flag the graphs were captured for
   bool graphs_broken = false;     // capture not possible: host-driven loop
+  bool loop_refused = false;      // the persistent CG loop could not be launched: two launches an iteration
   int64_t graph_steps = 0;        // steps of the current call run as graphs
   int64_t graph_fixed = 0;        // kernels of those steps outside the Krylov loops
   int64_t graph_solves = 0;       // Poisson solves of those steps
@@ -861,6 +862,7 @@ cudaError_t append_step(pf_ctx* ctx, cudaGraph_t graph, std::vector<cudaGraphNod
     e = cudaStreamBeginCaptureToGraph(st, graph, deps.empty() ? nullptr : deps.data(), nullptr, deps.size(), mode);
     if (e != cudaSuccess) return;
     body();
+    const cudaError_t launched = cudaGetLastError();     // a launch that failed is not in the graph
     cudaStreamCaptureStatus cs;
     const cudaGraphNode_t* fr = nullptr;
     size_t nfr = 0;
@@ -869,6 +871,7 @@ cudaError_t append_step(pf_ctx* ctx, cudaGraph_t graph, std::vector<cudaGraphNod
     cudaGraph_t g_out = graph;
     const cudaError_t e2 = cudaStreamEndCapture(st, &g_out);
     if (e == cudaSuccess) e = e2;
+    if (launched != cudaSuccess) e = launched;
   };
   // One Poisson solve for the state P with its own loop condition.
   pf::Dev<T> ds = d;
@@ -919,7 +922,9 @@ cudaError_t append_step(pf_ctx* ctx, cudaGraph_t graph, std::vector<cudaGraphNod
       pf::launch_cg_p<T>(ctx->L, g, d, mg);
       pf::launch_cg_r<T>(ctx->L, g, d, mg, h, 1);
     }
+    const cudaError_t launched = cudaGetLastError();
     e = cudaStreamEndCapture(st, &body);
+    if (launched != cudaSuccess) e = launched;
     deps.assign(1, cnode);
     segment([&] {
       pf::launch_cg_finish<T>(ctx->L, g, d, ctx->singular);
@@ -988,8 +993,10 @@ pf_status capture_loop(pf_ctx* ctx, cudaGraphExec_t* out) {
                                         cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
       pf::launch_loop_next((long long*)(ctx->ws + ctx->lay.loop), h, ctx->cap_stream);
+      const cudaError_t launched = cudaGetLastError();
       cudaGraph_t g2 = body;
       e = cudaStreamEndCapture(ctx->cap_stream, &g2);
+      if (launched != cudaSuccess) e = launched;
     }
   }
   if (e == cudaSuccess) e = cudaGraphInstantiate(&exec, graph, 0);
@@ -1822,6 +1829,7 @@ cudaError_t batch_append(pf_batch* b, cudaGraph_t graph, std::vector<cudaGraphNo
     e = cudaStreamBeginCaptureToGraph(b->cap, graph, dp.empty() ? nullptr : dp.data(), nullptr, dp.size(), mode);
     if (e != cudaSuccess) return;
     body();
+    const cudaError_t launched = cudaGetLastError();     // a launch that failed is not in the graph
     cudaStreamCaptureStatus cs;
     const cudaGraphNode_t* fr = nullptr;
     size_t nfr = 0;
@@ -1830,6 +1838,7 @@ cudaError_t batch_append(pf_batch* b, cudaGraph_t graph, std::vector<cudaGraphNo
     cudaGraph_t g_out = graph;
     const cudaError_t e2 = cudaStreamEndCapture(b->cap, &g_out);
     if (e == cudaSuccess) e = e2;
+    if (launched != cudaSuccess) e = launched;
   };
   std::vector<cudaGraphNode_t> ramp = deps;
   segment(ramp, [&] { pf::launch_batch_ramp(table, nf, b->max_nxy, bs, b->cap); });
@@ -1891,8 +1900,10 @@ pf_status batch_capture_loop(pf_batch* b, cudaGraphExec_t* out) {
                                         cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
       pf::launch_loop_next((long long*)(b->ws + b->off_loop), h, b->cap);
+      const cudaError_t launched = cudaGetLastError();
       cudaGraph_t g2 = body;
       e = cudaStreamEndCapture(b->cap, &g2);
+      if (launched != cudaSuccess) e = launched;
     }
   }
   if (e == cudaSuccess) e = cudaGraphInstantiate(&exec, graph, 0);
