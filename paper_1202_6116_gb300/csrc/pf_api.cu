@@ -725,7 +725,12 @@ pf_status solve(pf_ctx* ctx, const T* P, bool adj = false, bool step_solve = fal
   if (cg_loop_of(ctx)) {                   // every iteration in one launch
     before_launch(ctx);
     looped = pf::launch_cg_loop<T>(ctx->L, g, d, false);
-    PF_CUDA(cudaGetLastError());
+    if (!looped) {                         // refused: two launches an iteration, here and from now on
+      cudaGetLastError();
+      ctx->loop_refused = true;
+    }
+  }
+  if (looped) {
     after_launch(ctx, F_CG_LOOP, 9 * N * w, 3);
     pf_status st = read_scalars(ctx);
     if (st != PF_OK) return st;
@@ -791,7 +796,7 @@ void drop_graphs(pf_ctx* ctx) {
 
 // Does a solve run its Krylov loop as one persistent launch?
 bool cg_loop_of(pf_ctx* ctx) {
-  if (ctx->prm.solver != PF_PCG_JACOBI || ctx->prm.has_eps || ctx->L.loop_halves) return false;
+  if (ctx->prm.solver != PF_PCG_JACOBI || ctx->prm.has_eps || ctx->L.loop_halves || ctx->loop_refused) return false;
   return ctx->prm.precision == PF_FP32 ? pf::launch_cg_loop<float>(ctx->L, ctx->geo, pf::Dev<float>{}, true)
                                        : pf::launch_cg_loop<double>(ctx->L, ctx->geo, pf::Dev<double>{}, true);
 }
@@ -902,7 +907,7 @@ cudaError_t append_step(pf_ctx* ctx, cudaGraph_t graph, std::vector<cudaGraphNod
         }
       }
     });
-    if (e == cudaSuccess && loop && !looped) e = cudaErrorNotSupported;
+    if (loop && !looped) ctx->loop_refused = true;       // the capture failed with it: once more without
     if (e != cudaSuccess || loop) return;
     cudaGraphNode_t cnode = nullptr;
     cudaGraphNodeParams cp{};
@@ -949,6 +954,7 @@ cudaError_t append_step(pf_ctx* ctx, cudaGraph_t graph, std::vector<cudaGraphNod
 // Capture one whole time step of this film as its own executable graph.
 template <typename T>
 pf_status capture_step(pf_ctx* ctx, int cur, int refresh, cudaGraphExec_t* out) {
+  const bool refused = ctx->loop_refused;
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
   std::vector<cudaGraphNode_t> deps;
@@ -958,6 +964,7 @@ pf_status capture_step(pf_ctx* ctx, int cur, int refresh, cudaGraphExec_t* out) 
   if (graph) cudaGraphDestroy(graph);
   if (e != cudaSuccess) {
     cudaGetLastError();
+    if (ctx->loop_refused != refused) return capture_step<T>(ctx, cur, refresh, out);
     return ctx->fail(PF_ERR_CUDA, "graph capture: %s", cudaGetErrorString(e));
   }
   *out = exec;
@@ -971,6 +978,7 @@ pf_status capture_step(pf_ctx* ctx, int cur, int refresh, cudaGraphExec_t* out) 
 // one graph launch however many steps it takes.
 template <typename T>
 pf_status capture_loop(pf_ctx* ctx, cudaGraphExec_t* out) {
+  const bool refused = ctx->loop_refused;
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
   cudaError_t e = cudaGraphCreate(&graph, 0);
@@ -1003,6 +1011,7 @@ pf_status capture_loop(pf_ctx* ctx, cudaGraphExec_t* out) {
   if (graph) cudaGraphDestroy(graph);
   if (e != cudaSuccess) {
     cudaGetLastError();
+    if (ctx->loop_refused != refused) return capture_loop<T>(ctx, out);
     return ctx->fail(PF_ERR_CUDA, "step loop graph: %s", cudaGetErrorString(e));
   }
   *out = exec;
@@ -1858,7 +1867,16 @@ cudaError_t batch_append(pf_batch* b, cudaGraph_t graph, std::vector<cudaGraphNo
   return e;
 }
 
+// (A capture that failed because a film's persistent loop was refused is done
+// once more: that film then iterates with two launches.)
+int batch_refused(const pf_batch* b) {
+  int n = 0;
+  for (const pf_ctx* c : b->films) n += c->loop_refused;
+  return n;
+}
+
 pf_status batch_capture(pf_batch* b, int cur, int refresh, cudaGraphExec_t* out) {
+  const int refused = batch_refused(b);
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
   cudaError_t e = cudaGraphCreate(&graph, 0);
@@ -1868,6 +1886,7 @@ pf_status batch_capture(pf_batch* b, int cur, int refresh, cudaGraphExec_t* out)
   if (graph) cudaGraphDestroy(graph);
   if (e != cudaSuccess) {
     cudaGetLastError();
+    if (batch_refused(b) != refused) return batch_capture(b, cur, refresh, out);
     return b->fail(PF_ERR_CUDA, "batch graph capture: %s", cudaGetErrorString(e));
   }
   *out = exec;
@@ -1878,6 +1897,7 @@ pf_status batch_capture(pf_batch* b, int cur, int refresh, cudaGraphExec_t* out)
 // device-driven while loop counted down by k_loop_next, so that a whole
 // pf_batch_step call is one graph launch.
 pf_status batch_capture_loop(pf_batch* b, cudaGraphExec_t* out) {
+  const int refused = batch_refused(b);
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
   cudaError_t e = cudaGraphCreate(&graph, 0);
@@ -1910,6 +1930,7 @@ pf_status batch_capture_loop(pf_batch* b, cudaGraphExec_t* out) {
   if (graph) cudaGraphDestroy(graph);
   if (e != cudaSuccess) {
     cudaGetLastError();
+    if (batch_refused(b) != refused) return batch_capture_loop(b, out);
     return b->fail(PF_ERR_CUDA, "batch step loop graph: %s", cudaGetErrorString(e));
   }
   *out = exec;

@@ -158,10 +158,9 @@ pf_status solve(const pf_params* prm, cudaStream_t st, char* base, const Layout&
   pf::launch_rhs<T>(L, g, d, P, 0, 0);
   if (launched("rhs") != PF_OK) return PF_ERR_CUDA;
   pf::Scalars host;
-  const bool loop = pf::launch_cg_loop<T>(L, g, d, true);
+  const bool loop = pf::launch_cg_loop<T>(L, g, d, true) && pf::launch_cg_loop<T>(L, g, d, false);
+  if (!loop) cudaGetLastError();           // refused: two launches an iteration
   if (loop) {                              // every iteration in one launch
-    pf::launch_cg_loop<T>(L, g, d, false);
-    if (launched("cg_loop") != PF_OK) return PF_ERR_CUDA;
     launches += 1;
     NA_CUDA(cudaMemcpyAsync(&host, d.S, sizeof(host), cudaMemcpyDeviceToHost, st));
     NA_CUDA(cudaStreamSynchronize(st));

@@ -1,6 +1,7 @@
 // Host-only stand-ins for the kernel launchers, linked with the compiled C ABI
 // (pf_api) and fake_runtime.cpp: launches are counted and can fail.
-//   fake_cuda solve|step|nograph|batch pcg|mg loop|sub|none
+// Arguments: a scenario, the solver and what fails
+//   fake_cuda solve|noalloc|step|nograph|batch pcg|mg loop|sub|none
 // Prints the status, the launches outside and inside captures, and pf_step_info.
 #include <cstdio>
 #include <cstdlib>
@@ -140,6 +141,8 @@ int main(int argc, char** argv) {
     pf_status st;
     if (what == "solve") {
       st = pf_solve_potential(films[0], &info);
+    } else if (what == "noalloc") {
+      st = pf_solve_potential_noalloc(&p, nullptr, std::calloc(3 * n, 8), std::calloc(n, 8), nullptr, nullptr, nullptr, nullptr, &info);
     } else if (what == "batch") {
       static pf_batch* b = nullptr;
       const size_t bb = pf_batch_workspace_bytes(nf, 4);

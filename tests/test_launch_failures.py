@@ -14,10 +14,11 @@ OK, ERR_CUDA = 0, 2
 @pytest.fixture(scope="module")
 def fake(tmp_path_factory):
     B.build()
-    obj = os.path.join(B.OBJ_DIR, "pf_api.o")
     exe = str(tmp_path_factory.mktemp("fake") / "fake_cuda")
     srcs = [os.path.join(HERE, "fakes", f) for f in ("fake_cuda.cu", "fake_runtime.cpp")]
-    srcs += [obj if os.path.exists(obj) else os.path.join(B.CSRC, "pf_api.cu")]
+    for f in ("pf_api", "pf_noalloc"):
+        obj = os.path.join(B.OBJ_DIR, f + ".o")
+        srcs.append(obj if os.path.exists(obj) else os.path.join(B.CSRC, f + ".cu"))
     r = subprocess.run([B._nvcc(), "-O1", "-std=c++17", "--expt-relaxed-constexpr", "-cudart", "none", "-I" + B.INCLUDE,
                         "-I" + B.CSRC] + B.ARCH + srcs + ["-o", exe], capture_output=True, text=True)
     assert r.returncode == 0, r.stdout + r.stderr
@@ -37,6 +38,29 @@ def test_without_failures(fake):
         assert st == OK and direct["cg_loop"] == 1 and "cg_p" not in direct
     (st, steps, _, captured), _ = fake("step", "mg", "none")
     assert st == OK and steps == 1 and captured["mg_sub"] >= 1
+    for st, _, direct, _ in fake("noalloc", "pcg", "none"):
+        assert st == OK and direct["cg_loop"] == 1 and "cg_p" not in direct
+
+
+def test_refused_loop_iterates_with_two_launches(fake):
+    """Solves and host-driven steps clear the refusal, iterate as without the loop and do not try it again."""
+    for what in ("solve", "nograph"):
+        first, second = fake(what, "pcg", "loop")
+        assert first[0] == second[0] == OK
+        assert first[2]["cg_loop"] == 1 and first[2]["cg_p"] >= 1 and first[2]["cg_r"] >= 1
+        assert "cg_loop" not in second[2] and second[2]["cg_p"] >= 1
+    for st, _, direct, _ in fake("noalloc", "pcg", "loop"):       # it keeps nothing between calls
+        assert st == OK and direct["cg_p"] >= 1
+
+
+@pytest.mark.parametrize("what", ["step", "batch"])
+def test_refused_loop_in_a_capture(fake, what):
+    """The graph is captured once more with the two launches, and steps still run as graphs."""
+    first, second = fake(what, "pcg", "loop")
+    assert first[0] == second[0] == OK
+    assert first[1] == 1 and second[1] == 5
+    assert first[3]["cg_p"] >= 1 and first[2]["graph"] == 1
+    assert "cg_loop" not in second[3]
 
 
 @pytest.mark.parametrize("what", ["step", "batch", "nograph", "solve"])
