@@ -56,7 +56,7 @@ typedef enum {
   PF_ERR_CUDA = 2,       /* a CUDA runtime call failed; see pf_last_error */
   PF_ERR_NOCONV = 3,     /* a Poisson solve hit poisson_maxit (state stays valid) */
   PF_ERR_NONFINITE = 4,  /* NaN or Inf detected in the solver scalars */
-  PF_ERR_TIMEOUT = 5,    /* reserved: a bounded device wait gave up */
+  PF_ERR_TIMEOUT = 5,    /* a bounded device wait gave up (see pf_set_wait_limit) */
   PF_ERR_STATE = 6,      /* call out of order (e.g. pf_step before pf_bind) */
   PF_ERR_NOTIMPL = 7     /* entry point declared but not available */
 } pf_status;
@@ -416,6 +416,17 @@ pf_status pf_get_tiling(const pf_ctx* ctx, pf_tiling* out);
  * products and norms are summed per tile).  Drops captured graphs. */
 pf_status pf_set_tiling(pf_ctx* ctx, const pf_tiling* tiling);
 
+/* ----------------------------------------------------------- bounded waits
+ * Jacobi-PCG solves of small grids run as one launch whose thread blocks wait
+ * for one another (csrc/pf_cgloop.cu).  Each such wait gives up after `polls`
+ * polls of its flag (0: the default, some seconds), for instance because the GPU
+ * does not let all blocks run.  The solve then ends where it is, later solves
+ * of the same call end before their first iteration, and the call returns
+ * PF_ERR_TIMEOUT with those solves counted as nonconverged.  P and phi hold no
+ * valid state then: give the context a state again (and potentials, or zero
+ * them) before the next call.  Drops captured graphs. */
+pf_status pf_set_wait_limit(pf_ctx* ctx, uint32_t polls);
+
 /* ------------------------------------------------------------------- batch
  * Many independent films advanced together: a batch step is a CUDA graph
  * holding, per film, its whole time step (its device-driven Krylov loops
@@ -452,8 +463,8 @@ pf_status pf_batch_set_ramp(pf_batch* batch, int32_t film, int32_t face, double 
 
 /* Advance every film by nsteps steps (blocks until done).  info (may be
  * NULL) sums the films' solver statistics (last_iters, last_relres: the
- * largest over the films); the result is the worst film status
- * (PF_ERR_NONFINITE before PF_ERR_NOCONV before PF_OK). */
+ * largest over the films); the result is the worst film status (PF_ERR_TIMEOUT,
+ * PF_ERR_NONFINITE, PF_ERR_NOCONV, PF_OK in that order). */
 pf_status pf_batch_step(pf_batch* batch, int32_t nsteps, pf_step_info* info);
 
 /* Statistics of film i over the last pf_batch_step call. */

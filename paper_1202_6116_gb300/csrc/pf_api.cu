@@ -735,8 +735,7 @@ pf_status solve(pf_ctx* ctx, const T* P, bool adj = false, bool step_solve = fal
     pf_status st = read_scalars(ctx);
     if (st != PF_OK) return st;
     prof_harvest(ctx, ctx->S_host->iter, ctx->S_host->done);
-    if (ctx->S_host->timeout) return ctx->fail(PF_ERR_TIMEOUT, "a wait of the persistent CG loop ran out");
-    if (!ctx->S_host->done) return ctx->fail(PF_ERR_STATE, "internal: the CG loop did not finish");
+    if (!ctx->S_host->done && !ctx->S_host->timeout) return ctx->fail(PF_ERR_STATE, "internal: the CG loop did not finish");
   }
   // Every issued iteration either runs or returns at entry once the device
   // flag is set, and the device sets it by iteration maxit at the latest.
@@ -1695,6 +1694,15 @@ pf_status pf_set_tiling(pf_ctx* ctx, const pf_tiling* t) {
   return PF_OK;
 }
 
+pf_status pf_set_wait_limit(pf_ctx* ctx, uint32_t polls) {
+  if (!ctx) return PF_ERR_ARG;
+  if (ctx->async_open) return ctx->fail(PF_ERR_STATE, "pf_step_async work is pending (call pf_step_wait first)");
+  drop_graphs(ctx);
+  ctx->L.loop_polls = polls ? polls : pf::LOOP_POLLS;
+  ctx->gen += 1;
+  return PF_OK;
+}
+
 pf_status pf_destroy(pf_ctx* ctx) {
   if (!ctx) return PF_OK;
   drop_graphs(ctx);
@@ -2123,9 +2131,10 @@ pf_status pf_batch_step(pf_batch* b, int32_t nsteps, pf_step_info* info) {
     pf_step_info& fi = b->infos[i];
     fi = pf_step_info{};
     const pf_status st = finish_info(c, nsteps, &fi);
-    if (st == PF_ERR_CUDA || st == PF_ERR_STATE || st == PF_ERR_TIMEOUT)
-      return b->fail(st, "film %d: %s", i, c->err.c_str());
-    if (st == PF_ERR_NONFINITE || (st == PF_ERR_NOCONV && worst == PF_OK)) worst = st;
+    if (st == PF_ERR_CUDA || st == PF_ERR_STATE) return b->fail(st, "film %d: %s", i, c->err.c_str());
+    if (st == PF_ERR_TIMEOUT || (st == PF_ERR_NONFINITE && worst != PF_ERR_TIMEOUT) ||
+        (st == PF_ERR_NOCONV && worst == PF_OK))
+      worst = st;
     sum.last_iters = std::max(sum.last_iters, fi.last_iters);
     sum.total_iters += fi.total_iters;
     sum.max_iters = std::max(sum.max_iters, fi.max_iters);
@@ -2138,7 +2147,9 @@ pf_status pf_batch_step(pf_batch* b, int32_t nsteps, pf_step_info* info) {
   sum.kernel_launches += 2LL * nsteps + loop_launches;   // the ramp and record kernels (and loop counters)
   sum.status = worst;
   if (info) *info = sum;
-  if (worst != PF_OK) b->fail(worst, "%s", worst == PF_ERR_NONFINITE ? "a film went non-finite" : "a Poisson solve hit poisson_maxit");
+  if (worst != PF_OK) b->fail(worst, "%s", worst == PF_ERR_TIMEOUT     ? "a wait of the persistent CG loop ran out"
+                                            : worst == PF_ERR_NONFINITE ? "a film went non-finite"
+                                                                        : "a Poisson solve hit poisson_maxit");
   return worst;
 }
 

@@ -28,7 +28,9 @@
 // BatchLoops in pf_api.cu.
 //
 // The barrier's wait is bounded: a block that gives up marks the solve and
-// leaves, and so do the others, each at its own limit.
+// leaves, and so do the others, each at its own limit.  The solve then ends as one
+// that did not converge, and the call's later solves end before their first
+// iteration (rhs_close), so that a call of many steps waits once.
 #include <type_traits>
 
 #include "pf_internal.h"
@@ -42,7 +44,6 @@ constexpr int LOOP_ROWS = 16;           // tile: 16 threads along x by 16 rows
 // of 256 x 256 x 64, 16 MB, 45.7 against 42.4.  FP64, bound by its unit: 192 x 192
 // x 48, 13.5 MB, 106.7 against 111.7; 256 x 256 x 32, 16 MB, 137.4 against 136.0.)
 constexpr size_t LOOP_BYTES = 15u << 20;
-constexpr unsigned LOOP_SPIN = 1u << 22;   // polls before a barrier gives up (seconds)
 
 // Sums of NV values over the block; value k in lane 0 of warp k.  FP32 pairs:
 // a shuffle tree per warp, then one over the warps (a pair_add is 11 FP32
@@ -98,7 +99,7 @@ __device__ __forceinline__ double loop_total(const double* v, int nvb, int lane)
 // ran out.
 template <int NV>
 __device__ __forceinline__ bool loop_reduce(const double* set, unsigned* bar, int ph, int nvb, int tid, double* tot,
-                                            int* ok) {
+                                            int* ok, unsigned polls) {
   const int lane = tid & 31, wid = tid >> 5;
   __syncthreads();
   if (tid == 0) {
@@ -108,7 +109,7 @@ __device__ __forceinline__ bool loop_reduce(const double* set, unsigned* bar, in
     unsigned n = 0, c;
     do {
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(c) : "l"(bar) : "memory");
-    } while ((int)(c - target) < 0 && ++n < LOOP_SPIN);
+    } while ((int)(c - target) < 0 && ++n < polls);
     *ok = (int)(c - target) >= 0;
   }
   __syncthreads();
@@ -264,7 +265,7 @@ __device__ __forceinline__ void loop_r(const Geo& g, const Bc<T>& bc, const Loop
 
 template <typename T, int VX, int G>
 __global__ void __launch_bounds__(256 * G)
-k_cg_loop(Geo g, Bc<T> bc, LoopVecs<T> v, double* part, Scalars* S, MarchCfg mc, int nvb) {
+k_cg_loop(Geo g, Bc<T> bc, LoopVecs<T> v, double* part, Scalars* S, MarchCfg mc, int nvb, unsigned polls) {
   constexpr int NT = 256 * G;
   __shared__ typename SumOf<T>::type scratch[2 * NT];
   __shared__ double tot[2], alpha_s, beta_s, rel_s;
@@ -282,8 +283,8 @@ k_cg_loop(Geo g, Bc<T> bc, LoopVecs<T> v, double* part, Scalars* S, MarchCfg mc,
     loop_p<T, VX, G>(g, bc, v, it, mc, nvb, set, scratch, tid);
     // alpha = r.z / p.q
     {
-      if (!loop_reduce<1>(set, &S->bar, ph++, nvb, tid, tot, &ok)) {
-        if (tid == 0) S->timeout = 1;
+      if (!loop_reduce<1>(set, &S->bar, ph++, nvb, tid, tot, &ok, polls)) {
+        if (tid == 0) S->timeout = S->status = 3;
         return;
       }
       if (tid == 0) {
@@ -303,8 +304,8 @@ k_cg_loop(Geo g, Bc<T> bc, LoopVecs<T> v, double* part, Scalars* S, MarchCfg mc,
     set = part + (size_t)(ph & 1) * 2 * nvb;
     loop_r<T, VX, G>(g, bc, v, it.alpha, mc, nvb, set, scratch, tid);
     {
-      if (!loop_reduce<2>(set, &S->bar, ph++, nvb, tid, tot, &ok)) {
-        if (tid == 0) S->timeout = 1;
+      if (!loop_reduce<2>(set, &S->bar, ph++, nvb, tid, tot, &ok, polls)) {
+        if (tid == 0) S->timeout = S->status = 3;
         return;
       }
       if (tid == 0) {
@@ -460,7 +461,7 @@ static bool cg_loop_t(const LaunchCfg& L, const Geo& g, const Dev<T>& d, bool dr
   cfg.attrs = &at;
   cfg.numAttrs = 1;
   const LoopVecs<T> v{d.r, d.p0, d.p1, d.q, d.phi};
-  return cudaLaunchKernelEx(&cfg, kernel, g, d.bc, v, d.part, d.S, mc, nvb) == cudaSuccess;
+  return cudaLaunchKernelEx(&cfg, kernel, g, d.bc, v, d.part, d.S, mc, nvb, L.loop_polls) == cudaSuccess;
 }
 
 template <typename T, int VX, int G>

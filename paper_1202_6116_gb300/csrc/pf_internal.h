@@ -45,6 +45,7 @@ inline bool mg_split_level(long long n, int nz, int periodic_z, int eps) {
   return !periodic_z && nz >= 2 * MG_SPLIT_B + 2 && n >= (eps ? MG_SPLIT_CELLS_EPS : MG_SPLIT_CELLS);
 }
 
+constexpr unsigned LOOP_POLLS = 1u << 22;   // polls before a barrier of the persistent CG loop gives up (seconds)
 constexpr int PLAN_OCC = 6;      // tilings are planned for up to this many blocks per SM
 
 struct LaunchCfg {
@@ -57,6 +58,7 @@ struct LaunchCfg {
   int tiled;           // 1: another tiling was set (pf_set_tiling)
   int nsm, word, nx, ny, nz;
   int loop_share = 1;  // virtual blocks per block of the persistent Jacobi-PCG loop
+  unsigned loop_polls = LOOP_POLLS;   // (pf_set_wait_limit)
   int loop_halves = 0; // 1: that loop as two launches an iteration (both: films of a batch, see pf_cgloop.cu)
   mutable MarchCfg plan[2][PLAN_OCC];   // planned tilings (ntiles = 0: not yet), see kernel_tiling
   int flat_grid;       // flat vector kernels (FLAT_THREADS blocks, grid-stride)

@@ -107,6 +107,10 @@ __device__ __forceinline__ void rhs_close(const Geo& g, double* part, Scalars* S
     S->last_rel = rel;
     S->done = (rel < S->rtol) ? 1 : 0;
   }
+  if (S->timeout) {                   // an earlier solve of the call gave up: no more waits
+    S->status = 3;
+    S->done = 1;
+  }
   S->ticket = 0;
   if (use_cond) cudaGraphSetConditional(cond, S->done ? 0u : 1u);
 }

@@ -32,6 +32,7 @@ EXPORTS = ["pf_workspace_bytes", "pf_create", "pf_bind", "pf_set_bc", "pf_step",
            "pf_step_host", "pf_true_residual",
            "pf_solve_potential", "pf_adjoint_step", "pf_diagnostics", "pf_profile_enable", "pf_profile_read", "pf_destroy",
            "pf_last_error", "pf_solve_potential_noalloc", "pf_set_noise", "pf_get_tiling", "pf_set_tiling",
+           "pf_set_wait_limit",
            "pf_batch_workspace_bytes", "pf_batch_create", "pf_batch_set_ramp", "pf_batch_step",
            "pf_batch_film_info", "pf_batch_read_loops", "pf_batch_destroy", "pf_batch_last_error"]
 
@@ -121,6 +122,8 @@ def lib():
         L.pf_get_tiling.argtypes = [vp, C.POINTER(pf_tiling)]
         L.pf_set_tiling.restype = i32
         L.pf_set_tiling.argtypes = [vp, C.POINTER(pf_tiling)]
+        L.pf_set_wait_limit.restype = i32
+        L.pf_set_wait_limit.argtypes = [vp, C.c_uint32]
         L.pf_batch_workspace_bytes.restype = sz
         L.pf_batch_workspace_bytes.argtypes = [i32, C.c_int64]
         L.pf_batch_create.restype = i32
@@ -289,6 +292,11 @@ def pf_get_tiling(ctx) -> pf_tiling:
     t = pf_tiling()
     check(lib().pf_get_tiling(ctx, C.byref(t)), ctx)
     return t
+
+
+def pf_set_wait_limit(ctx, polls=0):
+    """Polls after which a wait inside a kernel gives up (0: the default)."""
+    return check(lib().pf_set_wait_limit(ctx, int(polls)), ctx)
 
 
 def pf_set_tiling(ctx, vx, tz, blocks_per_sm=0, mg_whole=0):
