@@ -48,24 +48,33 @@ constexpr size_t LOOP_BYTES = 15u << 20;
 // Sums of NV values over the block; value k in lane 0 of warp k.  FP32 pairs:
 // a shuffle tree per warp, then one over the warps (a pair_add is 11 FP32
 // operations; 32 of them in a row, as one warp over all threads would take,
-// are 1400 cycles).  FP64: block_sums.
+// are 1400 cycles), each again in doubles where a pair leaves the range of a
+// float.  scratch: 2 NV NT / 32 elements.  FP64: block_sums.
 template <int NV, int NT>
 __device__ __forceinline__ double loop_sums(const float2 (&v)[NV], void* scratch, int tid) {
-  float2* sm = static_cast<float2*>(scratch);
   constexpr int NW = NT / 32;
+  float2* sm = static_cast<float2*>(scratch);
+  double* wide = reinterpret_cast<double*>(sm + NV * NW);
   const int lane = tid & 31, wid = tid >> 5;
 #pragma unroll
   for (int k = 0; k < NV; ++k) {
     float2 d = v[k];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) d = pair_add(d, sum_xor(d, o));
+    if (__any_sync(0xffffffffu, !isfinite(d.x))) {
+      const double e = warp_total(sum_double(v[k]));
+      if (lane == 0) wide[k * NW + wid] = e;
+      d.x = NAN;
+    }
     if (lane == 0) sm[k * NW + wid] = d;
   }
   __syncthreads();
   if (wid >= NV) return 0.0;
-  float2 d = lane < NW ? sm[wid * NW + lane] : make_float2(0.f, 0.f);
+  const float2 w = lane < NW ? sm[wid * NW + lane] : make_float2(0.f, 0.f);
+  float2 d = w;
 #pragma unroll
   for (int o = NW / 2; o > 0; o >>= 1) d = pair_add(d, sum_xor(d, o));
+  if (__any_sync(0xffffffffu, !isfinite(d.x))) return warp_total(isfinite(w.x) ? sum_double(w) : wide[wid * NW + lane]);
   return sum_double(d);
 }
 template <int NV, int NT>
@@ -85,9 +94,7 @@ __device__ __forceinline__ void loop_partial(const V (&v)[NV], void* scratch, do
 __device__ __forceinline__ double loop_total(const double* v, int nvb, int lane) {
   double a = 0.0;
   for (int i = lane; i < nvb; i += 32) a += __ldcg(v + i);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-  return a;
+  return warp_total(a);
 }
 
 // Sums of NV values over the nvb partials in set, in tot, after a barrier of

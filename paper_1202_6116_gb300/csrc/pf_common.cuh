@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 namespace pf {
 
 // Tile of one thread block in the simple per-cell kernels: TX x TY columns of
@@ -178,7 +180,8 @@ struct SumOf<float> {
 
 // (a.x + a.y) + (b.x + b.y) as a normalised pair: TwoSum (Knuth) of the
 // leading parts, the rest in the second part; relative error about 2^-46 of
-// |a| + |b|.
+// |a| + |b|.  Past the range of a float the pair is NaN, and the reductions sum
+// once more in doubles, as they would the threads' FP32 sums otherwise.
 __device__ __forceinline__ float2 pair_add(float2 a, float2 b) {
   const float s = __fadd_rn(a.x, b.x);
   const float z = __fsub_rn(s, a.x);
@@ -241,15 +244,19 @@ __device__ __forceinline__ double sum_xor(double v, int o) { return __shfl_xor_s
 __device__ __forceinline__ float2 sum_xor(float2 v, int o) {
   return make_float2(__shfl_xor_sync(0xffffffffu, v.x, o), __shfl_xor_sync(0xffffffffu, v.y, o));
 }
+__device__ __forceinline__ double warp_total(double v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
 __device__ __forceinline__ double sum_double(double v) { return v; }
 __device__ __forceinline__ double sum_double(float2 v) { return (double)v.x + (double)v.y; }
 
 // Sums of NV values over the NT threads of a block; the sum of value k
 // is returned (as a double) in lane 0 of warp k.  Every thread must call it
-// with its linear index;
-// it ends without a barrier.  Warp k adds value k of all threads from shared
+// with its linear index; it ends without a barrier.  Warp k adds value k of all threads from shared
 // memory: 12 additions a value with 256 threads, where a shuffle tree in each
-// of the eight warps takes 45.  sm: sum_scratch<V>(NV) bytes, 8-byte aligned, that nobody
+// of the eight warps takes 45.  sm: NV NT elements, 8-byte aligned, that nobody
 // else uses until the block's next barrier -- the plane marches lend their
 // staging buffers, which are idle between tiles (12 KB of static shared
 // memory beside them shrank the L1 and cost k_rhs_w 7 %).  Not inlined: it
@@ -262,6 +269,15 @@ __device__ __noinline__ double shared_sums(const V* sm, int tid) {
   for (int j = 1; j < NT / 32; ++j) d = sum_add(d, sm[wid * NT + lane + 32 * j]);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) d = sum_add(d, sum_xor(d, o));
+  if constexpr (std::is_same<V, float2>::value) {
+    // past the range of a float (or not finite at all): the threads' pairs as doubles
+    if (__any_sync(0xffffffffu, !isfinite(d.x))) {
+      double e = 0.0;
+#pragma unroll 1
+      for (int j = 0; j < NT / 32; ++j) e += sum_double(sm[wid * NT + lane + 32 * j]);
+      return warp_total(e);
+    }
+  }
   return sum_double(d);
 }
 template <int NV, int NT, typename V>
