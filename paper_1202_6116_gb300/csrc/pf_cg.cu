@@ -67,15 +67,10 @@ __global__ void __launch_bounds__(MTX* MTY, (sizeof(T) == 4 && !EPS) ? 3 : 2) k_
   TileGeo<MTX, MTY, VX> s;
 
   auto val = [&](const T (&h)[NH], int xy, int z, int, int, const bool bt) -> F {
-    T zz;
-    if constexpr (MG) {
-      zz = h[0];
-    } else {
-      T inv;
-      if constexpr (EPS) inv = h[NH - 1];
-      else inv = bt ? inv_diag_unit(g, bc, xy, z, inv6) : inv6;
-      zz = h[0] * inv;
-    }
+    T inv;
+    if constexpr (EPS) inv = h[NH - 1];
+    else inv = bt ? inv_diag_unit(g, bc, xy, z, inv6) : inv6;
+    const T zz = h[0] * inv;
     const T v = first ? zz : zz + beta * h[1];
     if constexpr (EPS) return F{v, h[2]};
     else return v;

@@ -35,10 +35,7 @@ namespace pf {
 constexpr int SUB_CLUSTER = 16;
 constexpr int SUB_ROWS = 64;      // coarsest levels up to this size: a row per thread of block 0
 
-template <typename T>
-struct SubThreads {
-  static constexpr int value = 512;
-};
+constexpr int SUB_THREADS = 512;
 
 __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;\n" ::: "memory");
@@ -558,7 +555,7 @@ int launch_coarse_inverse(const LaunchCfg& L, const MgView<T>& C, int singular, 
 template <typename T, bool EPS>
 static cudaError_t mg_sub_t(const LaunchCfg& L, const MgTail& t, const void* blob, const double* cinv, int last,
                             double* part, Scalars* S) {
-  constexpr int NT = SubThreads<T>::value;
+  constexpr int NT = SUB_THREADS;
   auto kernel = k_mg_sub<T, NT, EPS>;
   static int cluster = 0;                            // blocks per cluster that this device launches
   cudaLaunchConfig_t cfg{};

@@ -27,8 +27,9 @@ constexpr int MG_MAX_COARSE = 1024;   // cells of the coarsest multigrid level (
 // / 16.58 / 16.66.
 inline long long mg_sub_cells(size_t word) { return word == 4 ? 65536 : 16384; }
 inline long long mg_solo_cells(size_t word) { return word == 4 ? 1024 : 256; }
-constexpr int MG_TAIL_LEVELS = 24;
-constexpr int MG_TAIL_SMEM = 192 * 1024;   // shared-memory limit of the solo levels' arrays (bytes)
+// Dynamic shared memory of that launch at most: descriptors and masks of 24 levels, three fields of a coarsest
+// level of 1024 cells (FP64) or of solo levels from 1024 cells down (FP32), 34 KB either way.
+constexpr int MG_TAIL_SMEM = 40 * 1024;
 // A multigrid sweep over a large level whose z faces are not periodic runs as
 // two launches: the interior planes [b, nz - b), compiled without the face
 // code (fewer registers, more resident blocks), and the two face slabs of b
@@ -307,7 +308,7 @@ inline double march_cost(long long cols, int nz, int tz, int nsm, int occ, int w
     double t;
     long long m;
   };
-  Group q[160];
+  Group q[160];                                   // three are needed: every chunk but the last is equally deep
   int nq = 1;
   q[0] = Group{0.0, nsm};
   auto insert = [&](double t, long long m) {      // groups in ascending order of t
@@ -352,8 +353,7 @@ inline double march_cost(long long cols, int nz, int tz, int nsm, int occ, int w
 // columns takes the deepest tiles, one of 64 x 64 a couple of planes per tile.
 // (The rule before it, the deepest of 32 .. 2 planes with three tiles per
 // resident block, gave a 256 x 256 x 64 film tiles of 2 planes: 55 us for the
-// right-hand side, 33 for the search direction; planned, 39 with 16 planes and
-// 22 with 10.)
+// right-hand side, 33 for the search direction; planned, 37 and 23.)
 inline MarchCfg march_cfg(int nx, int ny, int nz, int nsm, int occ, int tzmax, bool even_tz, int word) {
   MarchCfg m{};
   const int v = 16 / word;
