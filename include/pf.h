@@ -186,7 +186,11 @@ typedef struct {
 /* Bytes of device workspace needed for these parameters (0 on invalid
  * parameters).  The workspace holds the second polarization buffer, the
  * Krylov vectors, the multigrid hierarchy, the boundary masks and the
- * reduction scratch. */
+ * reduction scratch.  With PF_PCG_MG it also holds the inverse of the coarsest
+ * level's operator in FP64: 8 n^2 bytes for n cells there, n <= 1024, so up to 8
+ * MB.  The first solve after pf_bind or a change of electrode layout forms it: in
+ * one launch where n <= 64, as on grids that halve down to a few cells, in n short
+ * launches above that. */
 size_t pf_workspace_bytes(const pf_params* params);
 
 /* Validate params and create a context bound to a CUDA stream (a
