@@ -1795,32 +1795,41 @@ pf_status batch_upload_table(pf_batch* b) {
 }
 
 // How the films of a batch run their Jacobi-PCG loops, for as long as this
-// object lives.  While all the films' loops have a few blocks per SM together, each
-// as it does alone.  Beyond that, small films (pf_cgloop.cu) as two launches an
-// iteration: ms a step with loops / launches for 10 films of 32^3 in FP32 0.41 / 0.59,
-// 8 of 64 x 64 x 32 0.69 / 0.59; in FP64 5 of 48 x 40 x 24 0.64 / 0.53, 4 of 64 x 64
-// x 32 0.84 / 0.77.  Films that fill the GPU by themselves keep the loop, in FP32 from
-// 32 films on with an eighth of the blocks each, so that fewer of them share the L2:
-// 64 of 96 x 96 x 48 13.2 against 22.1 with two plane marches (16 films: 5.1 on all
-// blocks, 5.5; FP64 is slower with an eighth: 29 against 20 for 16 films of mixed sizes).
+// object lives.  A loop's blocks wait for one another, so that a film starts only
+// when the GPU has room for all of them: the films go through in rounds, in each
+// of which SMs idle at barriers.  With few rounds every film runs its loop as it
+// does alone; beyond two (FP32 films that share the GPU with others: three) all
+// take two launches an iteration, which interleave.  us per film and iteration,
+// loops / launches: FP32 32^3 (four at a time) 12 films 3.15 / 3.26, 14 films
+// 3.08 / 2.92; 64 x 64 x 32 (two) 5 films 6.26 / 6.37, 7 films 6.04 / 5.21; 128 x
+// 128 x 64 (one) 2 films 16.2 / 17.8, 3 films 17.8 / 15.2; FP64 96 x 96 x 48 (one)
+// 2 films 35.4 / 39.2, 3 films 35.3 / 34.1; 32^3 (four) 6 films 6.07 / 6.66, 8 films
+// 5.91 / 5.56.  (Two plane marches an iteration, at the tile depth that suits each
+// shape best: 16 films of 96 x 96 x 48 in FP32 10.8, launches 10.5, loops 14.8; 16 of
+// four sizes 11.0, 10.2 and 13.9.)
+// From 32 FP32 films on, those that fill the GPU but have at most 10 MB in the loop's
+// vectors run it on a quarter of the blocks each, so that four of them share the L2
+// and the others wait: 64 of 96 x 96 x 48 9.2 against 10.5 with launches (an eighth of the
+// blocks 9.4; of 128 x 128 x 64, 21 MB, a quarter 14.6, launches 13.7).
 struct BatchLoops {
   pf_batch* b;
   explicit BatchLoops(pf_batch* batch) : b(batch) {
-    long long blocks = 0;
-    std::vector<int> small(b->films.size(), 0);
-    for (size_t i = 0; i < b->films.size(); ++i) {
-      pf_ctx* c = b->films[i];
-      if (cg_loop_of(c))
-        blocks += c->prm.precision == PF_FP32 ? pf::cg_loop_blocks<float>(c->L, c->geo, &small[i])
-                                              : pf::cg_loop_blocks<double>(c->L, c->geo, &small[i]);
-    }
-    for (size_t i = 0; i < b->films.size(); ++i) {
-      pf_ctx* c = b->films[i];
+    double load = 0.0;
+    for (pf_ctx* c : b->films) {
       if (!cg_loop_of(c)) continue;
       const bool fp32 = c->prm.precision == PF_FP32;
-      if (blocks <= (fp32 ? 6LL : 4LL) * c->nsm) continue;
-      if (small[i]) c->L.loop_halves = 1;
-      else if (fp32 && b->films.size() >= 32) c->L.loop_share = 8;
+      int held = 0;
+      const int blocks = fp32 ? pf::cg_loop_blocks<float>(c->L, c->geo, &held)
+                              : pf::cg_loop_blocks<double>(c->L, c->geo, &held);
+      const int fit = std::max(1, held / blocks);
+      load += 1.0 / fit / (fp32 && fit > 1 ? 3.0 : 2.0);
+    }
+    if (load <= 1.0 + 1e-9) return;
+    for (pf_ctx* c : b->films) {
+      if (!cg_loop_of(c)) continue;
+      const bool big = pf::loop_fills(c->L, c->geo) && 5 * 4 * c->geo.n <= 10LL << 20;
+      if (c->prm.precision == PF_FP32 && big && b->films.size() >= 32) c->L.loop_share = 4;
+      else c->L.loop_halves = 1;
     }
   }
   ~BatchLoops() {

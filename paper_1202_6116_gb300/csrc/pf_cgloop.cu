@@ -441,20 +441,27 @@ static int loop_blocks(const LaunchCfg& L, const Geo& g, int vx, int groups, Mar
   return (int)std::min<long long>(L.nsm, (mc.ntiles + groups - 1) / groups);
 }
 
+// Blocks of the loop that an SM holds at a time; 0: it cannot be launched here.
+template <typename T, int VX, int G>
+static int loop_resident() {
+  static int n = -1;
+  if (n < 0) {
+    int nb = 0, coop = 0, dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_cg_loop<T, VX, G>, 256 * G, 0) != cudaSuccess)
+      coop = 0;
+    cudaGetLastError();
+    n = coop ? nb : 0;
+  }
+  return n;
+}
+
 // dry: only whether it can be launched here.
 template <typename T, int VX, int G>
 static bool cg_loop_t(const LaunchCfg& L, const Geo& g, const Dev<T>& d, bool dry) {
   auto kernel = k_cg_loop<T, VX, G>;
-  static int can = -1;
-  if (can < 0) {
-    int nb = 0, coop = 0, dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kernel, 256 * G, 0) != cudaSuccess)
-      coop = 0;
-    cudaGetLastError();
-    can = coop && nb > 0;
-  }
+  const bool can = loop_resident<T, VX, G>() > 0;
   if (dry || !can) return can;
   MarchCfg mc;
   const int nvb = loop_blocks(L, g, VX, G, mc);
@@ -481,13 +488,6 @@ static void cg_halves_t(const LaunchCfg& L, const Geo& g, const Dev<T>& d, cudaG
   k_half_r<T, VX, G><<<nvb, block, 0, L.stream>>>(g, d.bc, v, d.part, d.S, mc, cond);
 }
 
-// Does a film have a 16-byte vector for every thread that the GPU holds?
-template <typename T>
-static bool loop_fills(const LaunchCfg& L, const Geo& g) {
-  constexpr int V = 16 / sizeof(T);
-  return g.n / V >= (long long)L.nsm * 512;
-}
-
 // Calls f with the cells of a film's threads and the thread groups of its blocks.
 // Films that do not fill the GPU take vectors all the same (half as long where 16 of
 // them are longer than a row) and one group a block: ms a step of a film alone 0.123
@@ -501,7 +501,7 @@ static auto loop_form(const LaunchCfg& L, const Geo& g, F f) {
   constexpr int V = 16 / sizeof(T), F32 = sizeof(T) == 4;
   const bool vec = L.march.vx == V;
   using std::integral_constant;
-  if (loop_fills<T>(L, g)) {
+  if (loop_fills(L, g)) {
     if (vec) return f(integral_constant<int, V>(), integral_constant<int, 2>());
     return f(integral_constant<int, 1>(), integral_constant<int, F32 ? 4 : 2>());
   }
@@ -517,10 +517,12 @@ bool launch_cg_loop(const LaunchCfg& L, const Geo& g, const Dev<T>& d, bool dry)
 }
 
 template <typename T>
-int cg_loop_blocks(const LaunchCfg& L, const Geo& g, int* small) {
+int cg_loop_blocks(const LaunchCfg& L, const Geo& g, int* held) {
   MarchCfg mc;
-  *small = !loop_fills<T>(L, g);
-  return loop_form<T>(L, g, [&](auto vx, auto groups) { return loop_blocks(L, g, vx, groups, mc); });
+  return loop_form<T>(L, g, [&](auto vx, auto groups) {
+    *held = loop_resident<T, vx, groups>() * L.nsm;
+    return loop_blocks(L, g, vx, groups, mc);
+  });
 }
 
 template <typename T>

@@ -207,12 +207,14 @@ void launch_cg_r(const LaunchCfg& L, const Geo& g, const Dev<T>& d, int mg, cuda
 template <typename T>
 bool launch_cg_loop(const LaunchCfg& L, const Geo& g, const Dev<T>& d, bool dry);
 // One iteration of that loop as two launches, with the same bits (in a graph's
-// conditional loop); and the blocks of a film's loop when it runs alone (*small: 1
-// when the film does not fill the GPU).
+// conditional loop); and the blocks of a film's loop when it runs alone (*held: of
+// such blocks, as many as the GPU holds at a time).
 template <typename T>
 void launch_cg_halves(const LaunchCfg& L, const Geo& g, const Dev<T>& d, cudaGraphConditionalHandle cond);
 template <typename T>
-int cg_loop_blocks(const LaunchCfg& L, const Geo& g, int* small);
+int cg_loop_blocks(const LaunchCfg& L, const Geo& g, int* held);
+// Does a film have a 16-byte vector for each of 512 threads per SM?
+inline bool loop_fills(const LaunchCfg& L, const Geo& g) { return g.n * L.word / 16 >= L.nsm * 512LL; }
 template <typename T>
 void launch_cg_finish(const LaunchCfg& L, const Geo& g, const Dev<T>& d, int singular);
 template <typename T>

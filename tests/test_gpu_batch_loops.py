@@ -67,7 +67,7 @@ def test_large_batch_of_small_jacobi_films_equals_films_alone(precision):
 
 
 def test_batch_of_32_with_large_jacobi_films_equals_films_alone():
-    """FP32 films whose loops fill the GPU by themselves run them on an eighth of the blocks from 32 films on."""
+    """FP32 films whose loops fill the GPU by themselves run them on fewer blocks from 32 films on."""
     ws = films_of([(16, 16, 8)] * 27 + [(96, 96, 48), (128, 96, 40), (100, 104, 44), (96, 96, 48), (72, 96, 64)], "fp32")
     infos = batch_against_alone(ws, 4)
     assert all(i["kernel_launches"] < 40 for i in infos[27:])          # one launch a loop
@@ -77,3 +77,14 @@ def test_small_batch_keeps_the_persistent_loop():
     ws = films_of([(32, 32, 32)] * 2, "fp32")
     infos = batch_against_alone(ws, 5)
     assert all(i["kernel_launches"] < 40 for i in infos)
+
+
+@pytest.mark.parametrize("precision,shapes", [
+    ("fp32", [(128, 64, 80), (96, 96, 48), (101, 75, 40), (128, 64, 80)]),   # loops that need the whole GPU each
+    ("fp32", [(100, 104, 44), (32, 32, 32), (97, 96, 52), (64, 64, 32), (96, 96, 48)]),
+    ("fp64", [(96, 96, 48), (75, 101, 50), (96, 80, 56)]),
+])
+def test_batch_of_few_large_jacobi_films_equals_films_alone(precision, shapes):
+    infos = batch_against_alone(films_of(shapes, precision), 4)
+    # two launches an iteration, from the third film on that has the GPU to itself
+    assert all(i["kernel_launches"] >= 2 * i["total_iters"] for i in infos)
