@@ -11,8 +11,10 @@ permittivity) in memory and, optionally, in a JSON file.
 Every candidate starts from the same polarization and its solved potential with
 no history of earlier solves (the iterations a start needs, over which a step's
 other kernels are spread, are then the same).  The default gives every kernel its
-own planned depth, which no other candidate does, so another one has to be faster
-by more than runs differ (MARGIN).
+own planned depth, which no other candidate does, so another one has to be clearly
+faster (MARGIN).  Tilings 2 to 3 % faster than it on a film alone, another set in
+every run, cost a batch of 64 multigrid films 1.68 ms a step where the default takes
+1.54.
 """
 from __future__ import annotations
 
@@ -26,7 +28,7 @@ from .film import Film
 from .workloads import Workload
 
 _CACHE: dict = {}
-MARGIN = 0.02
+MARGIN = 0.05
 
 
 def key_of(w: Workload) -> str:
