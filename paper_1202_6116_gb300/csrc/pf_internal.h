@@ -61,7 +61,7 @@ struct LaunchCfg {
   int loop_share = 1;  // virtual blocks per block of the persistent Jacobi-PCG loop
   unsigned loop_polls = LOOP_POLLS;   // (pf_set_wait_limit)
   int loop_halves = 0; // 1: that loop as two launches an iteration (both: films of a batch, see pf_cgloop.cu)
-  mutable MarchCfg plan[2][PLAN_OCC];   // planned tilings (ntiles = 0: not yet), see kernel_tiling
+  mutable MarchCfg plan[3][PLAN_OCC];   // planned tilings (ntiles = 0: not yet), see kernel_tiling
   int flat_grid;       // flat vector kernels (FLAT_THREADS blocks, grid-stride)
   cudaStream_t stream;
 };
@@ -351,12 +351,15 @@ inline double march_cost(long long cols, int nz, int tz, int nsm, int occ, int w
 
 // Tiling of a plane march over an nx x ny x nz grid: 16 bytes of cells per
 // thread when nx allows it, and the tile depth (at most tzmax planes, even for
-// even_tz) of least march_cost.  One rule for every size: a film of 1024 x 1024
+// even_tz) of least march_cost.  turns > 0: among those of at most two planes, with
+// turns tiles per resident block, or whose tiles fill the resident blocks a whole
+// number of times but for 6 %.  One rule for every size: a film of 1024 x 1024
 // columns takes the deepest tiles, one of 64 x 64 a couple of planes per tile.
 // (The rule before it, the deepest of 32 .. 2 planes with three tiles per
 // resident block, gave a 256 x 256 x 64 film tiles of 2 planes: 55 us for the
 // right-hand side, 33 for the search direction; planned, 37 and 23.)
-inline MarchCfg march_cfg(int nx, int ny, int nz, int nsm, int occ, int tzmax, bool even_tz, int word) {
+inline MarchCfg march_cfg(int nx, int ny, int nz, int nsm, int occ, int tzmax, bool even_tz, int word,
+                          int turns = 0) {
   MarchCfg m{};
   const int v = 16 / word;
   m.vx = nx % v == 0 ? v : 1;
@@ -370,6 +373,8 @@ inline MarchCfg march_cfg(int nx, int ny, int nz, int nsm, int occ, int tzmax, b
   for (int tz = std::min(tzmax, nz); tz >= 1; --tz) {
     if (even_tz && (tz & 1)) continue;
     const int chunks = (nz + tz - 1) / tz;
+    const long long tiles = cols * chunks, slots = (long long)nsm * occ;
+    if (tz > 2 && tiles < turns * slots && 50 * tiles < 47 * ((tiles + slots - 1) / slots * slots)) continue;
     if (chunks > 128) {          // march_cost is a sum over the chunks: very tall grids take a plain rule
       if (best == 0.0) {
         m.tz = tz;
@@ -395,9 +400,12 @@ inline MarchCfg march_cfg(int nx, int ny, int nz, int nsm, int occ, int tzmax, b
 // already raised; occ caches its occupancy): the one asked for, on its own
 // occupancy, or the planned one.  deep: tiles of up to 64 planes (the kernels
 // that sum over their tiles), else 32 (the TDGL update on 1024 x 1024 x 128:
-// 1.00 ms with 32 planes, 1.02 with 64).
+// 1.00 ms with 32 planes, 1.02 with 64).  turns: three for the FP32 update with noise,
+// whose blocks keep the issue slots busy: two on an SM take nearly twice as long as one,
+// which march_cost does not know, so its tiles balance the load or fill the SMs evenly
+// (512 x 512 x 64 256 us, 286 without; 256 x 256 x 16 29 and 33; 96 x 96 x 48 17.5 and 20.6).
 template <class K>
-inline MarchCfg kernel_tiling(K kernel, size_t bytes, const LaunchCfg& L, int& occ, bool deep) {
+inline MarchCfg kernel_tiling(K kernel, size_t bytes, const LaunchCfg& L, int& occ, bool deep, int turns = 0) {
   if (occ == 0) {
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, MTX * MTY, bytes) != cudaSuccess) occ = 1;
     cudaGetLastError();
@@ -410,8 +418,8 @@ inline MarchCfg kernel_tiling(K kernel, size_t bytes, const LaunchCfg& L, int& o
     return m;
   }
   const int o = std::min(occ, PLAN_OCC);
-  MarchCfg& m = L.plan[deep ? 1 : 0][o - 1];
-  if (m.ntiles == 0) m = march_cfg(L.nx, L.ny, L.nz, L.nsm, o, deep ? 64 : 32, false, L.word);
+  MarchCfg& m = L.plan[turns ? 2 : deep ? 1 : 0][o - 1];
+  if (m.ntiles == 0) m = march_cfg(L.nx, L.ny, L.nz, L.nsm, o, deep ? 64 : 32, false, L.word, turns);
   return m;
 }
 

@@ -976,7 +976,7 @@ static void tdgl_t(const LaunchCfg& L, const Geo& g, const Dev<T>& d, const T* P
   const size_t bytes = StepPipe<T, false, VX>::bytes();
   smem_attr(k_tdgl<T, CORR, NOISE, VX, COMP>, bytes, f);
   static int occ = 0;
-  const MarchCfg mc = kernel_tiling(k_tdgl<T, CORR, NOISE, VX, COMP>, bytes, L, occ, false);
+  const MarchCfg mc = kernel_tiling(k_tdgl<T, CORR, NOISE, VX, COMP>, bytes, L, occ, false, NOISE && sizeof(T) == 4 ? 3 : 0);
   k_tdgl<T, CORR, NOISE, VX, COMP><<<mc.grid, dim3(MTX, MTY), bytes, L.stream>>>(g, d.bc, P, Pn, d.phi, k, d.S, mc,
                                                                                 d.plo);
 }

@@ -1,5 +1,6 @@
 """pf_set_tiling with what pf_get_tiling reports for a new context leaves the
 film as it was: every kernel keeps (or gets back) its own planned depth."""
+import numpy as np
 import pytest
 import torch
 
@@ -68,3 +69,21 @@ def test_depths_differ_between_kernels_and_the_tuner_can_keep_them():
         assert same((f.P, f.phi, f.diagnostics()), ref)
         f.close()
     assert differ
+
+
+@pytest.mark.parametrize("shape", [(128, 128, 64), (96, 96, 48), (75, 48, 40), (64, 64, 3)])
+def test_noisy_steps_do_not_depend_on_the_depth(shape):
+    """The update with noise plans its own depth; with the potential held it sums nothing, so that every depth
+    gives the same bits."""
+    out = []
+    for tz in (None, 1, 5, 32):
+        f = Film(mixed_workload(*shape, 84, precision="fp32", rtol=1e-5), poisson_every=1000)
+        f.set_noise(0.05, 3)
+        f.step(1)
+        if tz is not None:
+            t = pf.pf_get_tiling(f.ctx)
+            pf.pf_set_tiling(f.ctx, t.vx, min(tz, shape[2]), 0)
+        f.step(4)
+        out.append(f.numpy()[0])
+        f.close()
+    assert all(np.array_equal(o, out[0]) for o in out[1:])
